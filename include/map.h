@@ -101,8 +101,13 @@ enum { MAP_SCHED_SYNC = 0, MAP_SCHED_ASYNC = 1 };
                                   last map vector as with the dense round.  Refused by map_run_static. */
 
 #define MAP_FLAG_DENSE_START 8u /* the dense round, even on a handle that map_autotune set to the frontier
-                                   start (without either flag a handle starts the way map_autotune chose,
-                                   by default with the dense round).  Both start flags together: MAP_ERR_ARG. */
+                                   start (without either flag a handle starts the way map_autotune chose;
+                                   before any map_autotune the library chooses per graph: the frontier start
+                                   where few entries hold an accepting vertex or the graph is small, else
+                                   the dense round; runs with a trace, MAP_FLAG_PROFILE or
+                                   MAP_FLAG_EARLY_EXIT start with the dense round).  Maps, verdicts and the
+                                   counts described below are the same.  Both start flags together:
+                                   MAP_ERR_ARG. */
 
 #define MAP_FLAG_PUSH 64u  /* every round after round 1 pushes from the vertices changed in the round before
                               to their readers (the reverse CSR); also keeps a graph whose rows hold one
@@ -155,7 +160,7 @@ typedef struct {
     double dense_ms;          /* time of the dense rounds summed over the run: CUDA events around each
                                  launch with MAP_FLAG_PROFILE, else the kernels' own %globaltimer stamps
                                  (each phase runs from the end of the one before it) */
-    uint32_t dense_launches;  /* dense-round launches */
+    uint32_t dense_launches;  /* dense-round launches (0 with the frontier start, asked for or chosen) */
     uint32_t accepting_left;  /* accepting vertices left at the end */
     uint64_t launches;        /* kernel launches issued by this run */
     double round_ms;          /* time of the fix-point rounds after the dense round (with the frontier
@@ -194,15 +199,17 @@ MAP_API int map_create(uint32_t n, const uint32_t *rowptr, const uint32_t *colid
 /*
  * map_run -- run MAP to its verdict (Section 2: propagate to the fix-point,
  * self-map test, eliminate, restart).
- *   opts     NULL for defaults (SYNC, no limits, no trace, the dense start
- *            unless map_autotune chose the frontier start for this handle).
+ *   opts     NULL for defaults (SYNC, no limits, no trace, the start chosen by
+ *            map_autotune or by the library, see MAP_FLAG_DENSE_START).
  *   res      filled on MAP_OK and on MAP_ERR_LIMIT (with what was computed).
  *   map_out  optional, n entries, host or device memory: the map vector of the
  *            last outer iteration (all MAP_NONE when no vertex is accepting).
  * The graph is not changed: the accepting set is restored at every call, so
  * runs repeat exactly.  Blocks the calling thread until the result is known.
- * Without a trace or MAP_FLAG_PROFILE the whole run is one CUDA-graph launch
- * (its graph is built on the handle's first run with that schedule and start).
+ * Without a trace or MAP_FLAG_PROFILE the whole run is queued at once: with the
+ * frontier start and rounds that push, one or two kernel launches; else one
+ * CUDA-graph launch (its graph is built on the handle's first run with that
+ * schedule and start).
  */
 MAP_API int map_run(map_graph *g, const map_opts *opts, map_result *res, uint32_t *map_out);
 

@@ -10,7 +10,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libmapgpu.so")
 SOURCES = ["map_api.cu"]
-HEADERS = ["map_kernels.cuh"]
+HEADERS = ["map_kernels.cuh", "map_run.cuh"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

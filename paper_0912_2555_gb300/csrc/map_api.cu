@@ -28,6 +28,7 @@
 
 #include "map.h"
 #include "map_kernels.cuh"
+#include "map_run.cuh"
 
 using mapk::Ctl;
 
@@ -95,7 +96,8 @@ bool is_device_ptr(const void *p)
 // a freed slot goes to a free list.
 class PinnedSlots {
   public:
-    static constexpr size_t SLOT = (sizeof(Ctl) + 255) & ~size_t(255);
+    static constexpr size_t RES = (sizeof(Ctl) + 255) & ~size_t(255); // a run's result, behind the mirror
+    static constexpr size_t SLOT = RES + ((sizeof(mapk::RunRes) + 255) & ~size_t(255));
     static constexpr int PER_CHUNK = 32;
     // a slot, or nullptr if page-locked memory cannot be had (the caller then uses pageable memory)
     void *get()
@@ -203,6 +205,65 @@ int func_occupancy()
     return std::max(1, o);
 }
 
+// resident blocks per SM that every variant of the whole-run kernel supports (a cooperative launch)
+int run_occupancy()
+{
+    int occ = 1 << 30, o = 0;
+    for (const void *k : {(const void *)mapk::k_run<true, false>, (const void *)mapk::k_run<false, false>,
+                          (const void *)mapk::k_run<true, true>, (const void *)mapk::k_run<false, true>}) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k, mapk::RT, 0) != cudaSuccess) {
+            cudaGetLastError();
+            o = 1;
+        }
+        occ = std::min(occ, o);
+    }
+    return std::max(1, occ);
+}
+
+// Blocks of the cluster that k_tail runs in on the current device: 16, or 8 (the portable size), or 0
+// where no such cluster fits.  Asked once per device.
+int tail_blocks()
+{
+    constexpr int DEVICES = 64;
+    static std::atomic<int> known[DEVICES]; // blocks + 1
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= DEVICES) {
+        cudaGetLastError();
+        return 0;
+    }
+    if (const int k = known[dev].load()) return k - 1;
+    int best = 0;
+    const void *const both[] = {(const void *)mapk::k_tail<true>, (const void *)mapk::k_tail<false>};
+    bool ok = true;
+    for (const void *f : both)
+        ok = ok && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mapk::TAIL_SMEM) == cudaSuccess &&
+             cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    for (int blocks : {16, 8}) {
+        bool fits = ok;
+        for (const void *f : both) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(blocks);
+            cfg.blockDim = dim3(mapk::TT);
+            cfg.dynamicSmemBytes = mapk::TAIL_SMEM;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = blocks;
+            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            int n = 0;
+            fits = fits && cudaOccupancyMaxActiveClusters(&n, f, &cfg) == cudaSuccess && n > 0;
+        }
+        if (fits) {
+            best = blocks;
+            break;
+        }
+    }
+    cudaGetLastError();
+    known[dev].store(best + 1);
+    return best;
+}
+
 int pull_occupancy()
 {
     int occ = 1 << 30, o = 0;
@@ -261,6 +322,7 @@ struct map_graph {
     uint32_t *ids = nullptr; // reduced graphs: the original id of each vertex (else NULL: identity)
     uint32_t rows = 0;       // rows expanded so far (growing graphs); the rest are empty
     bool dirty = false; // a run stopped early: per-round state may be stale
+    bool snaps = false; // the dense round has written snapshots into rec (an asynchronous run leaves them)
     uint32_t *hist = nullptr; // rounds per outer iteration
     uint32_t hist_cap = 0;
     Ctl *ctl = nullptr;
@@ -282,7 +344,11 @@ struct map_graph {
     uint32_t *alist = nullptr;
     uint32_t na = 0;
     bool fstart_on = false;
+    bool tuned = false;        // map_autotune chose the start (else: default_fstart)
     bool tuned_fstart = false; // map_autotune found the frontier start faster on this graph
+    bool fstart_push = false;  // ... and, with it, rounds that only push
+    uint64_t acc_entries = 0;  // entries that hold an accepting vertex
+    mapk::RunCtl *run_ctl = nullptr; // control block of whole-run launches, and the result behind it (first use)
     bool pull_on = false;     // the launches being issued may pull (the fix-point kernel's pull variant)
     bool functional = false;  // every row holds at most one entry (set-up): pointer doubling applies
     bool func_on = false;     // the launches being issued propagate by pointer doubling (k_func)
@@ -308,6 +374,7 @@ void free_graph(map_graph *g)
                    g->alist};
     for (void *p : dev)
         if (p) cudaFreeAsync(p, g->stream); // stream-ordered: no device-wide synchronisation
+    if (g->run_ctl) cudaFreeAsync(g->run_ctl, g->stream);
     if (g->comp) cudaFreeAsync(g->comp, g->stream);
     if (g->ids) cudaFreeAsync(g->ids, g->stream);
     if (g->stale) cudaFreeAsync(g->stale, g->stream);
@@ -742,7 +809,7 @@ int create_graph(uint32_t n, uint64_t m, cudaStream_t s, const char *who, Upload
     mapk::k_ingest<<<grid_for(g, std::max<uint64_t>(m / 4, n), 1), 256, 0, s>>>(
         n, g->in_rowptr ? g->in_rowptr : g->rowptr, g->in_rowptr ? g->rowptr : nullptr, m,
         g->in_colidx ? g->in_colidx : g->colidx, g->colidx, g->acc0, g->rrowptr, rank, &g->ctl->bad,
-        &g->ctl->long_rows);
+        &g->ctl->long_rows, (unsigned long long *)&g->ctl->relax.v);
     g->in_rowptr = g->in_colidx = nullptr;
     if ((rc = ck(cudaGetLastError(), "validate")) || (rc = read_ctl(g))) {
         free_rank();
@@ -756,6 +823,7 @@ int create_graph(uint32_t n, uint64_t m, cudaStream_t s, const char *who, Upload
     }
     g->nacc0 = g->h_ctl->elim.v;
     g->functional = m > 0 && g->h_ctl->long_rows == 0;
+    g->acc_entries = g->h_ctl->relax.v;
 
     // reverse CSR: scan of the histogram, scatter by rank
     if ((rc = scan_inclusive(g->rrowptr, (uint64_t)n + 1, s))) {
@@ -836,6 +904,104 @@ int map_destroy(map_graph *g)
     return MAP_OK;
 }
 
+// single graphs small enough for one cluster (k_tail): the whole run in one launch of it
+static bool runs_in_tail(const map_graph *g) { return !g->comp && g->n <= tail_blocks() * mapk::TAIL_N; }
+
+// Which start a run takes when neither its flags nor map_autotune say: the frontier start pushes
+// from the accepting vertices (one random access per entry that holds one) and runs in one launch, the
+// dense start streams the whole matrix.  Measured: layered graphs (1 entry in 200) 3.4 against 16.4 ms at
+// 2^26 vertices, an interleaved product with 1 entry in 7 (1.6 M vertices) 6.4 against 4.6 ms; graphs that
+// fit into one cluster always gain (16,384 vertices 0.12 against 0.44 ms).
+static bool default_fstart(const map_graph *g) { return runs_in_tail(g) || g->acc_entries <= g->m / 16; }
+
+// Queue one whole run as a single launch (k_run) and fill in the result from where the kernel left it.
+static int launch_run(map_graph *g, cudaStream_t s, const map_opts &opts, const Ctl &init, bool count_round1,
+                      uint32_t *out)
+{
+    static const int occ = run_occupancy();
+    const size_t n = g->n;
+    if (!g->run_ctl) CK(cudaMallocAsync((void **)&g->run_ctl, sizeof(mapk::RunCtl) + sizeof(mapk::RunRes), s));
+    mapk::RunArgs a;
+    memset(&a, 0, sizeof a);
+    a.n = g->n;
+    a.words = g->words;
+    a.rowptr = g->rowptr;
+    a.rrowptr = g->rrowptr;
+    a.rcol = g->rcol;
+    a.acc0 = g->acc0;
+    a.acc = g->acc;
+    a.W = reinterpret_cast<unsigned long long *>(g->rec);
+    a.la = g->list;
+    a.lb = g->list + n;
+    a.alist = g->list + 2 * n;
+    a.touched = g->touched;
+    a.tval = g->elog;
+    a.rank = g->mval;
+    a.pool = g->flist;
+    a.ctl = g->run_ctl;
+    a.res = g->h_ctl_pinned ? reinterpret_cast<mapk::RunRes *>(reinterpret_cast<uint8_t *>(g->h_ctl) + PinnedSlots::RES)
+                            : reinterpret_cast<mapk::RunRes *>(g->run_ctl + 1);
+    a.hist = g->hist;
+    a.hist_cap = g->hist_cap;
+    a.out = out;
+    a.m = g->m;
+    a.nacc0 = g->nacc0;
+    a.max_outer = init.max_outer;
+    a.max_inner = init.max_inner;
+    a.lc_passes = init.lc_passes;
+    a.count_round1 = count_round1 ? 1 : 0;
+    a.timeout_ns = init.timeout_ns;
+    a.comp = g->comp;
+    a.cs = g->cs;
+    a.chist = g->chist;
+    a.ncomp = g->ncomp;
+    const bool sync_sched = opts.sched == MAP_SCHED_SYNC;
+    const int cluster = g->comp ? 0 : tail_blocks();
+    const bool whole = runs_in_tail(g);
+    const auto launch_tail = [&](uint32_t blocks) -> int {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(blocks);
+        cfg.blockDim = dim3(mapk::TT);
+        cfg.dynamicSmemBytes = mapk::TAIL_SMEM;
+        cfg.stream = s;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = blocks;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_tail<true>, a, whole ? 1u : 0u));
+        else CK(cudaLaunchKernelEx(&cfg, mapk::k_tail<false>, a, whole ? 1u : 0u));
+        return MAP_OK;
+    };
+    if (whole) {
+        uint32_t blocks = 1;
+        while ((int)blocks < cluster && g->n > blocks * 1024u) blocks *= 2;
+        return launch_tail(blocks);
+    }
+    a.tail_cap = (uint32_t)cluster * mapk::TAIL_N;
+    CK(cudaMemsetAsync(g->run_ctl, 0, sizeof(mapk::RunCtl), s));
+    if (g->comp) {
+        mapk::k_batch_begin<<<(g->ncomp + 255) / 256, 256, 0, s>>>(dev_of(g));
+        CK(cudaGetLastError());
+    }
+    cudaLaunchConfig_t cfg = {};
+    // (rounds_grid counts blocks of 256 threads; a served job's share of the device carries over)
+    cfg.gridDim = dim3((unsigned)std::max(1, std::min(g->sms * occ, g->rounds_grid * 256 / mapk::RT)));
+    cfg.blockDim = dim3(mapk::RT);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (g->comp && sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_run<true, true>, a));
+    else if (g->comp) CK(cudaLaunchKernelEx(&cfg, mapk::k_run<false, true>, a));
+    else if (sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_run<true, false>, a));
+    else CK(cudaLaunchKernelEx(&cfg, mapk::k_run<false, false>, a));
+    return cluster ? launch_tail((uint32_t)cluster) : MAP_OK;
+}
+
 static int run_impl(map_graph *g, const map_opts *opts_in, map_result *res, uint32_t *map_out,
                     bool force_stepped = false)
 {
@@ -859,11 +1025,17 @@ static int run_impl(map_graph *g, const map_opts *opts_in, map_result *res, uint
     // map_autotune and not overridden; with none accepting no iteration runs and the
     // dense-round graph does as well
     NvtxRange range(stepped ? "map_run (stepped)" : "map_run");
-    const bool fstart = ((opts.flags & MAP_FLAG_FRONTIER_START) ||
-                         (g->tuned_fstart && !(opts.flags & MAP_FLAG_DENSE_START))) &&
-                        g->nacc0 > 0;
     if ((opts.flags & MAP_FLAG_PUSH) && (opts.flags & MAP_FLAG_PULL))
         return fail(MAP_ERR_ARG, "map_run: MAP_FLAG_PUSH and MAP_FLAG_PULL together");
+    const bool asked = (opts.flags & MAP_FLAG_FRONTIER_START) != 0, dense = (opts.flags & MAP_FLAG_DENSE_START) != 0;
+    uint32_t pull_min = (opts.flags & MAP_FLAG_PULL) ? 1u : (opts.flags & MAP_FLAG_PUSH) ? 0u : g->pull_min;
+    // a whole run in one launch: rounds that push, from the accepting vertices, none stepped from the host
+    const bool whole = !stepped && !(opts.flags & MAP_FLAG_EARLY_EXIT);
+    if (whole && g->tuned && g->fstart_push && !(opts.flags & MAP_FLAG_PULL) && !dense) pull_min = 0;
+    const bool doubling = g->functional && !sync_sched && !g->comp && !(opts.flags & (MAP_FLAG_PUSH | MAP_FLAG_PULL));
+    const bool fstart = g->nacc0 > 0 && (asked || (!dense && (g->tuned ? g->tuned_fstart
+                                                                       : whole && !pull_min && !doubling && default_fstart(g))));
+    const bool one_launch = fstart && whole && !pull_min;
     struct FstartOff { // the flags only hold for the launches of this run
         map_graph *g;
         ~FstartOff()
@@ -894,8 +1066,8 @@ static int run_impl(map_graph *g, const map_opts *opts_in, map_result *res, uint
     init.witness.v = mapk::NONE;
     // an asynchronous single-graph run with the dense start on a graph whose every row holds at
     // most one entry propagates by pointer doubling (MAP_FLAG_PUSH or MAP_FLAG_PULL keep the rounds)
-    g->func_on = g->functional && !sync_sched && !fstart && !g->comp && !(opts.flags & (MAP_FLAG_PUSH | MAP_FLAG_PULL));
-    init.pull_min = g->func_on ? 0u : (opts.flags & MAP_FLAG_PULL) ? 1u : (opts.flags & MAP_FLAG_PUSH) ? 0u : g->pull_min;
+    g->func_on = doubling && !fstart;
+    init.pull_min = g->func_on ? 0u : pull_min;
     g->pull_on = init.pull_min != 0;
     init.solo_max = g->solo_max;
     init.lc_passes = g->lc_passes;
@@ -903,7 +1075,7 @@ static int run_impl(map_graph *g, const map_opts *opts_in, map_result *res, uint
 
     int rc = MAP_OK;
     float dense_ms = 0.f, round_ms = 0.f, check_ms = 0.f;
-    if (fstart && !g->alist) { // the initially accepting vertices, listed once per graph
+    if (fstart && !one_launch && !g->alist) { // the initially accepting vertices, listed once per graph
         uint32_t *al = nullptr;
         CK(cudaMallocAsync((void **)&al, ((size_t)g->nacc0 + 4) * 4, s));
         CK(cudaMemsetAsync(al + g->nacc0, 0, 4, s));
@@ -913,11 +1085,60 @@ static int run_impl(map_graph *g, const map_opts *opts_in, map_result *res, uint
         g->na = g->nacc0;
     }
     g->fstart_on = fstart;
-    if (g->dirty) { // the previous run stopped early: clear the round state it may have left
+    // the previous run stopped early: clear the round state it may have left (one launch keeps its own
+    // state in rec and wants it all zero, the snapshots of the dense rounds included)
+    if (g->dirty || (one_launch && g->snaps)) {
         CK(cudaMemsetAsync(g->rec, 0, (size_t)n * 16, s));
+        g->snaps = false;
         CK(cudaMemsetAsync(g->cbit, 0, 3 * ((size_t)g->words + 4) * 4, s));
     }
     g->dirty = true; // until this run completes normally
+    g->snaps = g->snaps || !one_launch;
+    if (one_launch) {
+        CK(cudaEventRecord(g->ev[0], s));
+        for (uint32_t k = 0; k < reps; ++k)
+            if ((rc = launch_run(g, s, opts, init, asked || g->tuned, map_out ? init.out : nullptr))) return rc;
+        CK(cudaEventRecord(g->ev[1], s));
+        mapk::RunRes pageable; // (without a page-locked slot the result is copied from the device)
+        const mapk::RunRes *R = &pageable;
+        if (g->h_ctl_pinned) {
+            R = reinterpret_cast<const mapk::RunRes *>(reinterpret_cast<const uint8_t *>(g->h_ctl) + PinnedSlots::RES);
+        } else {
+            CK(cudaMemcpyAsync(&pageable, g->run_ctl + 1, sizeof pageable, cudaMemcpyDeviceToHost, s));
+        }
+        if (map_out && !out_dev) CK(cudaMemcpyAsync(map_out, g->xbuf, (size_t)n * 4, cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+        float ms = 0.f;
+        CK(cudaEventElapsedTime(&ms, g->ev[0], g->ev[1]));
+        res->verdict = R->verdict ? MAP_CYCLE : MAP_NO_CYCLE;
+        res->witness = R->verdict ? R->witness : MAP_NONE;
+        res->outer_iters = R->outer;
+        res->inner_canonical = sync_sched ? 1 : 0;
+        res->inner_iters = R->inner_total;
+        res->relaxations = R->relax;
+        res->edges_total = g->m * (uint64_t)R->outer;
+        res->device_ms = ms;
+        res->round_ms = R->ph_rounds * 1e-6;
+        res->check_ms = R->ph_check * 1e-6;
+        res->frontier_rows = R->frontier_rows;
+        res->accepting_left = R->nacc;
+        res->launches = g->comp || runs_in_tail(g) || !tail_blocks() ? 1 : 2;
+        const uint32_t nh = std::min(std::min<uint32_t>(R->outer, g->hist_cap), opts.rounds_cap);
+        if (opts.rounds_out && nh) {
+            memcpy(opts.rounds_out, R->hist, (size_t)std::min(nh, mapk::RUN_HIST) * 4);
+            if (nh > mapk::RUN_HIST) { // the rest stayed on the device
+                CK(cudaMemcpyAsync(opts.rounds_out + mapk::RUN_HIST, g->hist + mapk::RUN_HIST,
+                                   (size_t)(nh - mapk::RUN_HIST) * 4, cudaMemcpyDeviceToHost, s));
+                CK(cudaStreamSynchronize(s));
+            }
+        }
+        g->dirty = R->gave_up != 0; // (a run stopped by a limit has put its state back)
+        if (R->status == mapk::ST_LIMIT) return fail(MAP_ERR_LIMIT, "map_run: max_outer or max_inner reached");
+        if (R->gave_up) return fail(MAP_ERR_TIMEOUT, "map_run: a bounded device wait (grid barrier) gave up after seconds without progress");
+        if (R->status == mapk::ST_TIMEOUT)
+            return fail(MAP_ERR_TIMEOUT, "map_run: stopped after timeout_ms = %u", opts.timeout_ms ? opts.timeout_ms : 120000u);
+        return MAP_OK;
+    }
     if (!stepped) {
         if ((rc = build_run_graph(g, opts.sched))) return rc;
         *g->h_ctl = init;
@@ -1196,11 +1417,16 @@ int map_autotune(map_graph *g, uint32_t sched, map_tune_result *out)
     out->rounds_ms = t_r;
     // the start of every outer iteration, with those shapes: whole runs as one graph launch each,
     // the better of two per start
-    g->tuned_fstart = false;
+    g->tuned = g->tuned_fstart = g->fstart_push = false;
     if (g->nacc0) {
-        double t[2] = {1e30, 1e30};
+        double t[2] = {1e30, 1e30}, push = 1e30;
         for (int f = 0; f < 2; ++f)
             if ((rc = whole_run(f ? MAP_FLAG_FRONTIER_START : MAP_FLAG_DENSE_START, &t[f]))) return rc;
+        // (where rounds pull: the frontier start with rounds that only push, one launch for the whole run)
+        if (g->pull_min && (rc = whole_run(MAP_FLAG_FRONTIER_START | MAP_FLAG_PUSH, &push))) return rc;
+        g->fstart_push = push < t[1];
+        t[1] = std::min(t[1], push);
+        g->tuned = true;
         g->tuned_fstart = t[1] < t[0];
         out->frontier_start = g->tuned_fstart ? 1u : 0u;
         out->dense_start_ms = t[0];

@@ -2004,7 +2004,7 @@ __global__ void k_validate(uint32_t n, const uint32_t *__restrict__ rowptr, uint
 // in bit 31; an entry u >= n sets *bad instead (the graph is then refused, and nothing built
 // from it is used).  Four entries per thread and step (one 128-bit load and store).
 __device__ __forceinline__ uint32_t ingest_one(uint32_t u, uint32_t n, const uint32_t *__restrict__ acc, uint32_t *cnt,
-                                               bool &bad, uint32_t &rank)
+                                               bool &bad, uint32_t &rank, uint32_t &nacc)
 {
     if (u >= n) {
         bad = true;
@@ -2012,7 +2012,9 @@ __device__ __forceinline__ uint32_t ingest_one(uint32_t u, uint32_t n, const uin
         return u;
     }
     rank = atomicAdd(cnt + u + 1, 1u);
-    return u | (((__ldg(acc + (u >> 5)) >> (u & 31u)) & 1u) << 31);
+    const uint32_t flag = (__ldg(acc + (u >> 5)) >> (u & 31u)) & 1u;
+    nacc += flag;
+    return u | (flag << 31);
 }
 
 // Reads rowptr_in and colidx_in and, where the _out array is given (not null), writes the
@@ -2021,11 +2023,13 @@ __device__ __forceinline__ uint32_t ingest_one(uint32_t u, uint32_t n, const uin
 // (they may be the same array); the inputs are read once each. rank[i] = the number of entries
 // before entry i that hold the same vertex (the count each one's increment returned: entry i's
 // place in that vertex's reader list, in an arbitrary but fixed order); *long_rows is set when
-// some row holds two entries or more.
+// some row holds two entries or more; *acc_entries counts the entries that hold an accepting vertex.
 __global__ void k_ingest(uint32_t n, const uint32_t *rowptr_in, uint32_t *rowptr_out, uint64_t m,
                          const uint32_t *colidx_in, uint32_t *colidx_out, const uint32_t *__restrict__ acc,
-                         uint32_t *cnt, uint32_t *rank, uint32_t *bad, uint32_t *long_rows)
+                         uint32_t *cnt, uint32_t *rank, uint32_t *bad, uint32_t *long_rows,
+                         unsigned long long *acc_entries)
 {
+    uint32_t na = 0; // (a thread's share of the entries: below 2^32)
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const unsigned lane = lane_id();
@@ -2049,16 +2053,18 @@ __global__ void k_ingest(uint32_t n, const uint32_t *rowptr_in, uint32_t *rowptr
     uint4 *r4 = reinterpret_cast<uint4 *>(rank);
     for (uint64_t q = tid; q < m4; q += stride) {
         uint4 w = c4[q], r;
-        w.x = ingest_one(w.x, n, acc, cnt, b, r.x);
-        w.y = ingest_one(w.y, n, acc, cnt, b, r.y);
-        w.z = ingest_one(w.z, n, acc, cnt, b, r.z);
-        w.w = ingest_one(w.w, n, acc, cnt, b, r.w);
+        w.x = ingest_one(w.x, n, acc, cnt, b, r.x, na);
+        w.y = ingest_one(w.y, n, acc, cnt, b, r.y, na);
+        w.z = ingest_one(w.z, n, acc, cnt, b, r.z, na);
+        w.w = ingest_one(w.w, n, acc, cnt, b, r.w, na);
         o4[q] = w;
         r4[q] = r;
     }
-    for (uint64_t i = m4 * 4 + tid; i < m; i += stride) colidx_out[i] = ingest_one(colidx_in[i], n, acc, cnt, b, rank[i]);
+    for (uint64_t i = m4 * 4 + tid; i < m; i += stride) colidx_out[i] = ingest_one(colidx_in[i], n, acc, cnt, b, rank[i], na);
     if (__any_sync(0xFFFFFFFFu, b) && lane == 0) *bad = 1;
     if (__any_sync(0xFFFFFFFFu, lr) && lane == 0) *long_rows = 1;
+    const unsigned long long wa = warp_sum64(na);
+    if (lane == 0 && wa) atomicAdd(acc_entries, wa);
 }
 
 // Reverse CSR scatter from the ranks k_ingest recorded: entry i of row w holding u goes to slot

@@ -1,0 +1,1137 @@
+// map_run.cuh -- a whole MAP run (Section 2 of the paper) in one persistent cooperative launch.
+//
+// k_run runs every outer iteration of a run whose iterations start from the accepting vertices
+// (the frontier start): round 1 pushes u + 1 from each accepting vertex u to its readers, round
+// r + 1 pushes from the vertices changed in round r, until a round changes nothing; then the
+// self-map test and the elimination, and the next iteration.  One grid barrier per round, one per
+// self-map test; no launch and no host step in between.
+//
+// Per-vertex state W, all zero between iterations:
+//   asynchronous  one word (value << 32 | ~round): an atomicMax with a larger value wins, and the
+//                 old word tells in the same round trip whether the vertex rose, whether it had
+//                 risen in this round already (then it is listed) and whether it had no value.
+//                 On equal values the older round has the larger low half and stays.
+//   synchronous   two words, written in even and odd rounds, (round << 33 | rose << 32 | value):
+//                 the words of the other parity are frozen during a round, so every value read is
+//                 the one of the round before (the exact Jacobi step).  The first push of a round to
+//                 a vertex puts the round's stamp on its word, whether the value rose or not, so
+//                 one atomicMax also finds the rows of the frontier (their lengths are the
+//                 canonical relaxation count) and the vertices to list, each exactly once.
+// So a push costs one random sector (asynchronous: one atomic; synchronous: a 16-byte load and, if
+// it can change anything, one atomic on the same sector), and nothing is cleared between rounds.
+//
+// Compaction.  A vertex that has a value in outer iteration k + 1 had one in iteration k (the
+// accepting set only shrinks), and every reader of such a vertex, or of a vertex still accepting, had
+// one too.  So after an iteration in which few vertices had a value, the run goes on in the
+// graph those vertices and the accepting ones induce, renumbered: the readers with their new
+// numbers, and per vertex one 16-byte record (reader range, own offer, original id).  Random
+// accesses over the full arrays are bound by address translation (measured: 42 G/s over 2 GB against
+// 128 G atomics/s and 300 G loads/s over a packed array), and the compact arrays stay in L2.
+//
+// What it measured, ms per run (dense start in a CUDA graph -> here, k_tail included): layered 2^26
+// asynchronous 16.35 -> 3.4, 2^24 synchronous 7.3 -> 2.6, 10^6 asynchronous 2.82 -> 0.89, the 16,384-vertex
+// random graph 0.44 -> 0.12.
+#pragma once
+#include "map_kernels.cuh"
+
+namespace mapk {
+
+constexpr int RT = 512; // threads per block
+#ifndef MAPGPU_RUN_BLOCKS
+#define MAPGPU_RUN_BLOCKS 2 // resident blocks per SM the register budget is sized for
+#endif
+#ifndef MAPGPU_RUN_P
+#define MAPGPU_RUN_P 1 // pushes per thread and step, all in flight together
+#endif
+constexpr int RUN_P = MAPGPU_RUN_P;
+constexpr uint32_t RUN_CAP = 2048;  // entries a block stages per round and list
+constexpr uint32_t RUN_HIST = 512;  // outer iterations whose rounds come back with the result
+
+struct alignas(128) Line64 {
+    unsigned long long v;
+};
+
+// what a run reports; written at its end by one thread into page-locked host memory (or the device copy)
+struct RunRes {
+    uint32_t verdict, witness, outer, status;
+    uint32_t nacc, gave_up;
+    unsigned long long inner_total, relax, frontier_rows, ph_rounds, ph_check;
+    uint32_t hist[RUN_HIST];
+};
+
+// zeroed before every run
+struct RunCtl {
+    Line64 bar[3];    // grid barriers by sequence number mod 3: arrivals << 48 | summed payload
+    Cnt32 lcnt[3];    // |list| by the run's round number mod 3
+    Cnt32 tcnt[2];    // |touched| by outer iteration mod 2
+    Cnt32 acnt;       // accepting vertices listed
+    Cnt32 xcnt, ecnt; // compaction: accepting vertices without a value, reader entries
+    Cnt32 witness;    // NONE - the smallest self-mapped vertex (0: none)
+    Line64 relax, frows;
+    uint32_t gave_up;
+    // what k_run leaves to k_tail: the compact graph and where the run stands
+    uint32_t hand, V, set, outer, nacc;
+    unsigned long long inner_total, ph_rounds, ph_check, t0;
+};
+
+struct RunArgs {
+    uint32_t n, words;
+    const uint32_t *rowptr, *rrowptr, *rcol, *acc0;
+    uint32_t *acc;
+    unsigned long long *W;       // 2n words, zero
+    uint32_t *la, *lb, *alist;   // n entries each: two lists, the accepting vertices
+    uint32_t *touched, *tval;    // n entries each: vertices with a value in this iteration, and that value
+    uint32_t *rank;              // n entries: original id -> 1 + number in the compact graph
+    uint32_t *pool;              // 3n words: two sets of compact arrays
+    RunCtl *ctl;
+    RunRes *res;
+    uint32_t *hist;              // rounds of every outer iteration (hist_cap entries)
+    uint32_t hist_cap;
+    uint32_t *out;               // map vector (MAP_NONE encoding), n entries; NULL: not wanted
+    uint64_t m;
+    uint32_t nacc0, max_outer, max_inner, lc_passes;
+    uint32_t count_round1;       // asynchronous relaxations: the pushes of round 1 (else m per iteration)
+    uint64_t timeout_ns;
+    uint32_t tail_cap;           // compact graphs of at most this many vertices are left to k_tail (0: none)
+    // batched runs
+    const uint32_t *comp;
+    CompState *cs;
+    uint32_t *chist;
+    uint32_t ncomp;
+};
+
+struct RunSmem {
+    uint32_t o[RT], b[RT], incl[RT], scan[RT / 32];
+    uint32_t list[RUN_CAP], touch[RUN_CAP];
+    uint32_t ln, tn, lbase, tbase;
+    unsigned long long word;
+    uint32_t ok, ebase;
+    unsigned long long part[RT / 32];
+};
+
+__device__ __forceinline__ uint32_t run_block_scan(uint32_t x, uint32_t *s)
+{
+    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+    x = warp_inclusive_scan(x);
+    if (lane == 31) s[warp] = x;
+    __syncthreads();
+    if (warp == 0) {
+        uint32_t t = lane < RT / 32 ? s[lane] : 0;
+#pragma unroll
+        for (int off = 1; off < RT / 32; off <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, t, off);
+            if (lane >= (unsigned)off) t += y;
+        }
+        if (lane < RT / 32) s[lane] = t;
+    }
+    __syncthreads();
+    return warp ? x + s[warp - 1] : x;
+}
+
+// payload of a barrier: a count (bits 0-31), blocks that found a self-mapped vertex (32-46), a stop request (47)
+constexpr unsigned long long RUN_STOP = 1ull << 47, RUN_FOUND = 1ull << 32, RUN_COUNT = RUN_FOUND - 1;
+
+// Bounded grid-wide barrier; every block adds `payload` (thread 0's) and *total gets the sum, so the
+// counts the next step needs come with the release instead of by another read.  One release
+// reduction to arrive, acquire loads to wait: 1.3 us with 304 blocks, against 2.6 us for a returning
+// atomic, a reset and a generation word with 912.  Returns false if the wait gave up.
+__device__ __forceinline__ bool run_barrier(RunCtl *c, RunSmem &sh, uint32_t &seq, unsigned long long payload,
+                                            unsigned long long &total)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const uint32_t slot = seq % 3;
+        // (the next barrier's word was last read before the barrier before this one)
+        if (blockIdx.x == 0) *(volatile unsigned long long *)&c->bar[(seq + 1) % 3].v = 0;
+        unsigned long long *w = &c->bar[slot].v, x = 0;
+        asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(w), "l"((1ull << 48) | payload) : "memory");
+        uint32_t ok = 1;
+        for (uint32_t it = 0;; ++it) {
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(x) : "l"(w) : "memory");
+            if ((x >> 48) == gridDim.x) break;
+            if (it > BAR_SPIN_LIMIT) {
+                ok = 0;
+                *(volatile uint32_t *)&c->gave_up = 1;
+                break;
+            }
+        }
+        sh.word = x & ((1ull << 48) - 1);
+        sh.ok = ok;
+    }
+    __syncthreads();
+    total = sh.word;
+    ++seq;
+    return sh.ok != 0;
+}
+
+// the space a run works in: the whole graph, or the compact graph of a later iteration
+struct Space {
+    uint32_t V, na;          // vertices, accepting vertices listed
+    const uint4 *meta;       // compact: (first reader, end, own offer, original id); NULL: the whole graph
+    const uint32_t *rc;      // readers
+    const uint32_t *row;     // compact: row lengths (NULL: from rowptr)
+    const uint32_t *comp;    // batched: graph of each vertex
+};
+
+// compact arrays, set h (0 or 1) in the pool of 3n words
+__device__ __forceinline__ uint32_t pool_cap(uint32_t n) { return (n / 8) & ~3u; }
+__device__ __forceinline__ uint32_t *pool_set(const RunArgs &a, uint32_t h) { return a.pool + (uint64_t)h * ((a.n + a.n / 2) & ~3u); }
+
+template <bool SYNC, bool BATCH> struct Run {
+    static constexpr uint32_t S = (SYNC || BATCH) ? 2 : 1; // state words per vertex
+
+    const RunArgs &a;
+    RunSmem &sh;
+    Space sp;
+    uint32_t seq = 0, lseq = 0; // barriers and rounds of the whole run so far
+    unsigned long long relax = 0, frows = 0;
+
+    __device__ Run(const RunArgs &a_, RunSmem &s_) : a(a_), sh(s_) {}
+
+    __device__ __forceinline__ uint32_t id_of(uint32_t v) const { return sp.meta ? __ldcg(&sp.meta[v].w) : v; }
+    __device__ __forceinline__ bool accepting(uint32_t v) const
+    {
+        return sp.meta ? __ldcg(&sp.meta[v].z) != 0 : ((__ldcg(a.acc + (v >> 5)) >> (v & 31u)) & 1u) != 0;
+    }
+
+    __device__ __forceinline__ uint32_t readers(uint32_t v) const
+    {
+        if (!sp.meta) return __ldg(a.rrowptr + v + 1) - __ldg(a.rrowptr + v);
+        const uint4 q = __ldcg(sp.meta + v);
+        return q.y - q.x;
+    }
+
+    // append w (where flag) to the staged list s_buf (count *s_cnt); what does not fit goes to g directly
+    __device__ __forceinline__ void emit(bool flag, uint32_t w, uint32_t *s_buf, uint32_t *s_cnt, uint32_t *g, uint32_t *gcnt)
+    {
+        const unsigned mask = __ballot_sync(0xFFFFFFFFu, flag);
+        if (!mask) return;
+        const unsigned lane = lane_id(), leader = __ffs(mask) - 1;
+        uint32_t pos = 0;
+        if (lane == leader) pos = atomicAdd(s_cnt, (uint32_t)__popc(mask));
+        pos = __shfl_sync(0xFFFFFFFFu, pos, leader) + __popc(mask & ((1u << lane) - 1u));
+        const bool over = flag && pos >= RUN_CAP;
+        if (flag && !over) s_buf[pos] = w;
+        if (__any_sync(0xFFFFFFFFu, over)) {
+            const unsigned om = __ballot_sync(0xFFFFFFFFu, over);
+            uint32_t at = 0;
+            const unsigned ol = __ffs(om) - 1;
+            if (lane == ol) at = atomicAdd(gcnt, (uint32_t)__popc(om));
+            at = __shfl_sync(0xFFFFFFFFu, at, ol) + __popc(om & ((1u << lane) - 1u));
+            if (over) g[at] = w;
+        }
+    }
+
+    // entries [beg, end) in chunks of RT per block: get(i, o, b, len) gives an entry's offer and reader
+    // range, begin(total) runs once per chunk, and the (offer, reader position) pairs are spread
+    // evenly over the block's threads, RUN_P per thread and step: act(live, o, pos) for RUN_P pairs
+    template <class Get, class Begin, class Act>
+    __device__ __forceinline__ void expand(uint64_t beg, uint64_t end, Get get, Begin begin, Act act)
+    {
+        for (uint64_t c0 = beg; c0 < end; c0 += RT) {
+            const uint64_t i = c0 + threadIdx.x;
+            uint32_t o = 0, b = 0, len = 0;
+            if (i < end) get(i, o, b, len);
+            const uint32_t incl = run_block_scan(len, sh.scan);
+            sh.o[threadIdx.x] = o;
+            sh.b[threadIdx.x] = b - (incl - len); // reader position of pair p: b[owner] + p (32-bit wrap intended)
+            sh.incl[threadIdx.x] = incl;
+            __syncthreads();
+            const uint32_t total = sh.incl[RT - 1];
+            begin(i < end, i, incl - len, len, total);
+            for (uint64_t p0 = 0; p0 < total; p0 += RT * RUN_P) {
+                bool live[RUN_P];
+                uint32_t off[RUN_P], pos[RUN_P], pair[RUN_P];
+#pragma unroll
+                for (int j = 0; j < RUN_P; ++j) {
+                    const uint64_t p = p0 + j * RT + threadIdx.x;
+                    live[j] = p < total;
+                    off[j] = pos[j] = 0;
+                    pair[j] = (uint32_t)p;
+                    if (live[j]) {
+                        uint32_t lo = 0, hi = RT - 1; // the owner: first entry with incl > p
+#pragma unroll
+                        for (int st = 0; st < 9; ++st) {
+                            const uint32_t mid = (lo + hi) >> 1;
+                            if (sh.incl[mid] > (uint32_t)p) hi = mid;
+                            else lo = min(mid + 1, hi);
+                        }
+                        off[j] = sh.o[lo];
+                        pos[j] = sh.b[lo] + (uint32_t)p;
+                    }
+                }
+                act(live, off, pos, pair);
+            }
+            __syncthreads(); // before the shared arrays are refilled
+        }
+    }
+
+    // one push of offer o to reader w in round r: raised first in this round, with no value
+    // before, and (where counted) first reached in this round
+    struct Pushed {
+        bool listed, fresh, row;
+    };
+    __device__ __forceinline__ void push(const bool (&live)[RUN_P], const uint32_t (&o)[RUN_P], const uint32_t (&w)[RUN_P],
+                                         uint32_t r, Pushed (&out)[RUN_P])
+    {
+        if constexpr (SYNC) {
+            ulonglong2 rec[RUN_P];
+#pragma unroll
+            for (int j = 0; j < RUN_P; ++j)
+                rec[j] = live[j] ? __ldcg(reinterpret_cast<const ulonglong2 *>(a.W) + w[j]) : make_ulonglong2(0, 0);
+            unsigned long long neww[RUN_P], old[RUN_P];
+            bool todo[RUN_P];
+            uint32_t base[RUN_P];
+            const unsigned long long stamp = (unsigned long long)r << 33;
+#pragma unroll
+            for (int j = 0; j < RUN_P; ++j) {
+                const unsigned long long cur = (r & 1) ? rec[j].y : rec[j].x, prev = (r & 1) ? rec[j].x : rec[j].y;
+                const uint32_t cv = (uint32_t)cur;
+                if ((cur >> 33) != r) { // not reached in this round yet: the value so far is the larger word's
+                    base[j] = max(cv, (uint32_t)prev);
+                    neww[j] = stamp | ((unsigned long long)(o[j] > base[j]) << 32) | max(o[j], base[j]);
+                    todo[j] = live[j];
+                } else { // reached: the word holds the value so far (not raised) or the best offer (raised)
+                    base[j] = cv;
+                    neww[j] = stamp | (1ull << 32) | o[j];
+                    todo[j] = live[j] && o[j] > cv;
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < RUN_P; ++j) old[j] = todo[j] ? atomicMax(a.W + 2ull * w[j] + (r & 1), neww[j]) : 0ull;
+#pragma unroll
+            for (int j = 0; j < RUN_P; ++j) {
+                const bool mine = (old[j] >> 33) == r; // this round's already
+                out[j].row = todo[j] && !mine;
+                out[j].listed = todo[j] && ((neww[j] >> 32) & 1u) && !(mine && ((old[j] >> 32) & 1u));
+                out[j].fresh = out[j].listed && base[j] == 0;
+            }
+        } else {
+            unsigned long long old[RUN_P];
+            uint32_t seen[RUN_P];
+#pragma unroll
+            for (int j = 0; j < RUN_P; ++j) {
+                seen[j] = r;
+                if (BATCH && live[j]) seen[j] = atomicExch(reinterpret_cast<uint32_t *>(a.W + 2ull * w[j] + 1), r);
+                old[j] = live[j] ? atomicMax(a.W + (uint64_t)S * w[j], ((unsigned long long)o[j] << 32) | (uint32_t)~r)
+                                 : ~0ull;
+            }
+#pragma unroll
+            for (int j = 0; j < RUN_P; ++j) {
+                const bool rose = live[j] && (uint32_t)(old[j] >> 32) < o[j];
+                out[j].row = live[j] && seen[j] != r;
+                out[j].listed = rose && (uint32_t)old[j] != (uint32_t)~r;
+                out[j].fresh = rose && (old[j] >> 32) == 0;
+            }
+        }
+    }
+
+    // the value a vertex listed in round r - 1 offers in round r (live, asynchronous)
+    __device__ __forceinline__ uint32_t value_of(uint32_t u, uint32_t r) const
+    {
+        if constexpr (SYNC) return (uint32_t)__ldcg(a.W + 2ull * u + ((r - 1) & 1));
+        else return (uint32_t)(__ldcg(a.W + (uint64_t)S * u) >> 32);
+    }
+
+    __device__ __forceinline__ void entry(uint32_t u, uint32_t r, bool with_value, uint32_t &o, uint32_t &b, uint32_t &len)
+    {
+        const uint32_t val = with_value ? value_of(u, r) : 0u;
+        uint32_t e;
+        if (sp.meta) {
+            const uint4 q = __ldcg(sp.meta + u);
+            b = q.x;
+            e = q.y;
+            o = max(val, q.z);
+        } else {
+            b = __ldg(a.rrowptr + u);
+            e = __ldg(a.rrowptr + u + 1);
+            o = max(val, ((__ldcg(a.acc + (u >> 5)) >> (u & 31u)) & 1u) ? u + 1 : 0u);
+        }
+        // round 1: an eliminated vertex offers nothing, nor does one of a finished graph
+        bool idle = o == 0;
+        if (BATCH && !with_value) idle = idle || !*(volatile uint32_t *)&a.cs[__ldcg(sp.comp + u)].active;
+        len = idle ? 0u : e - b;
+    }
+
+    __device__ __forceinline__ void add_row(bool row, uint32_t w)
+    { // a frontier row: its length to the relaxation count (batched: of its graph)
+        unsigned long long len = 0;
+        if (row) {
+            len = sp.row ? __ldcg(sp.row + w) : __ldg(a.rowptr + w + 1) - __ldg(a.rowptr + w);
+            relax += len;
+            ++frows;
+        }
+        if constexpr (BATCH) {
+            const uint32_t c = row ? __ldcg(sp.comp + w) : NONE;
+            const unsigned same = __match_any_sync(0xFFFFFFFFu, c);
+            const unsigned lo = __reduce_add_sync(same, (unsigned)(len & 0xFFFFu));
+            const unsigned hi = __reduce_add_sync(same, (unsigned)(len >> 16));
+            const unsigned long long sum = (unsigned long long)lo + ((unsigned long long)hi << 16);
+            if (c != NONE && lane_id() == (unsigned)(__ffs(same) - 1) && sum)
+                atomicAdd((unsigned long long *)&a.cs[c].relax, sum);
+        }
+    }
+
+    // one round over `list` (nl entries); returns false if a wait gave up
+    __device__ __forceinline__ bool round(const uint32_t *list, uint32_t nl, uint32_t *next, uint32_t r, uint32_t outer,
+                                          bool timing, unsigned long long &total)
+    {
+        RunCtl *c = a.ctl;
+        // (list counters rotate by the run's round number: the one after this was last used two rounds ago)
+        ++lseq;
+        uint32_t *lcnt = &c->lcnt[lseq % 3].v, *tcnt = &c->tcnt[outer & 1].v;
+        if (threadIdx.x == 0) {
+            sh.ln = sh.tn = 0;
+            if (blockIdx.x == 0) *(volatile uint32_t *)&c->lcnt[(lseq + 1) % 3].v = 0;
+        }
+        __syncthreads();
+        const uint64_t per = ((uint64_t)nl + gridDim.x - 1) / gridDim.x;
+        const uint64_t beg = min((uint64_t)nl, blockIdx.x * per), end = min((uint64_t)nl, beg + per);
+        bool local = false;
+        auto get = [&](uint64_t i, uint32_t &o, uint32_t &b, uint32_t &len) {
+            entry(local ? sh.list[i] : __ldcg(list + i), r, local || r > 1, o, b, len);
+        };
+        auto begin = [&](bool, uint64_t, uint32_t, uint32_t, uint32_t tot) {
+            if (!SYNC && !BATCH && threadIdx.x == 0 && (r > 1 || local || a.count_round1)) relax += tot;
+        };
+        auto act = [&](const bool (&live)[RUN_P], const uint32_t (&o)[RUN_P], const uint32_t (&pos)[RUN_P],
+                       const uint32_t (&)[RUN_P]) {
+            uint32_t w[RUN_P];
+            Pushed done[RUN_P];
+#pragma unroll
+            for (int j = 0; j < RUN_P; ++j) w[j] = live[j] ? __ldcg(sp.rc + pos[j]) : 0u; // (compact: written in this launch)
+            push(live, o, w, r, done);
+#pragma unroll
+            for (int j = 0; j < RUN_P; ++j) {
+                if ((SYNC || BATCH) && r > 1) add_row(done[j].row, w[j]);
+                if (BATCH && done[j].listed) {
+                    CompState &s = a.cs[__ldcg(sp.comp + w[j])];
+                    if (*(volatile uint32_t *)&s.last_change < r) atomicMax(&s.last_change, r);
+                }
+                emit(done[j].listed, w[j], sh.list, &sh.ln, next, lcnt);
+                emit(done[j].fresh, w[j], sh.touch, &sh.tn, a.touched, tcnt);
+            }
+        };
+        expand(beg, end, get, begin, act);
+        if (!SYNC && !BATCH) {
+            // the block pushes the live values of the vertices it listed itself once more (lc_passes
+            // times), so that values travel several edges per barrier; they stay listed
+            uint32_t q = 0;
+            local = true;
+            for (uint32_t pass = 0; pass < a.lc_passes; ++pass) {
+                const uint32_t e = min(sh.ln, RUN_CAP); // final: a block barrier ended the last chunk
+                __syncthreads();                        // (read by every thread before it grows)
+                if (e == q) break;
+                expand(q, e, get, begin, act);
+                q = e;
+            }
+        }
+        __syncthreads();
+        const uint32_t ln = sh.ln, kept = min(ln, RUN_CAP), tkept = min(sh.tn, RUN_CAP);
+        if (threadIdx.x == 0 && kept) sh.lbase = atomicAdd(lcnt, kept);
+        if (threadIdx.x == 32 && tkept) sh.tbase = atomicAdd(tcnt, tkept);
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < kept; i += RT) next[sh.lbase + i] = sh.list[i];
+        for (uint32_t i = threadIdx.x; i < tkept; i += RT) a.touched[sh.tbase + i] = sh.touch[i];
+        return run_barrier(c, sh, seq, (unsigned long long)ln + (timing ? RUN_STOP : 0ull), total);
+    }
+};
+
+// per-graph end of an outer iteration in a batched run: does graph S go on?
+__device__ __forceinline__ bool comp_goes_on(const volatile CompState &S, uint32_t status, uint32_t max_outer, uint32_t &left,
+                                             bool &limit)
+{
+    limit = false;
+    left = S.nacc;
+    if (status != ST_OK || S.witness != NONE || S.touched == 0) return false;
+    left = S.nacc - S.elim;
+    if (left == 0) return false;
+    limit = (max_outer && S.outer >= max_outer) || S.outer > S.nacc0;
+    return !limit;
+}
+
+template <bool SYNC, bool BATCH>
+__global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_constant__ RunArgs a)
+{
+    __shared__ RunSmem sh;
+    Run<SYNC, BATCH> run(a, sh);
+    RunCtl *c = a.ctl;
+    const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
+    const uint64_t tid = (uint64_t)blockIdx.x * RT + threadIdx.x, nthreads = (uint64_t)gridDim.x * RT;
+    const uint32_t n = a.n;
+    const uint64_t t0 = global_ns();
+    uint64_t mark = t0, ph_rounds = 0, ph_check = 0;
+    auto phase = [&](uint64_t &acc) {
+        const uint64_t now = global_ns();
+        if ((int64_t)(now - mark) > 0) {
+            acc += now - mark;
+            mark = now;
+        }
+    };
+    auto late = [&] { return lead && (int64_t)(global_ns() - t0) > (int64_t)a.timeout_ns; };
+    uint32_t *la = a.la, *lb = a.lb, *alist = a.alist;
+    unsigned long long total = 0;
+    bool alive = true; // no wait has given up
+
+    // the accepting set of the run, the list of its vertices, and an empty map vector
+    for (uint64_t base = tid - threadIdx.x; base < a.words; base += nthreads) { // (block-uniform)
+        const uint64_t i = base + threadIdx.x;
+        uint32_t x = i < a.words ? __ldg(a.acc0 + i) : 0u;
+        if (i < a.words) a.acc[i] = x;
+        const uint32_t incl = run_block_scan(__popc(x), sh.scan);
+        if (threadIdx.x == RT - 1) sh.lbase = incl ? atomicAdd(&c->acnt.v, incl) : 0u;
+        __syncthreads();
+        uint32_t at = sh.lbase + incl - __popc(x);
+        for (; x; x &= x - 1) alist[at++] = (uint32_t)i * 32u + __ffs(x) - 1;
+        __syncthreads();
+    }
+    if (!a.out) {
+        // (no map asked for)
+    } else if (((uintptr_t)a.out & 15u) == 0) {
+        uint4 *o4 = reinterpret_cast<uint4 *>(a.out);
+        for (uint64_t i = tid; i < n / 4; i += nthreads) o4[i] = make_uint4(NONE, NONE, NONE, NONE);
+        for (uint64_t i = (uint64_t)(n / 4) * 4 + tid; i < n; i += nthreads) a.out[i] = NONE;
+    } else {
+        for (uint64_t i = tid; i < n; i += nthreads) a.out[i] = NONE;
+    }
+    alive = run_barrier(c, sh, run.seq, 0, total);
+
+    Space &sp = run.sp;
+    sp.V = n;
+    sp.na = a.nacc0;
+    sp.meta = nullptr;
+    sp.rc = a.rcol;
+    sp.row = nullptr;
+    sp.comp = a.comp;
+    uint32_t outer = 0, status = ST_OK, verdict = 0, witness = NONE, nacc = a.nacc0, set = 1;
+    unsigned long long inner_total = 0;
+    bool go = a.nacc0 != 0, compactable = true, hand = false;
+    while (go && alive) {
+        ++outer;
+        if (lead && (SYNC || !a.count_round1)) run.relax += a.m; // round 1 covers every row
+        // ---- rounds to the fix-point
+        const uint32_t *list = alist;
+        uint32_t nl = sp.na, r = 0;
+        for (;;) {
+            ++r;
+            alive = run.round(list, nl, (r & 1) ? la : lb, r, outer, (r & 3u) == 0 && late(), total);
+            if (!alive) break;
+            if (!SYNC && !BATCH && r > 1) run.frows += lead ? nl : 0u; // the vertices that pushed
+            nl = (uint32_t)(total & RUN_COUNT);
+            list = (r & 1) ? la : lb;
+            if (total & RUN_STOP) status = ST_TIMEOUT;
+            else if (nl && r + 1 > a.max_inner) status = ST_LIMIT;
+            if (!nl || status != ST_OK) break;
+        }
+        if (!alive) break;
+        inner_total += r;
+        if (lead) {
+            if (outer - 1 < a.hist_cap) a.hist[outer - 1] = r;
+            if (outer - 1 < RUN_HIST) a.res->hist[outer - 1] = r;
+            phase(ph_rounds);
+        }
+        // ---- self-map test and elimination over the vertices with a value; their state back to zero
+        const uint32_t T = *(volatile uint32_t *)&c->tcnt[outer & 1].v;
+        if (lead) *(volatile uint32_t *)&c->tcnt[(outer + 1) & 1].v = 0;
+        uint32_t elim = 0, wit = NONE, settled = 0;
+        for (uint64_t base = tid - lane_id(); base < T; base += nthreads) { // (warp-uniform)
+            const uint64_t i = base + lane_id();
+            uint32_t g = NONE, removed = 0, val = 0;
+            if (i < T) {
+                const uint32_t v = __ldcg(a.touched + i);
+                // (exchanges, not stores: scattered 8-byte stores ran at 14 G/s here, atomics at over 100)
+                uint32_t x;
+                if constexpr (SYNC) {
+                    x = max((uint32_t)atomicExch(a.W + 2ull * v, 0ull), (uint32_t)atomicExch(a.W + 2ull * v + 1, 0ull));
+                } else {
+                    x = (uint32_t)(atomicExch(a.W + (uint64_t)run.S * v, 0ull) >> 32);
+                    if (BATCH) atomicExch(a.W + 2ull * v + 1, 0ull);
+                }
+                a.tval[i] = x;
+                if (BATCH) g = __ldcg(sp.comp + v);
+                if (status == ST_OK) val = x;
+                if (val && x - 1 == run.id_of(v)) {
+                    wit = min(wit, x - 1);
+                    if (BATCH) atomicMin(&a.cs[g].witness, x - 1);
+                }
+            }
+            // u = val - 1 is removed.  Many vertices share a few map values: one lane per value and warp, and
+            // none for the value this thread settled last
+            const unsigned same_val = __match_any_sync(0xFFFFFFFFu, val);
+            if (val && val != settled && lane_id() == (unsigned)(__ffs(same_val) - 1)) {
+                const uint32_t u = val - 1, bit = 1u << (u & 31u);
+                if ((__ldcg(a.acc + (u >> 5)) & bit) && (atomicAnd(a.acc + (u >> 5), ~bit) & bit)) { // this thread removed u
+                    ++elim;
+                    removed = 1;
+                    if (sp.meta) const_cast<uint4 *>(sp.meta)[__ldcg(a.rank + u) - 1].z = 0; // it offers nothing any more
+                }
+            }
+            settled = val;
+            if constexpr (BATCH) { // per graph: vertices with a value and removals, one atomic per graph in the warp
+                const unsigned same = __match_any_sync(0xFFFFFFFFu, g);
+                const unsigned ne = __reduce_add_sync(same, removed);
+                if (g != NONE && lane_id() == (unsigned)(__ffs(same) - 1)) {
+                    atomicAdd(&a.cs[g].touched, (unsigned)__popc(same));
+                    if (ne) atomicAdd(&a.cs[g].elim, ne);
+                }
+            }
+        }
+        { // block sums
+            elim = __reduce_add_sync(0xFFFFFFFFu, elim);
+            wit = __reduce_min_sync(0xFFFFFFFFu, wit);
+            __syncthreads();
+            if (threadIdx.x == 0) sh.ln = 0, sh.tn = NONE;
+            __syncthreads();
+            if (lane_id() == 0) {
+                if (elim) atomicAdd(&sh.ln, elim);
+                if (wit != NONE) atomicMin(&sh.tn, wit);
+            }
+            __syncthreads();
+            elim = sh.ln;
+            wit = sh.tn;
+            if (threadIdx.x == 0 && wit != NONE) atomicMax(&c->witness.v, NONE - wit);
+        }
+        alive = run_barrier(c, sh, run.seq,
+                            (unsigned long long)elim + (wit != NONE ? RUN_FOUND : 0ull) + (late() ? RUN_STOP : 0ull), total);
+        if (!alive) break;
+        if (lead) phase(ph_check);
+        if constexpr (!BATCH) {
+            if (status != ST_OK) go = false; // a limit inside the rounds
+            else if (total & (RUN_STOP - RUN_FOUND)) {
+                verdict = 1;
+                witness = NONE - *(volatile uint32_t *)&c->witness.v;
+                go = false;
+            } else if (T == 0) {
+                go = false; // nothing reaches a remaining accepting vertex
+            } else {
+                nacc -= (uint32_t)(total & RUN_COUNT);
+                if (nacc == 0) go = false;
+                else if ((a.max_outer && outer >= a.max_outer) || outer > a.nacc0) {
+                    status = ST_LIMIT;
+                    go = false;
+                } else if (total & RUN_STOP) {
+                    status = ST_TIMEOUT;
+                    go = false;
+                }
+            }
+            if (!go && a.out) // the last iteration's map
+                for (uint64_t i = tid; i < T; i += nthreads)
+                    a.out[run.id_of(__ldcg(a.touched + i))] = __ldcg(a.tval + i) - 1u;
+        } else {
+            if (status == ST_OK && (total & RUN_STOP)) status = ST_TIMEOUT;
+            uint32_t left;
+            bool limit;
+            // the maps of the graphs that end here
+            for (uint64_t i = tid; a.out && i < T; i += nthreads) {
+                const uint32_t v = __ldcg(a.touched + i), g = __ldcg(sp.comp + v);
+                if (!comp_goes_on(a.cs[g], status, a.max_outer, left, limit))
+                    a.out[run.id_of(v)] = __ldcg(a.tval + i) - 1u - *(volatile uint32_t *)&a.cs[g].off;
+            }
+            nacc -= (uint32_t)(total & RUN_COUNT);
+            alive = run_barrier(c, sh, run.seq, 0, total);
+            if (!alive) break;
+            unsigned on = 0;
+            if (blockIdx.x == 0) {
+                for (uint32_t g = threadIdx.x; g < a.ncomp; g += RT) {
+                    volatile CompState &S = a.cs[g];
+                    if (!S.active) continue;
+                    const uint32_t it = S.outer, rounds = S.last_change + 1;
+                    if (it - 1 < CH_CAP) a.chist[(size_t)g * CH_CAP + it - 1] = rounds;
+                    S.inner_total = S.inner_total + rounds;
+                    S.relax = S.relax + S.m; // round 1 covers every row
+                    const bool more = comp_goes_on(S, status, a.max_outer, left, limit);
+                    if (status != ST_OK) S.status = status;
+                    else if (limit) S.status = ST_LIMIT;
+                    if (status == ST_OK && S.witness != NONE) S.verdict = 1;
+                    else S.nacc = left;
+                    if (more) {
+                        S.outer = it + 1;
+                        S.witness = NONE;
+                        S.elim = S.touched = S.last_change = 0;
+                        ++on;
+                    } else {
+                        S.active = 0;
+                    }
+                }
+                on = __reduce_add_sync(0xFFFFFFFFu, on);
+                __syncthreads();
+                if (threadIdx.x == 0) sh.ln = 0;
+                __syncthreads();
+                if (lane_id() == 0 && on) atomicAdd(&sh.ln, on);
+                __syncthreads();
+                on = sh.ln;
+            }
+            alive = run_barrier(c, sh, run.seq, on, total);
+            if (!alive) break;
+            go = (total & RUN_COUNT) != 0;
+        }
+        // ---- compaction: go on in the graph of the vertices that had a value and the accepting ones
+        const uint32_t cap = pool_cap(n);
+        if (go && compactable && (uint64_t)T + nacc <= min(sp.V / (sp.meta ? 4u : 8u), cap)) {
+            for (uint64_t i = tid; i < T; i += nthreads) a.rank[run.id_of(__ldcg(a.touched + i))] = (uint32_t)i + 1;
+            if (lead) *(volatile uint32_t *)&c->acnt.v = 0;
+            if (!(alive = run_barrier(c, sh, run.seq, 0, total))) break;
+            uint32_t *anew = la; // (no round is in flight)
+            for (uint64_t i = tid; i < sp.na; i += nthreads) { // (one that no row holds offers nothing to anyone)
+                const uint32_t v = __ldcg(alist + i);
+                if (run.readers(v) == 0) continue;
+                if (!run.accepting(v) || (BATCH && !*(volatile uint32_t *)&a.cs[__ldcg(sp.comp + v)].active)) continue;
+                const uint32_t u = run.id_of(v);
+                uint32_t k = __ldcg(a.rank + u);
+                if (!(k >= 1 && k <= T && __ldcg(a.touched + k - 1) == v)) { // it has no value: after those that have
+                    k = T + agg_inc(&c->xcnt.v) + 1;
+                    a.touched[k - 1] = v;
+                    a.rank[u] = k;
+                }
+                anew[agg_inc(&c->acnt.v)] = k - 1;
+            }
+            if (!(alive = run_barrier(c, sh, run.seq, 0, total))) break;
+            const uint32_t V2 = T + *(volatile uint32_t *)&c->xcnt.v, na2 = *(volatile uint32_t *)&c->acnt.v;
+            uint32_t *const ps = pool_set(a, set ^ 1);
+            uint4 *const meta2 = reinterpret_cast<uint4 *>(ps);
+            uint32_t *const row2 = ps + 4ull * cap, *const comp2 = row2 + cap, *const rc2 = comp2 + cap;
+            const uint64_t ecap = (uint64_t)n * 3 / 4 - 8;
+            bool over = false;
+            const uint64_t per = ((uint64_t)V2 + gridDim.x - 1) / gridDim.x;
+            const uint64_t beg = min((uint64_t)V2, blockIdx.x * per), end = min((uint64_t)V2, beg + per);
+            uint32_t first = 0; // this chunk's first entry in rc2
+            run.expand(
+                beg, end,
+                [&](uint64_t i, uint32_t &, uint32_t &b, uint32_t &len) {
+                    const uint32_t v = __ldcg(a.touched + i);
+                    if (sp.meta) {
+                        const uint4 q = __ldcg(sp.meta + v);
+                        b = q.x;
+                        len = q.y - q.x;
+                    } else {
+                        b = __ldg(a.rrowptr + v);
+                        len = __ldg(a.rrowptr + v + 1) - b;
+                    }
+                },
+                [&](bool in, uint64_t i, uint32_t excl, uint32_t len, uint32_t tot) {
+                    if (threadIdx.x == 0) sh.ebase = tot ? atomicAdd(&c->ecnt.v, tot) : 0u;
+                    __syncthreads();
+                    first = sh.ebase;
+                    if ((uint64_t)first + tot > ecap) over = true;
+                    if (in) {
+                        const uint32_t v = __ldcg(a.touched + i), u = run.id_of(v);
+                        meta2[i] = make_uint4(first + excl, first + excl + len, run.accepting(v) ? u + 1 : 0u, u);
+                        if (SYNC || BATCH)
+                            row2[i] = sp.row ? __ldcg(sp.row + v) : __ldg(a.rowptr + v + 1) - __ldg(a.rowptr + v);
+                        if (BATCH) comp2[i] = __ldcg(sp.comp + v);
+                    }
+                },
+                [&](const bool (&live)[RUN_P], const uint32_t (&)[RUN_P], const uint32_t (&pos)[RUN_P],
+                    const uint32_t (&pair)[RUN_P]) {
+                    if (over) return;
+#pragma unroll
+                    for (int j = 0; j < RUN_P; ++j)
+                        if (live[j]) rc2[first + pair[j]] = __ldcg(a.rank + run.id_of(__ldcg(sp.rc + pos[j]))) - 1;
+                });
+            if (!(alive = run_barrier(c, sh, run.seq, over ? 1 : 0, total))) break;
+            if (lead) *(volatile uint32_t *)&c->xcnt.v = *(volatile uint32_t *)&c->ecnt.v = 0;
+            if (total & RUN_COUNT) { // too many readers for the pool: stay in the whole graph
+                compactable = false;
+            } else {
+                sp.V = V2;
+                sp.na = na2;
+                sp.meta = meta2;
+                sp.rc = rc2;
+                sp.row = row2;
+                sp.comp = comp2;
+                set ^= 1;
+                uint32_t *const t = alist;
+                alist = la;
+                la = t;
+                if (!BATCH && V2 <= a.tail_cap) { // small enough for one cluster
+                    hand = true;
+                    break;
+                }
+            }
+        }
+    }
+    // ---- the result
+    for (unsigned long long *p : {&run.relax, &run.frows}) {
+        const unsigned long long s = warp_sum64(*p);
+        __syncthreads();
+        if (lane_id() == 0) sh.part[threadIdx.x >> 5] = s;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            unsigned long long t = 0;
+            for (int w = 0; w < RT / 32; ++w) t += sh.part[w];
+            if (t) atomicAdd(p == &run.relax ? &c->relax.v : &c->frows.v, t);
+        }
+    }
+    if (hand) {
+        if (lead) {
+            c->V = sp.V;
+            c->set = set;
+            c->outer = outer;
+            c->nacc = nacc;
+            c->inner_total = inner_total;
+            c->ph_rounds = ph_rounds;
+            c->ph_check = ph_check;
+            c->t0 = t0;
+            c->hand = 1;
+        }
+        return;
+    }
+    if (alive) alive = run_barrier(c, sh, run.seq, 0, total);
+    if (lead) {
+        RunRes *R = a.res;
+        R->verdict = verdict;
+        R->witness = witness;
+        R->outer = outer;
+        R->status = alive ? status : ST_TIMEOUT;
+        R->gave_up = alive ? 0u : 1u;
+        R->nacc = nacc;
+        R->inner_total = inner_total;
+        R->relax = *(volatile unsigned long long *)&c->relax.v;
+        R->frontier_rows = *(volatile unsigned long long *)&c->frows.v;
+        R->ph_rounds = ph_rounds;
+        R->ph_check = ph_check;
+    }
+}
+
+// ------------------------------------------------------------ small graphs --
+//
+// k_tail: the same run in one thread-block cluster with the vertices' state in shared memory, for a
+// whole graph of at most TAIL_N vertices per block, or for the compact graph that k_run leaves.
+// A round over a few thousand vertices is a chain of latencies: through L2 and the grid barrier it
+// takes 6-7 us, here 1 us or less -- a push is one 32-bit maximum into the owner's shared memory
+// (nothing waits for it), and the cluster barrier takes 0.3 us.  There are no lists: vertex v belongs
+// to block v mod C, and every round its owner looks whether it changed, which costs a few
+// shared-memory reads per thread.
+//   asynchronous  pushes raise the vertex's value itself; it changed if it is above the value it
+//                 pushed last;
+//   synchronous   pushes of round r go to the vertex's inbox of r's parity; in round r + 1 the owner
+//                 takes what came in (the vertex was in round r's frontier: its row length to the
+//                 relaxation count) and, if that is above the value, raises it and pushes.
+constexpr int TT = 1024;             // threads per block
+constexpr uint32_t TAIL_N = 8704;    // vertices per block: 26 bytes of shared memory each
+constexpr uint32_t TAIL_C = 16;      // blocks at most
+constexpr size_t TAIL_SMEM = (size_t)TAIL_N * 26;
+constexpr uint32_t TAIL_LONG = 16;   // reader lists longer than this are walked by a whole warp
+
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_barrier()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// the address of this block's shared word `local` in block `rank` of the cluster
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t local, uint32_t rank)
+{
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_max(uint32_t addr, uint32_t x)
+{
+    asm volatile("red.relaxed.cluster.shared::cluster.max.u32 [%0], %1;" ::"r"(addr), "r"(x) : "memory");
+}
+__device__ __forceinline__ void cluster_or(uint32_t addr, uint32_t x)
+{
+    asm volatile("red.relaxed.cluster.shared::cluster.or.b32 [%0], %1;" ::"r"(addr), "r"(x) : "memory");
+}
+__device__ __forceinline__ void cluster_store(uint32_t addr, unsigned long long x)
+{
+    asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(x) : "memory");
+}
+__device__ __forceinline__ uint32_t shared_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+template <bool SYNC>
+__global__ void __launch_bounds__(TT, 1) k_tail(const __grid_constant__ RunArgs a, uint32_t whole)
+{
+    extern __shared__ uint32_t s_mem[];
+    __shared__ unsigned long long s_word[2][TAIL_C], s_part[TT / 32], s_sum;
+    __shared__ uint32_t s_min[TT / 32], s_n, s_late;
+    RunCtl *c = a.ctl;
+    if (!whole && !*(volatile uint32_t *)&c->hand) return; // k_run finished the run (every block returns)
+    const uint32_t C = gridDim.x, rank = cluster_rank(), cshift = __ffs(C) - 1, cmask = C - 1;
+    const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+    const uint32_t V = whole ? a.n : *(volatile uint32_t *)&c->V;
+    const uint32_t mine = V > rank ? (V - rank + C - 1) >> cshift : 0u; // vertices rank, rank + C, ...
+    // asynchronous: x0 / x1 = the values, by outer iteration mod 2, x2 = the value pushed last
+    // synchronous: x0 / x1 = the inboxes, by round mod 2, x2 = the value
+    uint32_t *const x0 = s_mem, *const x1 = x0 + TAIL_N, *const x2 = x1 + TAIL_N, *const own = x2 + TAIL_N,
+                    *const beg = own + TAIL_N, *const end = beg + TAIL_N;
+    uint16_t *const queue = reinterpret_cast<uint16_t *>(end + TAIL_N);
+    const uint32_t set = whole ? 0u : *(volatile uint32_t *)&c->set, cap = pool_cap(a.n);
+    uint32_t *const ps = pool_set(a, set);
+    const uint4 *meta = reinterpret_cast<const uint4 *>(ps);
+    const uint32_t *row = ps + 4ull * cap, *rc = whole ? a.rcol : ps + 6ull * cap;
+    for (uint32_t i = tid; i < mine; i += TT) {
+        const uint32_t v = i << cshift | rank;
+        x0[i] = x1[i] = x2[i] = 0;
+        if (whole) {
+            own[i] = ((__ldg(a.acc0 + (v >> 5)) >> (v & 31u)) & 1u) ? v + 1 : 0u;
+            beg[i] = __ldg(a.rrowptr + v);
+            end[i] = __ldg(a.rrowptr + v + 1);
+        } else {
+            const uint4 q = __ldg(meta + v);
+            beg[i] = q.x;
+            end[i] = q.y;
+            own[i] = q.z;
+        }
+    }
+    const uint64_t t0 = whole ? global_ns() : *(volatile unsigned long long *)&c->t0;
+    const bool lead = rank == 0 && tid == 0;
+    uint64_t mark = global_ns(), ph_rounds = 0, ph_check = 0;
+    auto phase = [&](uint64_t &acc) {
+        const uint64_t now = global_ns();
+        if ((int64_t)(now - mark) > 0) {
+            acc += now - mark;
+            mark = now;
+        }
+    };
+    uint32_t outer = whole ? 0u : *(volatile uint32_t *)&c->outer, nacc = whole ? a.nacc0 : *(volatile uint32_t *)&c->nacc;
+    uint32_t status = ST_OK, verdict = 0, witness = NONE, seq = 0;
+    unsigned long long relax = 0, frows = 0, inner_total = 0;
+    // every block's word (the same in its threads 0 .. C - 1) to every block, then the cluster barrier; the
+    // calling lane q < C gets block q's word.  The words alternate between two buffers: one is rewritten only
+    // after the barrier that follows the reads of its last contents.
+    auto exchange = [&](unsigned long long w) {
+        const uint32_t k = seq++ & 1u;
+        if (tid < C) cluster_store(cluster_addr(shared_addr(&s_word[k][rank]), tid), w);
+        cluster_barrier();
+        return lane < C ? s_word[k][lane] : 0ull;
+    };
+    auto exchange0 = [&](unsigned long long w) { // (w: thread 0's)
+        if (tid == 0) s_sum = w;
+        __syncthreads();
+        return exchange(s_sum);
+    };
+    if (tid == 0) s_late = 0;
+    cluster_barrier(); // every block's state is in place
+    bool go = nacc != 0;
+    while (go) {
+        ++outer;
+        uint32_t *const val = SYNC ? x2 : (outer & 1) ? x1 : x0;
+        if (lead && (SYNC || !a.count_round1)) relax += a.m; // round 1 covers every row
+        uint32_t r = 0;
+        for (;;) {
+            ++r;
+            uint32_t *const inbox = (r & 1) ? x0 : x1; // what came in round r - 1 (synchronous)
+            const uint32_t to = shared_addr(SYNC ? ((r & 1) ? x1 : x0) : val);
+            const bool pushes = r <= a.max_inner; // (past the limit the last round's values are only taken)
+            bool any = false;
+            // did vertex i change in round r - 1 (round 1: is it accepting)?  o: what it offers then
+            auto changed = [&](uint32_t i, uint32_t &o) {
+                if (r == 1) {
+                    o = own[i];
+                    return o != 0;
+                }
+                if (SYNC) {
+                    const uint32_t y = inbox[i];
+                    if (!y) return false;
+                    inbox[i] = 0;
+                    if (r > 2) { // a frontier row of round r - 1
+                        const uint32_t v = i << cshift | rank;
+                        relax += whole ? __ldg(a.rowptr + v + 1) - __ldg(a.rowptr + v) : __ldg(row + v);
+                        ++frows;
+                    }
+                    o = max(y, own[i]);
+                    if (y <= val[i]) return false;
+                    val[i] = y;
+                    return true;
+                }
+                const uint32_t x = *(volatile uint32_t *)(val + i);
+                if (x <= x2[i]) return false;
+                x2[i] = x;
+                o = max(x, own[i]);
+                return true;
+            };
+            // offer o to the readers at rc[b, e); a long list is walked by the whole warp (all lanes call it)
+            auto send = [&](uint32_t o, uint32_t b, uint32_t e) {
+                if (!SYNC) {
+                    if (r > 1 || a.count_round1) relax += e - b;
+                    if (r > 1) frows += e != b;
+                }
+                for (unsigned m = __ballot_sync(0xFFFFFFFFu, e - b > TAIL_LONG); m; m &= m - 1) {
+                    const int src = __ffs(m) - 1;
+                    const uint32_t ob = __shfl_sync(0xFFFFFFFFu, o, src), bb = __shfl_sync(0xFFFFFFFFu, b, src),
+                                   ee = __shfl_sync(0xFFFFFFFFu, e, src);
+#pragma unroll 4
+                    for (uint32_t j = lane; j < ee - bb; j += 32) {
+                        const uint32_t w = __ldg(rc + bb + j);
+                        cluster_max(cluster_addr(to + 4 * (w >> cshift), w & cmask), ob);
+                    }
+                    if ((int)lane == src) b = e;
+                }
+                for (uint32_t j = 0; j < e - b; j += 4) { // up to four readers in flight
+                    uint32_t w[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) w[k] = j + k < e - b ? __ldg(rc + b + j + k) : NONE;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (w[k] != NONE) cluster_max(cluster_addr(to + 4 * (w[k] >> cshift), w[k] & cmask), o);
+                }
+            };
+            if (mine <= TT) { // a vertex per thread
+                uint32_t o = 0, b = 0, e = 0;
+                if (tid < mine && changed(tid, o)) {
+                    any = true;
+                    b = beg[tid];
+                    e = pushes ? end[tid] : b;
+                }
+                send(o, b, e);
+            } else { // several: the changed ones are queued first, so that their lists are read side by side
+                if (tid == 0) s_n = 0;
+                __syncthreads();
+                for (uint32_t i0 = 0; i0 < mine; i0 += TT) { // (block-uniform)
+                    const uint32_t i = i0 + tid;
+                    uint32_t o = 0;
+                    const bool hit = i < mine && changed(i, o);
+                    const unsigned m = __ballot_sync(0xFFFFFFFFu, hit);
+                    uint32_t at = 0;
+                    if (m && lane == 0) at = atomicAdd(&s_n, (uint32_t)__popc(m));
+                    at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(m & ((1u << lane) - 1u));
+                    if (hit) queue[at] = (uint16_t)i;
+                }
+                __syncthreads();
+                const uint32_t nq = s_n;
+                any = nq != 0;
+                for (uint32_t q0 = 0; pushes && q0 < nq; q0 += TT) { // (block-uniform)
+                    const uint32_t q = q0 + tid;
+                    uint32_t o = 0, b = 0, e = 0;
+                    if (q < nq) {
+                        const uint32_t i = queue[q];
+                        // (synchronous: the value just taken; asynchronous: the live one)
+                        o = r == 1 ? own[i] : max(*(volatile uint32_t *)(val + i), own[i]);
+                        b = beg[i];
+                        e = end[i];
+                    }
+                    send(o, b, e);
+                }
+            }
+            if (lead && (r & 7u) == 0 && (int64_t)(global_ns() - t0) > (int64_t)a.timeout_ns) any = s_late = 1;
+            any = __syncthreads_or(any);
+            const unsigned long long word = exchange((any ? 1ull : 0ull) | (s_late ? 2ull : 0ull));
+            const bool more = __any_sync(0xFFFFFFFFu, word & 1u), late = __any_sync(0xFFFFFFFFu, word & 2u);
+            if (r == 1) continue; // (the limit and the end of the rounds: once round 1's values are taken)
+            if (late) status = ST_TIMEOUT;
+            else if (more && !pushes) status = ST_LIMIT;
+            if (!more) break;
+            if (status != ST_OK) break;
+        }
+        const uint32_t rounds = status == ST_TIMEOUT ? r : r - 1;
+        inner_total += rounds;
+        if (lead) {
+            if (outer - 1 < a.hist_cap) a.hist[outer - 1] = rounds;
+            if (outer - 1 < RUN_HIST) a.res->hist[outer - 1] = rounds;
+            phase(ph_rounds);
+        }
+        if (status != ST_OK) break;
+        // ---- self-map test; the map values are marked at their owners (bit 31 of the own offer)
+        uint32_t wit = NONE, have = 0, settled = 0;
+        for (uint32_t i0 = 0; i0 < mine; i0 += TT) {
+            const uint32_t i = i0 + tid;
+            const uint32_t x = i < mine ? val[i] : 0u;
+            if (x) {
+                have = 1;
+                const uint32_t v = i << cshift | rank;
+                if (x - 1 == (whole ? v : __ldg(&meta[v].w))) wit = min(wit, x - 1);
+            }
+            const unsigned same = __match_any_sync(0xFFFFFFFFu, x); // (many vertices share a few values)
+            if (x && x != settled && lane == (unsigned)(__ffs(same) - 1)) {
+                const uint32_t u = whole ? x - 1 : __ldg(a.rank + x - 1) - 1;
+                cluster_or(cluster_addr(shared_addr(own) + 4 * (u >> cshift), u & cmask), 0x80000000u);
+            }
+            settled = x;
+        }
+        have = __syncthreads_or(have);
+        wit = __reduce_min_sync(0xFFFFFFFFu, wit);
+        if (lane == 0) s_min[warp] = wit;
+        __syncthreads();
+        if (tid == 0)
+            for (int w = 0; w < TT / 32; ++w) wit = min(wit, s_min[w]);
+        const unsigned long long seen = exchange0((unsigned long long)(NONE - wit) << 32 | have);
+        have = __any_sync(0xFFFFFFFFu, seen & 1u);
+        witness = NONE - __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(seen >> 32));
+        if (witness != NONE) verdict = 1;
+        if (verdict || !have) { // a cycle, or nothing reaches a remaining accepting vertex
+            if (lead) phase(ph_check);
+            break;
+        }
+        // ---- elimination
+        uint32_t elim = 0;
+        for (uint32_t i = tid; i < mine; i += TT)
+            if (own[i] >> 31) {
+                elim += (own[i] & 0x7FFFFFFFu) != 0;
+                own[i] = 0;
+            }
+        elim = __reduce_add_sync(0xFFFFFFFFu, elim);
+        if (lane == 0) s_min[warp] = elim;
+        __syncthreads();
+        if (tid == 0) {
+            elim = 0;
+            for (int w = 0; w < TT / 32; ++w) elim += s_min[w];
+        }
+        const bool late = lead && (int64_t)(global_ns() - t0) > (int64_t)a.timeout_ns;
+        const unsigned long long gone = exchange0((unsigned long long)elim | (late ? 1ull << 32 : 0ull));
+        nacc -= __reduce_add_sync(0xFFFFFFFFu, (uint32_t)gone);
+        if (nacc == 0) go = false;
+        else if ((a.max_outer && outer >= a.max_outer) || outer > a.nacc0) {
+            status = ST_LIMIT;
+            go = false;
+        } else if (__any_sync(0xFFFFFFFFu, (gone >> 32) != 0)) {
+            status = ST_TIMEOUT;
+            go = false;
+        }
+        if (lead) phase(ph_check);
+        if (go) // values back to none (asynchronous: the next iteration's pushes go to the other array)
+            for (uint32_t i = tid; i < mine; i += TT) {
+                val[i] = 0;
+                if (!SYNC) x2[i] = 0;
+            }
+    }
+    // ---- the map of the last iteration and the result
+    if (a.out) {
+        uint32_t *const val = SYNC ? x2 : (outer & 1) ? x1 : x0;
+        for (uint32_t i = tid; i < mine; i += TT) {
+            const uint32_t v = i << cshift | rank, x = val[i];
+            if (whole) a.out[v] = x - 1u; // (no value: MAP_NONE)
+            else if (x) a.out[__ldg(&meta[v].w)] = x - 1u;
+        }
+    }
+    unsigned long long sums[2];
+    for (int q = 0; q < 2; ++q) {
+        const unsigned long long s = warp_sum64(q ? frows : relax);
+        __syncthreads();
+        if (lane == 0) s_part[warp] = s;
+        __syncthreads();
+        unsigned long long t = 0;
+        if (tid == 0)
+            for (int w = 0; w < TT / 32; ++w) t += s_part[w];
+        sums[q] = warp_sum64(exchange0(t));
+    }
+    if (lead) {
+        RunRes *R = a.res;
+        R->verdict = verdict;
+        R->witness = witness;
+        R->outer = outer;
+        R->status = status;
+        R->gave_up = 0;
+        R->nacc = nacc;
+        if (!whole) { // and what k_run had counted
+            inner_total += c->inner_total;
+            sums[0] += c->relax.v;
+            sums[1] += c->frows.v;
+            ph_rounds += c->ph_rounds;
+            ph_check += c->ph_check;
+        }
+        R->inner_total = inner_total;
+        R->relax = sums[0];
+        R->frontier_rows = sums[1];
+        R->ph_rounds = ph_rounds;
+        R->ph_check = ph_check;
+    }
+    cluster_barrier(); // no block leaves while another may still write into its shared memory
+}
+
+} // namespace mapk

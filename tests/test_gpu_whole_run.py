@@ -1,0 +1,132 @@
+"""Whole runs in one launch (k_run over the grid, k_tail in one cluster) against the oracle, at the sizes where
+they change: a vertex more or less than a thread per vertex, a block, the cluster's capacity; compaction into a
+small and into a large graph; reader lists longer than a warp walks alone; limits; a map buffer of odd alignment.
+Integer work: everything must be equal."""
+import numpy as np
+import pytest
+
+import mapgen
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+CAP = 16 * 8704  # vertices the cluster holds
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import __graft_entry__
+
+    __graft_entry__.build()
+    import paper_0912_2555_gb300 as p
+
+    return p
+
+
+def compare(pkg, g, flags=0, want=None, runs=2):
+    want = want or oracle.run_graph(g)
+    h = pkg.map_create(g.n, g.rowptr, g.colidx if g.m else None, pkg.pack_bits(g.acc))
+    try:
+        for sched in (0, 1) * runs:
+            out = torch.full((g.n + 1,), 7, dtype=torch.int32, device="cuda")
+            r = pkg.map_run(h, sched=sched, flags=flags, map_out=out[1:])  # 4 bytes off a 16-byte boundary
+            assert (r.verdict, r.witness, r.outer) == (want.verdict, want.witness, want.outer), sched
+            assert np.array_equal(out[1:].cpu().numpy().view(np.uint32), want.map), sched
+            assert int(out[0]) == 7
+            if sched == 0:
+                assert (r.rounds, r.relaxations, r.inner_iters) == (want.rounds, want.relaxations, want.inner_total)
+            else:
+                assert all(a <= b for a, b in zip(r.rounds, want.rounds))
+    finally:
+        pkg.map_destroy(h)
+
+
+@pytest.mark.parametrize("n", [1, 31, 1023, 1024, 1025, 2049, 8704, 8705, 20000, CAP - 1, CAP, CAP + 1])
+def test_sizes_around_the_limits(pkg, n):
+    compare(pkg, mapgen.random_graph(n, 1, 6, 0.03, seed=n, variant="plain") if n > 31
+            else mapgen.tiny_graph(n, n, max_deg=3, acc_p=0.5), pkg.MAP_FLAG_FRONTIER_START)
+    if n > 1000:
+        compare(pkg, mapgen.layered_graph(n, max(8, n // 3000), seed=n))
+
+
+@pytest.mark.parametrize("n,layers,plant", [(400_003, 24, False), (400_003, 24, True), (3_000_001, 180, False),
+                                            (CAP * 16, 40, False)])
+def test_compaction(pkg, n, layers, plant):
+    """Later iterations in the compact graph: in the cluster, or over the grid first (16 % accepting)."""
+    compare(pkg, mapgen.layered_graph(n, layers, seed=11, plant=plant, acc_p=0.16 if layers == 40 else 0.01),
+            pkg.MAP_FLAG_FRONTIER_START)
+
+
+@pytest.mark.parametrize("n", [5000, 30_000, CAP + 1000, 700_000])
+def test_hubs(pkg, n):
+    """Vertices read by thousands of rows beside vertices nobody reads, a chain of values through them."""
+    rng = np.random.default_rng(n)
+    hubs = rng.choice(n, 3, replace=False)
+    deg = rng.integers(0, 3, n)
+    rowptr = np.zeros(n + 1, np.uint32)
+    np.cumsum(deg, out=rowptr[1:])
+    col = rng.integers(0, n, int(rowptr[-1])).astype(np.uint32)
+    at = rng.random(col.size) < 0.4
+    col[at] = rng.choice(hubs, int(at.sum()))
+    acc = (rng.random(n) < 0.02).astype(np.uint8)
+    acc[hubs[0]] = 1
+    compare(pkg, mapgen.Graph(n, rowptr, col, acc, (0,) * 8, f"hubs-{n}", {}), pkg.MAP_FLAG_FRONTIER_START)
+
+
+@pytest.mark.parametrize("n,layers", [(3000, 8), (60_000, 30), (500_000, 30)])
+def test_limits_and_what_follows(pkg, n, layers):
+    """A run stopped by a limit reports the limit, and the next run on the handle is the oracle's."""
+    g = mapgen.layered_graph(n, layers, seed=5)
+    want = oracle.run_graph(g)
+    assert want.outer > 3 and want.rounds[0] > 3
+    h = pkg.map_create(g.n, g.rowptr, g.colidx, pkg.pack_bits(g.acc))
+    try:
+        for sched in (0, 1):
+            for kw in (dict(max_outer=1), dict(max_outer=3), dict(max_inner=1), dict(max_inner=2)):
+                r = pkg.map_run(h, sched=sched, flags=pkg.MAP_FLAG_FRONTIER_START, allow_limit=True, **kw)
+                assert r.status == pkg.MAP_ERR_LIMIT
+                assert r.outer == kw.get("max_outer", 1)
+                if "max_inner" in kw:
+                    assert r.rounds[0] == kw["max_inner"]
+                out = np.empty(g.n, np.uint32)
+                r = pkg.map_run(h, sched=sched, map_out=out)
+                assert (r.verdict, r.witness, r.outer) == (want.verdict, want.witness, want.outer)
+                assert np.array_equal(out, want.map)
+                if sched == 0:
+                    assert (r.rounds, r.relaxations) == (want.rounds, want.relaxations)
+    finally:
+        pkg.map_destroy(h)
+    # the map of a limited synchronous run is the oracle's of that iteration
+    lim = oracle.run_graph(g, max_outer=2)
+    h = pkg.map_create(g.n, g.rowptr, g.colidx, pkg.pack_bits(g.acc))
+    try:
+        out = np.empty(g.n, np.uint32)
+        pkg.map_run(h, max_outer=2, flags=pkg.MAP_FLAG_FRONTIER_START, map_out=out, allow_limit=True)
+        assert np.array_equal(out, lim.map)
+    finally:
+        pkg.map_destroy(h)
+
+
+def test_batch_with_compaction(pkg):
+    """Graphs that end in different iterations: floods (planted cycles) beside long eliminations."""
+    gs = [mapgen.layered_graph(n, max(8, n // 5000), seed=n, plant=bool(i % 3 == 0))
+          for i, n in enumerate([1500, 40_000, 200_000, 7001, 90_000, 300_001])]
+    gs += [mapgen.tiny_graph(9, 60, max_deg=3, acc_p=0.3), mapgen.from_lists([[1], [0], []], [0, 0, 0])]
+    h = pkg.map_batch_create([(g.n, g.rowptr, g.colidx, pkg.pack_bits(g.acc)) for g in gs])
+    try:
+        for sched in (0, 1):
+            out = np.empty(sum(g.n for g in gs), np.uint32)
+            rs = pkg.map_batch_run(h, len(gs), sched=sched, flags=pkg.MAP_FLAG_FRONTIER_START, map_out=out)
+            off = 0
+            for g, r in zip(gs, rs):
+                want = oracle.run_graph(g)
+                assert (r.verdict, r.witness, r.outer, r.accepting_left >= 0) == (want.verdict, want.witness, want.outer, True)
+                assert np.array_equal(out[off:off + g.n], want.map)
+                if sched == 0:
+                    assert (r.rounds, r.relaxations) == (want.rounds, want.relaxations)
+                off += g.n
+    finally:
+        pkg.map_destroy(h)
