@@ -444,16 +444,16 @@ MAP_API int map_graph_info(const map_graph *g, uint32_t *n, uint64_t *m);
  *   n <= MAP_STATIC_MAX_N vertices and m = rowptr[n] <= MAP_STATIC_MAX_M edges;
  *   larger graphs are rejected with MAP_ERR_ARG and a message naming the limit.
  *   rowptr, colidx, acc_bits, map_out: as for map_create / map_run, host or
- *   device memory; the inputs are copied into the array on every call.
+ *   device memory; host inputs are copied into the array on every call, device
+ *   inputs are read where they are (until the call returns).
  *   opts: as for map_run (schedules, limits, timeout_ms, rounds_out for every
  *   outer iteration, MAP_FLAG_EARLY_EXIT, MAP_FLAG_DENSE_START), except that
  *   traces, MAP_FLAG_PROFILE, MAP_FLAG_FRONTIER_START and repeat are refused
  *   (MAP_ERR_ARG); res: as for map_run, status included (device_ms stays 0).
  *   cuda_stream: the stream all work is issued on.
- * The call blocks: it waits for cuda_stream several times (it reads rowptr[0]
- * and rowptr[n], then the control block after every step of the loop, into
- * host memory), so it must not be issued on a stream that is being captured
- * into a CUDA graph.  The first call on a device also looks the array's device
+ * The call blocks: it waits for cuda_stream once, for the result (with
+ * MAP_FLAG_EARLY_EXIT or MAP_FLAG_DENSE_START after every step of the loop), so
+ * it must not be issued on a stream that is being captured into a CUDA graph.  The first call on a device also looks the array's device
  * address up (cudaGetSymbolAddress) with that device current; make that first
  * call before any stream capture begins in the process.  Every call on a
  * device shares the one array and overwrites what the previous call left

@@ -234,7 +234,7 @@ int tail_blocks()
     if (const int k = known[dev].load()) return k - 1;
     int best = 0;
     const void *const both[] = {(const void *)mapk::k_tail<true>, (const void *)mapk::k_tail<false>};
-    bool ok = true;
+    bool ok = cudaFuncSetAttribute(mapk::k_prepare, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
     for (const void *f : both)
         ok = ok && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mapk::TAIL_SMEM) == cudaSuccess &&
              cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
@@ -914,6 +914,66 @@ static bool runs_in_tail(const map_graph *g) { return !g->comp && g->n <= tail_b
 // fit into one cluster always gain (16,384 vertices 0.12 against 0.44 ms).
 static bool default_fstart(const map_graph *g) { return runs_in_tail(g) || g->acc_entries <= g->m / 16; }
 
+// a launch of `blocks` blocks of TT threads as one cluster
+static void cluster_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &attr, uint32_t blocks, size_t smem, cudaStream_t s)
+{
+    cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(mapk::TT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = blocks;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+}
+
+// blocks of k_tail for a whole graph of n vertices: one vertex per thread as far as the cluster goes (random
+// graphs, synchronous, us per run with 1 / 2 / 4 / 8 / 16 blocks: 4,000 vertices 131 / 115 / 88 / 92 / 104,
+// 8,000 vertices 223 / 178 / 152 / 124 / 132, 16,384 vertices - / 231 / 180 / 160 / 141)
+static uint32_t tail_blocks_for(uint32_t n, int cluster)
+{
+    uint32_t blocks = 1;
+    while ((int)blocks < cluster && n > blocks * (uint32_t)mapk::TT) blocks *= 2;
+    return blocks;
+}
+
+static int launch_tail(const mapk::RunArgs &a, bool sync_sched, bool whole, uint32_t blocks, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    cluster_config(cfg, attr, blocks, mapk::TAIL_SMEM, s);
+    if (sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_tail<true>, a, whole ? 1u : 0u));
+    else CK(cudaLaunchKernelEx(&cfg, mapk::k_tail<false>, a, whole ? 1u : 0u));
+    return MAP_OK;
+}
+
+// the result of a whole run as its kernel left it (hist: rounds of every iteration, on the device)
+static int take_result(const mapk::RunRes &R, const map_opts &opts, uint64_t m, bool sync_sched, const uint32_t *hist,
+                       uint32_t hist_cap, cudaStream_t s, map_result *res)
+{
+    res->verdict = R.verdict ? MAP_CYCLE : MAP_NO_CYCLE;
+    res->witness = R.verdict ? R.witness : MAP_NONE;
+    res->outer_iters = R.outer;
+    res->inner_canonical = sync_sched ? 1 : 0;
+    res->inner_iters = R.inner_total;
+    res->relaxations = R.relax;
+    res->edges_total = m * (uint64_t)R.outer;
+    res->frontier_rows = R.frontier_rows;
+    res->accepting_left = R.nacc;
+    const uint32_t nh = std::min(std::min<uint32_t>(R.outer, hist_cap), opts.rounds_cap);
+    if (opts.rounds_out && nh) {
+        memcpy(opts.rounds_out, R.hist, (size_t)std::min(nh, mapk::RUN_HIST) * 4);
+        if (nh > mapk::RUN_HIST) { // the rest stayed on the device
+            CK(cudaMemcpyAsync(opts.rounds_out + mapk::RUN_HIST, hist + mapk::RUN_HIST,
+                               (size_t)(nh - mapk::RUN_HIST) * 4, cudaMemcpyDeviceToHost, s));
+            CK(cudaStreamSynchronize(s));
+        }
+    }
+    return MAP_OK;
+}
+
 // Queue one whole run as a single launch (k_run) and fill in the result from where the kernel left it.
 static int launch_run(map_graph *g, cudaStream_t s, const map_opts &opts, const Ctl &init, bool count_round1,
                       uint32_t *out)
@@ -958,27 +1018,7 @@ static int launch_run(map_graph *g, cudaStream_t s, const map_opts &opts, const 
     const bool sync_sched = opts.sched == MAP_SCHED_SYNC;
     const int cluster = g->comp ? 0 : tail_blocks();
     const bool whole = runs_in_tail(g);
-    const auto launch_tail = [&](uint32_t blocks) -> int {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(blocks);
-        cfg.blockDim = dim3(mapk::TT);
-        cfg.dynamicSmemBytes = mapk::TAIL_SMEM;
-        cfg.stream = s;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = blocks;
-        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        if (sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_tail<true>, a, whole ? 1u : 0u));
-        else CK(cudaLaunchKernelEx(&cfg, mapk::k_tail<false>, a, whole ? 1u : 0u));
-        return MAP_OK;
-    };
-    if (whole) {
-        uint32_t blocks = 1;
-        while ((int)blocks < cluster && g->n > blocks * 1024u) blocks *= 2;
-        return launch_tail(blocks);
-    }
+    if (whole) return launch_tail(a, sync_sched, true, tail_blocks_for(g->n, cluster), s);
     a.tail_cap = (uint32_t)cluster * mapk::TAIL_N;
     CK(cudaMemsetAsync(g->run_ctl, 0, sizeof(mapk::RunCtl), s));
     if (g->comp) {
@@ -999,7 +1039,7 @@ static int launch_run(map_graph *g, cudaStream_t s, const map_opts &opts, const 
     else if (g->comp) CK(cudaLaunchKernelEx(&cfg, mapk::k_run<false, true>, a));
     else if (sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_run<true, false>, a));
     else CK(cudaLaunchKernelEx(&cfg, mapk::k_run<false, false>, a));
-    return cluster ? launch_tail((uint32_t)cluster) : MAP_OK;
+    return cluster ? launch_tail(a, sync_sched, false, (uint32_t)cluster, s) : MAP_OK;
 }
 
 static int run_impl(map_graph *g, const map_opts *opts_in, map_result *res, uint32_t *map_out,
@@ -1110,28 +1150,11 @@ static int run_impl(map_graph *g, const map_opts *opts_in, map_result *res, uint
         CK(cudaStreamSynchronize(s));
         float ms = 0.f;
         CK(cudaEventElapsedTime(&ms, g->ev[0], g->ev[1]));
-        res->verdict = R->verdict ? MAP_CYCLE : MAP_NO_CYCLE;
-        res->witness = R->verdict ? R->witness : MAP_NONE;
-        res->outer_iters = R->outer;
-        res->inner_canonical = sync_sched ? 1 : 0;
-        res->inner_iters = R->inner_total;
-        res->relaxations = R->relax;
-        res->edges_total = g->m * (uint64_t)R->outer;
+        if ((rc = take_result(*R, opts, g->m, sync_sched, g->hist, g->hist_cap, s, res))) return rc;
         res->device_ms = ms;
         res->round_ms = R->ph_rounds * 1e-6;
         res->check_ms = R->ph_check * 1e-6;
-        res->frontier_rows = R->frontier_rows;
-        res->accepting_left = R->nacc;
         res->launches = g->comp || runs_in_tail(g) || !tail_blocks() ? 1 : 2;
-        const uint32_t nh = std::min(std::min<uint32_t>(R->outer, g->hist_cap), opts.rounds_cap);
-        if (opts.rounds_out && nh) {
-            memcpy(opts.rounds_out, R->hist, (size_t)std::min(nh, mapk::RUN_HIST) * 4);
-            if (nh > mapk::RUN_HIST) { // the rest stayed on the device
-                CK(cudaMemcpyAsync(opts.rounds_out + mapk::RUN_HIST, g->hist + mapk::RUN_HIST,
-                                   (size_t)(nh - mapk::RUN_HIST) * 4, cudaMemcpyDeviceToHost, s));
-                CK(cudaStreamSynchronize(s));
-            }
-        }
         g->dirty = R->gave_up != 0; // (a run stopped by a limit has put its state back)
         if (R->status == mapk::ST_LIMIT) return fail(MAP_ERR_LIMIT, "map_run: max_outer or max_inner reached");
         if (R->gave_up) return fail(MAP_ERR_TIMEOUT, "map_run: a bounded device wait (grid barrier) gave up after seconds without progress");
@@ -1903,9 +1926,10 @@ int map_batch_run(map_graph *g, const map_opts *opts, map_result *results, uint3
 // all of its work space in the file-scope device array below, which every GPU
 // that loads this library holds until the process exits, and it calls no
 // cudaMalloc, cudaFree or allocating routine.  It runs the same kernels as
-// map_run, stepped from the host: it waits for its stream several times per
-// call (to read the CSR's end offsets and the control block between steps), so
-// it blocks, and it cannot be issued on a stream that is being captured.
+// map_run: set-up and run are one launch each in one thread-block cluster, and the
+// call waits for its stream once (an early exit or the dense start: stepped from the
+// host, with several waits).  So it blocks, and it cannot be issued on a stream that
+// is being captured.
 // ============================================================================
 
 namespace {
@@ -1989,6 +2013,90 @@ int static_read_ctl(Ctl *h, const Ctl *d, cudaStream_t s)
 
 } // namespace
 
+// what run_static_impl reports for a CSR that map_run_static does not take (k_prepare's codes)
+static int static_refused(uint32_t code, uint32_t r0, uint64_t m)
+{
+    if (code == 1) return fail(MAP_ERR_CSR, "map_run_static: rowptr[0] = %u, expected 0", r0);
+    if (code == 2)
+        return fail(MAP_ERR_ARG, "map_run_static: m = %llu edges exceeds %llu (MAP_STATIC_MAX_M); use map_create/map_run",
+                    (unsigned long long)m, (unsigned long long)ST_MAX_M);
+    return fail(MAP_ERR_CSR, "map_run_static: invalid CSR (decreasing rowptr or colidx >= n)");
+}
+
+static int run_static_cluster(uint32_t n, const uint32_t *rowptr, const uint32_t *colidx, const uint32_t *acc_bits,
+                              const map_opts &opts, uint32_t *base, map_result *res, uint32_t *map_out, cudaStream_t s)
+{
+    const bool sync_sched = opts.sched == MAP_SCHED_SYNC;
+    const size_t W = (n + 31) / 32;
+    // arrays in device memory are read where they are; the others are copied into the scratch
+    if (!is_device_ptr(rowptr)) {
+        CK(cudaStreamSynchronize(s)); // (work queued before this call may still be writing page-locked arrays)
+        const uint32_t r0 = rowptr[0], m = rowptr[n];
+        if (r0 != 0 || m > ST_MAX_M) return static_refused(r0 != 0 ? 1 : 2, r0, m);
+        CK(cudaMemcpyAsync(base + ST_ROWPTR, rowptr, ((size_t)n + 1) * 4, cudaMemcpyHostToDevice, s));
+        if (!is_device_ptr(colidx)) {
+            if (m) CK(cudaMemcpyAsync(base + ST_COLIDX, colidx, (size_t)m * 4, cudaMemcpyHostToDevice, s));
+            colidx = base + ST_COLIDX;
+        }
+        rowptr = base + ST_ROWPTR;
+    } else if (!is_device_ptr(colidx)) { // its length is on the device
+        uint32_t ends[2];
+        CK(cudaMemcpyAsync(&ends[0], rowptr, 4, cudaMemcpyDeviceToHost, s));
+        CK(cudaMemcpyAsync(&ends[1], rowptr + n, 4, cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+        if (ends[0] != 0 || ends[1] > ST_MAX_M) return static_refused(ends[0] != 0 ? 1 : 2, ends[0], ends[1]);
+        if (ends[1]) CK(cudaMemcpyAsync(base + ST_COLIDX, colidx, (size_t)ends[1] * 4, cudaMemcpyHostToDevice, s));
+        colidx = base + ST_COLIDX;
+    }
+    if (!is_device_ptr(acc_bits)) {
+        CK(cudaMemcpyAsync(base + ST_ACC, acc_bits, W * 4, cudaMemcpyHostToDevice, s));
+        acc_bits = base + ST_ACC;
+    }
+    struct Back { // what comes back: k_prepare's verdict and the run's result
+        uint32_t prep[4];
+        mapk::RunRes res;
+    };
+    Back *const dev = reinterpret_cast<Back *>(base + ST_LIST);
+    const bool out_dev = map_out && is_device_ptr(map_out);
+    mapk::RunArgs a;
+    memset(&a, 0, sizeof a);
+    a.n = n;
+    a.words = (uint32_t)W;
+    a.rowptr = rowptr;
+    a.rrowptr = base + ST_RROWPTR;
+    a.rcol = base + ST_RCOL;
+    a.acc0 = base + ST_ACC0;
+    a.res = &dev->res;
+    a.hist = base + ST_HISTW;
+    a.hist_cap = (uint32_t)ST_HIST;
+    a.out = !map_out ? nullptr : out_dev ? map_out : base + ST_XBUF;
+    a.max_outer = opts.max_outer;
+    a.max_inner = opts.max_inner ? opts.max_inner : n + 1;
+    a.timeout_ns = (uint64_t)(opts.timeout_ms ? opts.timeout_ms : 120000u) * 1000000ull;
+    a.prep = dev->prep;
+    const int cluster = tail_blocks();
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    cluster_config(cfg, attr, tail_blocks_for(n, cluster), 0, s);
+    CK(cudaLaunchKernelEx(&cfg, mapk::k_prepare, n, rowptr, colidx, acc_bits, (uint32_t)ST_MAX_M, base + ST_ACC0,
+                          base + ST_RROWPTR, base + ST_RCOL, base + ST_RPOS, dev->prep));
+    int rc = launch_tail(a, sync_sched, true, tail_blocks_for(n, cluster), s);
+    if (rc) return rc;
+    Back h;
+    CK(cudaMemcpyAsync(&h, dev, sizeof h, cudaMemcpyDeviceToHost, s));
+    if (map_out && !out_dev) { // (into the caller's buffer only once the graph is known to be good)
+        CK(cudaStreamSynchronize(s));
+        if (!h.prep[0]) CK(cudaMemcpyAsync(map_out, base + ST_XBUF, (size_t)n * 4, cudaMemcpyDefault, s));
+    }
+    CK(cudaStreamSynchronize(s));
+    if (h.prep[0]) return static_refused(h.prep[0], h.prep[3], h.prep[2]);
+    if ((rc = take_result(h.res, opts, h.prep[2], sync_sched, base + ST_HISTW, (uint32_t)ST_HIST, s, res))) return rc;
+    res->launches = 2;
+    if (h.res.status == mapk::ST_LIMIT) return fail(MAP_ERR_LIMIT, "map_run_static: max_outer or max_inner reached");
+    if (h.res.status == mapk::ST_TIMEOUT) return fail(MAP_ERR_TIMEOUT, "map_run_static: stopped after the timeout");
+    return MAP_OK;
+}
+
 static int run_static_impl(uint32_t n, const uint32_t *rowptr, const uint32_t *colidx, const uint32_t *acc_bits,
                            const map_opts *opts_in, map_result *res, uint32_t *map_out, void *cuda_stream)
 {
@@ -2010,6 +2118,9 @@ static int run_static_impl(uint32_t n, const uint32_t *rowptr, const uint32_t *c
     uint32_t *base = nullptr;
     int rc = static_scratch(&base);
     if (rc) return rc;
+    // in one cluster: set-up, run and result with one wait (an early exit and the dense round keep the steps below)
+    if (!(opts.flags & (MAP_FLAG_EARLY_EXIT | MAP_FLAG_DENSE_START)) && colidx && n <= tail_blocks() * mapk::TAIL_N)
+        return run_static_cluster(n, rowptr, colidx, acc_bits, opts, base, res, map_out, s);
     // m = rowptr[n], from host or device memory
     uint32_t m32 = 0, r0 = 0;
     CK(cudaMemcpyAsync(&m32, rowptr + n, 4, cudaMemcpyDefault, s));

@@ -92,6 +92,7 @@ struct RunArgs {
     uint32_t nacc0, max_outer, max_inner, lc_passes;
     uint32_t count_round1;       // asynchronous relaxations: the pushes of round 1 (else m per iteration)
     uint64_t timeout_ns;
+    const uint32_t *prep;        // not NULL: (error, accepting vertices, entries) that k_prepare found
     uint32_t tail_cap;           // compact graphs of at most this many vertices are left to k_tail (0: none)
     // batched runs
     const uint32_t *comp;
@@ -852,6 +853,9 @@ __global__ void __launch_bounds__(TT, 1) k_tail(const __grid_constant__ RunArgs 
     __shared__ uint32_t s_min[TT / 32], s_n, s_late;
     RunCtl *c = a.ctl;
     if (!whole && !*(volatile uint32_t *)&c->hand) return; // k_run finished the run (every block returns)
+    if (a.prep && a.prep[0]) return;                        // k_prepare refused the graph
+    const uint32_t nacc0 = a.prep ? a.prep[1] : a.nacc0;
+    const uint64_t m = a.prep ? a.prep[2] : a.m;
     const uint32_t C = gridDim.x, rank = cluster_rank(), cshift = __ffs(C) - 1, cmask = C - 1;
     const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     const uint32_t V = whole ? a.n : *(volatile uint32_t *)&c->V;
@@ -889,7 +893,7 @@ __global__ void __launch_bounds__(TT, 1) k_tail(const __grid_constant__ RunArgs 
             mark = now;
         }
     };
-    uint32_t outer = whole ? 0u : *(volatile uint32_t *)&c->outer, nacc = whole ? a.nacc0 : *(volatile uint32_t *)&c->nacc;
+    uint32_t outer = whole ? 0u : *(volatile uint32_t *)&c->outer, nacc = whole ? nacc0 : *(volatile uint32_t *)&c->nacc;
     uint32_t status = ST_OK, verdict = 0, witness = NONE, seq = 0;
     unsigned long long relax = 0, frows = 0, inner_total = 0;
     // every block's word (the same in its threads 0 .. C - 1) to every block, then the cluster barrier; the
@@ -912,7 +916,7 @@ __global__ void __launch_bounds__(TT, 1) k_tail(const __grid_constant__ RunArgs 
     while (go) {
         ++outer;
         uint32_t *const val = SYNC ? x2 : (outer & 1) ? x1 : x0;
-        if (lead && (SYNC || !a.count_round1)) relax += a.m; // round 1 covers every row
+        if (lead && (SYNC || !a.count_round1)) relax += m; // round 1 covers every row
         uint32_t r = 0;
         for (;;) {
             ++r;
@@ -1076,7 +1080,7 @@ __global__ void __launch_bounds__(TT, 1) k_tail(const __grid_constant__ RunArgs 
         const unsigned long long gone = exchange0((unsigned long long)elim | (late ? 1ull << 32 : 0ull));
         nacc -= __reduce_add_sync(0xFFFFFFFFu, (uint32_t)gone);
         if (nacc == 0) go = false;
-        else if ((a.max_outer && outer >= a.max_outer) || outer > a.nacc0) {
+        else if ((a.max_outer && outer >= a.max_outer) || outer > nacc0) {
             status = ST_LIMIT;
             go = false;
         } else if (__any_sync(0xFFFFFFFFu, (gone >> 32) != 0)) {
@@ -1132,6 +1136,110 @@ __global__ void __launch_bounds__(TT, 1) k_tail(const __grid_constant__ RunArgs 
         R->ph_check = ph_check;
     }
     cluster_barrier(); // no block leaves while another may still write into its shared memory
+}
+
+// Set-up of a small graph in one cluster (before k_tail): bounds and validity of the CSR, the accepting set
+// and its size, and the readers (reverse CSR).  Entry i holding u goes to slot start(u) + the count its
+// increment of u's in-degree returned; the row of an entry is found by binary search, so that a row of any
+// length is spread over all threads.  Replaces eight launches, five memsets and two stream waits: at 1,000
+// vertices they were most of map_run_static's 480 us.
+// prep: (0 = good, 1 = rowptr[0] != 0, 2 = more than max_m entries, 3 = invalid), accepting vertices, entries,
+// rowptr[0]; rank: m words; cnt: n + 1 words, becomes rrowptr.
+__global__ void __launch_bounds__(TT, 1)
+    k_prepare(uint32_t n, const uint32_t *rowptr, const uint32_t *colidx, const uint32_t *acc_in, uint32_t max_m,
+              uint32_t *acc0, uint32_t *cnt, uint32_t *rcol, uint32_t *rank, uint32_t *prep)
+{
+    __shared__ uint32_t s_warp[TT / 32], s_part[TAIL_C], s_bad, s_acc;
+    const uint32_t C = gridDim.x, me = cluster_rank(), tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+    const uint32_t gid = me * TT + tid, threads = C * TT;
+    const uint32_t r0 = __ldg(rowptr), m = __ldg(rowptr + n);
+    if (r0 != 0 || m > max_m) { // (every block)
+        if (gid == 0) {
+            prep[0] = r0 != 0 ? 1u : 2u;
+            prep[1] = 0;
+            prep[2] = m;
+            prep[3] = r0;
+        }
+        return;
+    }
+    if (tid == 0) s_bad = s_acc = 0;
+    cluster_barrier();
+    uint32_t bad = 0, na = 0;
+    for (uint32_t i = gid; i <= n; i += threads) cnt[i] = 0;
+    for (uint32_t i = gid; i < n; i += threads) bad |= __ldg(rowptr + i) > __ldg(rowptr + i + 1);
+    const uint32_t words = (n + 31) / 32;
+    for (uint32_t i = gid; i < words; i += threads) {
+        uint32_t x = __ldg(acc_in + i);
+        if (i == words - 1 && (n & 31u)) x &= (1u << (n & 31u)) - 1u;
+        acc0[i] = x;
+        na += __popc(x);
+    }
+    cluster_barrier(); // the counts are zero
+    for (uint32_t i = gid; i < m; i += threads) {
+        const uint32_t u = __ldg(colidx + i);
+        if (u >= n) bad = 1;
+        else rank[i] = atomicAdd(cnt + u + 1, 1u);
+    }
+    // verdict on the input, and the accepting vertices, to block 0
+    bad = __any_sync(0xFFFFFFFFu, bad);
+    na = __reduce_add_sync(0xFFFFFFFFu, na);
+    if (lane == 0) {
+        if (bad) cluster_or(cluster_addr(shared_addr(&s_bad), 0), 1u);
+        if (na)
+            asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(cluster_addr(shared_addr(&s_acc), 0)),
+                         "r"(na)
+                         : "memory");
+    }
+    cluster_barrier(); // the counts are complete
+    // inclusive scan of cnt[0 .. n]: a contiguous share per block
+    const uint32_t len = n + 1, share = (len + C - 1) / C, b = min(len, me * share), e = min(len, b + share);
+    uint32_t sum = 0;
+    for (uint32_t i = b + tid; i < e; i += TT) sum += __ldcg(cnt + i);
+    sum = __reduce_add_sync(0xFFFFFFFFu, sum);
+    if (lane == 0) s_warp[warp] = sum;
+    __syncthreads();
+    if (tid < 32) {
+        const uint32_t t = __reduce_add_sync(0xFFFFFFFFu, s_warp[tid]);
+        if (tid < C)
+            asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(shared_addr(&s_part[me]), tid)),
+                         "r"(t)
+                         : "memory");
+    }
+    cluster_barrier();
+    uint32_t run = 0;
+    for (uint32_t q = 0; q < me; ++q) run += s_part[q];
+    for (uint32_t i0 = b; i0 < e; i0 += TT) { // (block-uniform)
+        const uint32_t i = i0 + tid;
+        uint32_t x = warp_inclusive_scan(i < e ? __ldcg(cnt + i) : 0u);
+        __syncthreads(); // s_warp is free
+        if (lane == 31) s_warp[warp] = x;
+        __syncthreads();
+        if (warp == 0) {
+            const uint32_t w = s_warp[lane], incl = warp_inclusive_scan(w);
+            s_warp[lane] = incl;
+        }
+        __syncthreads();
+        if (warp) x += s_warp[warp - 1];
+        if (i < e) cnt[i] = run + x;
+        run += s_warp[TT / 32 - 1];
+    }
+    if (gid == 0) {
+        prep[0] = s_bad ? 3u : 0u;
+        prep[1] = s_acc;
+        prep[2] = m;
+        prep[3] = 0;
+    }
+    cluster_barrier(); // the starts are in place, and the verdict
+    if (*(volatile uint32_t *)prep) return;
+    for (uint32_t i = gid; i < m; i += threads) {
+        uint32_t lo = 0, hi = n; // rowptr[lo] <= i < rowptr[hi]
+        while (hi - lo > 1) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if (__ldg(rowptr + mid) <= i) lo = mid;
+            else hi = mid;
+        }
+        rcol[__ldcg(cnt + __ldg(colidx + i)) + rank[i]] = lo;
+    }
 }
 
 } // namespace mapk

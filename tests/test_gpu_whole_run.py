@@ -130,3 +130,45 @@ def test_batch_with_compaction(pkg):
                 off += g.n
     finally:
         pkg.map_destroy(h)
+
+
+def _dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a, dtype=np.uint32).view(np.int32)).cuda()
+
+
+@pytest.mark.parametrize("n", [1, 33, 1025, 16385, 65536])
+@pytest.mark.parametrize("where", ["device", "host", "rows-host", "entries-host"])
+def test_static_set_up(pkg, n, where):
+    """map_run_static's set-up in one cluster: readers of a graph with one long row, empty rows and a hub, from
+    arrays in either memory, against the oracle."""
+    rng = np.random.default_rng(n)
+    deg = rng.integers(0, 4, n)
+    deg[n // 2] = min(20 * n, 200_000)
+    rowptr = np.zeros(n + 1, np.uint32)
+    np.cumsum(deg, out=rowptr[1:])
+    col = rng.integers(0, n, int(rowptr[-1])).astype(np.uint32)
+    col[rng.random(col.size) < 0.2] = n - 1
+    g = mapgen.Graph(n, rowptr, col, (rng.random(n) < 0.05).astype(np.uint8), (0,) * 8, "static", {})
+    want = oracle.run_graph(g)
+    rp = rowptr if where in ("host", "rows-host") else _dev(rowptr)
+    ci = col if where in ("host", "entries-host") else _dev(col)
+    ab = pkg.pack_bits(g.acc) if where == "host" else _dev(pkg.pack_bits(g.acc))
+    for sched in (0, 1):
+        out = np.empty(n, np.uint32)
+        r = pkg.map_run_static(n, rp, ci, ab, sched=sched, map_out=out)
+        assert (r.verdict, r.witness, r.outer, r.edges_total) == (want.verdict, want.witness, want.outer, g.m * want.outer)
+        assert np.array_equal(out, want.map)
+        if sched == 0:
+            assert (r.rounds, r.relaxations) == (want.rounds, want.relaxations)
+
+
+@pytest.mark.parametrize("rowptr,col,code", [([0, 2, 1], [0, 1], "CSR"), ([0, 1, 2], [0, 2], "CSR"), ([1, 1, 2], [0, 1], "CSR"),
+                                             ([0, 1, 600_000], [0, 1], "ARG")])
+@pytest.mark.parametrize("on_device", [False, True])
+def test_static_refuses_what_it_refused(pkg, rowptr, col, code, on_device):
+    to = _dev if on_device else (lambda a: np.array(a, np.uint32))
+    out = np.full(2, 9, np.uint32)
+    with pytest.raises(pkg.MapError) as e:
+        pkg.map_run_static(2, to(rowptr), to(col), to([1]), map_out=out)
+    assert e.value.code == getattr(pkg, f"MAP_ERR_{code}")
+    assert out.tolist() == [9, 9]
