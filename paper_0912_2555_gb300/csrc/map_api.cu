@@ -264,6 +264,28 @@ int tail_blocks()
     return best;
 }
 
+// whether k_own's blocks fit on the current device (one per SM, a cooperative launch).  Asked once per device.
+bool own_fits()
+{
+    constexpr int DEVICES = 64;
+    static std::atomic<int> known[DEVICES]; // 1 + answer
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= DEVICES) {
+        cudaGetLastError();
+        return false;
+    }
+    if (const int k = known[dev].load()) return k == 2;
+    bool ok = true;
+    for (const void *f : {(const void *)mapk::k_own<true>, (const void *)mapk::k_own<false>}) {
+        int o = 0;
+        ok = ok && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mapk::OWN_SMEM) == cudaSuccess &&
+             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, f, mapk::TT, mapk::OWN_SMEM) == cudaSuccess && o >= 1;
+    }
+    cudaGetLastError();
+    known[dev].store(ok ? 2 : 1);
+    return ok;
+}
+
 int pull_occupancy()
 {
     int occ = 1 << 30, o = 0;
@@ -296,6 +318,7 @@ struct map_graph {
     uint32_t words = 0;
     int G = 4;
     int sms = 0;
+    int sm_share = 0;    // SMs a run may fill (served jobs: an even share; 0: all)
     int dense_grid = 0;  // blocks of the dense-round kernel
     int rounds_grid = 0; // blocks of the cooperative fix-point kernel (all resident)
     int check_grid = 0;  // blocks of the self-map / elimination kernel
@@ -905,14 +928,24 @@ int map_destroy(map_graph *g)
 }
 
 // single graphs small enough for one cluster (k_tail): the whole run in one launch of it
-static bool runs_in_tail(const map_graph *g) { return !g->comp && g->n <= tail_blocks() * mapk::TAIL_N; }
+static uint32_t tail_cap()
+{
+    const uint32_t room = (uint32_t)tail_blocks() * mapk::TAIL_N;
+    return own_fits() ? std::min(room, mapk::TAIL_BEST) : room;
+}
+static bool runs_in_tail(const map_graph *g) { return !g->comp && g->n <= tail_cap(); }
+
+// single graphs that fit into the shared memory of the SMs a run may fill (k_own)
+static uint32_t own_blocks(const map_graph *g) { return g->comp || !own_fits() ? 0u : (uint32_t)(g->sm_share ? g->sm_share : g->sms); }
+static bool runs_in_own(const map_graph *g) { return !runs_in_tail(g) && g->n <= (uint64_t)own_blocks(g) * mapk::OWN_N; }
 
 // Which start a run takes when neither its flags nor map_autotune say: the frontier start pushes
 // from the accepting vertices (one random access per entry that holds one) and runs in one launch, the
 // dense start streams the whole matrix.  Measured: layered graphs (1 entry in 200) 3.4 against 16.4 ms at
-// 2^26 vertices, an interleaved product with 1 entry in 7 (1.6 M vertices) 6.4 against 4.6 ms; graphs that
-// fit into one cluster always gain (16,384 vertices 0.12 against 0.44 ms).
-static bool default_fstart(const map_graph *g) { return runs_in_tail(g) || g->acc_entries <= g->m / 16; }
+// 2^26 vertices, an interleaved product with 1 entry in 7 (1.6 M vertices) 6.4 against 4.6 ms in k_run.  Graphs
+// that fit into one cluster or the SMs' shared memory gain whatever the share (16,384 vertices 0.12 against
+// 0.44 ms, that product 1.5 ms in k_own).
+static bool default_fstart(const map_graph *g) { return runs_in_tail(g) || runs_in_own(g) || g->acc_entries <= g->m / 16; }
 
 // a launch of `blocks` blocks of TT threads as one cluster
 static void cluster_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &attr, uint32_t blocks, size_t smem, cudaStream_t s)
@@ -1019,26 +1052,38 @@ static int launch_run(map_graph *g, cudaStream_t s, const map_opts &opts, const 
     const int cluster = g->comp ? 0 : tail_blocks();
     const bool whole = runs_in_tail(g);
     if (whole) return launch_tail(a, sync_sched, true, tail_blocks_for(g->n, cluster), s);
-    a.tail_cap = (uint32_t)cluster * mapk::TAIL_N;
+    a.tail_cap = tail_cap();
+    const uint32_t own = own_blocks(g);
+    a.own_cap = own * mapk::OWN_N;
     CK(cudaMemsetAsync(g->run_ctl, 0, sizeof(mapk::RunCtl), s));
     if (g->comp) {
         mapk::k_batch_begin<<<(g->ncomp + 255) / 256, 256, 0, s>>>(dev_of(g));
         CK(cudaGetLastError());
     }
     cudaLaunchConfig_t cfg = {};
-    // (rounds_grid counts blocks of 256 threads; a served job's share of the device carries over)
-    cfg.gridDim = dim3((unsigned)std::max(1, std::min(g->sms * occ, g->rounds_grid * 256 / mapk::RT)));
-    cfg.blockDim = dim3(mapk::RT);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (g->comp && sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_run<true, true>, a));
-    else if (g->comp) CK(cudaLaunchKernelEx(&cfg, mapk::k_run<false, true>, a));
-    else if (sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_run<true, false>, a));
-    else CK(cudaLaunchKernelEx(&cfg, mapk::k_run<false, false>, a));
+    const bool in_own = runs_in_own(g);
+    if (!in_own) {
+        const int sms = g->sm_share ? g->sm_share : g->sms;
+        cfg.gridDim = dim3((unsigned)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)sms * occ, (n + mapk::RT - 1) / mapk::RT)));
+        cfg.blockDim = dim3(mapk::RT);
+        if (g->comp && sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_run<true, true>, a));
+        else if (g->comp) CK(cudaLaunchKernelEx(&cfg, mapk::k_run<false, true>, a));
+        else if (sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_run<true, false>, a));
+        else CK(cudaLaunchKernelEx(&cfg, mapk::k_run<false, false>, a));
+    }
+    if (own) {
+        cfg.gridDim = dim3(own);
+        cfg.blockDim = dim3(mapk::TT);
+        cfg.dynamicSmemBytes = mapk::OWN_SMEM;
+        if (sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_own<true>, a, in_own ? 1u : 0u));
+        else CK(cudaLaunchKernelEx(&cfg, mapk::k_own<false>, a, in_own ? 1u : 0u));
+    }
     return cluster ? launch_tail(a, sync_sched, false, (uint32_t)cluster, s) : MAP_OK;
 }
 
@@ -1154,7 +1199,7 @@ static int run_impl(map_graph *g, const map_opts *opts_in, map_result *res, uint
         res->device_ms = ms;
         res->round_ms = R->ph_rounds * 1e-6;
         res->check_ms = R->ph_check * 1e-6;
-        res->launches = g->comp || runs_in_tail(g) || !tail_blocks() ? 1 : 2;
+        res->launches = runs_in_tail(g) ? 1 : 1 + (!runs_in_own(g) && own_blocks(g) ? 1 : 0) + (!g->comp && tail_blocks() ? 1 : 0);
         g->dirty = R->gave_up != 0; // (a run stopped by a limit has put its state back)
         if (R->status == mapk::ST_LIMIT) return fail(MAP_ERR_LIMIT, "map_run: max_outer or max_inner reached");
         if (R->gave_up) return fail(MAP_ERR_TIMEOUT, "map_run: a bounded device wait (grid barrier) gave up after seconds without progress");
@@ -2439,6 +2484,7 @@ void share_rounds(map_server *sv, map_graph *g)
     if (sv->slots <= 1) return;
     const int share = std::max(1, (int)((int64_t)g->sms * g->occ_rounds / (int64_t)sv->slots));
     g->rounds_grid = std::min(g->rounds_grid, share);
+    g->sm_share = std::max(1, g->sms / (int)sv->slots);
 }
 
 using Clock = std::chrono::steady_clock;

@@ -69,7 +69,9 @@ struct RunCtl {
     Cnt32 witness;    // NONE - the smallest self-mapped vertex (0: none)
     Line64 relax, frows;
     uint32_t gave_up;
-    // what k_run leaves to k_tail: the compact graph and where the run stands
+    Line64 obar[3];   // k_own's grid barriers
+    Cnt32 ocnt[2];    // k_own: vertices with a value, by outer iteration mod 2
+    // what k_run leaves to k_own (hand = 1), and either to k_tail (2): the compact graph and where the run stands
     uint32_t hand, V, set, outer, nacc;
     unsigned long long inner_total, ph_rounds, ph_check, t0;
 };
@@ -93,7 +95,7 @@ struct RunArgs {
     uint32_t count_round1;       // asynchronous relaxations: the pushes of round 1 (else m per iteration)
     uint64_t timeout_ns;
     const uint32_t *prep;        // not NULL: (error, accepting vertices, entries) that k_prepare found
-    uint32_t tail_cap;           // compact graphs of at most this many vertices are left to k_tail (0: none)
+    uint32_t tail_cap, own_cap;  // compact graphs of at most this many vertices are left to k_tail / k_own (0: none)
     // batched runs
     const uint32_t *comp;
     CompState *cs;
@@ -136,15 +138,16 @@ constexpr unsigned long long RUN_STOP = 1ull << 47, RUN_FOUND = 1ull << 32, RUN_
 // counts the next step needs come with the release instead of by another read.  One release
 // reduction to arrive, acquire loads to wait: 1.3 us with 304 blocks, against 2.6 us for a returning
 // atomic, a reset and a generation word with 912.  Returns false if the wait gave up.
-__device__ __forceinline__ bool run_barrier(RunCtl *c, RunSmem &sh, uint32_t &seq, unsigned long long payload,
+template <class Smem>
+__device__ __forceinline__ bool run_barrier(RunCtl *c, Line64 *bar, Smem &sh, uint32_t &seq, unsigned long long payload,
                                             unsigned long long &total)
 {
     __syncthreads();
     if (threadIdx.x == 0) {
         const uint32_t slot = seq % 3;
         // (the next barrier's word was last read before the barrier before this one)
-        if (blockIdx.x == 0) *(volatile unsigned long long *)&c->bar[(seq + 1) % 3].v = 0;
-        unsigned long long *w = &c->bar[slot].v, x = 0;
+        if (blockIdx.x == 0) *(volatile unsigned long long *)&bar[(seq + 1) % 3].v = 0;
+        unsigned long long *w = &bar[slot].v, x = 0;
         asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(w), "l"((1ull << 48) | payload) : "memory");
         uint32_t ok = 1;
         for (uint32_t it = 0;; ++it) {
@@ -434,7 +437,7 @@ template <bool SYNC, bool BATCH> struct Run {
         __syncthreads();
         for (uint32_t i = threadIdx.x; i < kept; i += RT) next[sh.lbase + i] = sh.list[i];
         for (uint32_t i = threadIdx.x; i < tkept; i += RT) a.touched[sh.tbase + i] = sh.touch[i];
-        return run_barrier(c, sh, seq, (unsigned long long)ln + (timing ? RUN_STOP : 0ull), total);
+        return run_barrier(c, c->bar, sh, seq, (unsigned long long)ln + (timing ? RUN_STOP : 0ull), total);
     }
 };
 
@@ -495,7 +498,7 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
     } else {
         for (uint64_t i = tid; i < n; i += nthreads) a.out[i] = NONE;
     }
-    alive = run_barrier(c, sh, run.seq, 0, total);
+    alive = run_barrier(c, c->bar, sh, run.seq, 0, total);
 
     Space &sp = run.sp;
     sp.V = n;
@@ -592,7 +595,7 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
             wit = sh.tn;
             if (threadIdx.x == 0 && wit != NONE) atomicMax(&c->witness.v, NONE - wit);
         }
-        alive = run_barrier(c, sh, run.seq,
+        alive = run_barrier(c, c->bar, sh, run.seq,
                             (unsigned long long)elim + (wit != NONE ? RUN_FOUND : 0ull) + (late() ? RUN_STOP : 0ull), total);
         if (!alive) break;
         if (lead) phase(ph_check);
@@ -629,7 +632,7 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
                     a.out[run.id_of(v)] = __ldcg(a.tval + i) - 1u - *(volatile uint32_t *)&a.cs[g].off;
             }
             nacc -= (uint32_t)(total & RUN_COUNT);
-            alive = run_barrier(c, sh, run.seq, 0, total);
+            alive = run_barrier(c, c->bar, sh, run.seq, 0, total);
             if (!alive) break;
             unsigned on = 0;
             if (blockIdx.x == 0) {
@@ -662,7 +665,7 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
                 __syncthreads();
                 on = sh.ln;
             }
-            alive = run_barrier(c, sh, run.seq, on, total);
+            alive = run_barrier(c, c->bar, sh, run.seq, on, total);
             if (!alive) break;
             go = (total & RUN_COUNT) != 0;
         }
@@ -671,7 +674,7 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
         if (go && compactable && (uint64_t)T + nacc <= min(sp.V / (sp.meta ? 4u : 8u), cap)) {
             for (uint64_t i = tid; i < T; i += nthreads) a.rank[run.id_of(__ldcg(a.touched + i))] = (uint32_t)i + 1;
             if (lead) *(volatile uint32_t *)&c->acnt.v = 0;
-            if (!(alive = run_barrier(c, sh, run.seq, 0, total))) break;
+            if (!(alive = run_barrier(c, c->bar, sh, run.seq, 0, total))) break;
             uint32_t *anew = la; // (no round is in flight)
             for (uint64_t i = tid; i < sp.na; i += nthreads) { // (one that no row holds offers nothing to anyone)
                 const uint32_t v = __ldcg(alist + i);
@@ -686,7 +689,7 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
                 }
                 anew[agg_inc(&c->acnt.v)] = k - 1;
             }
-            if (!(alive = run_barrier(c, sh, run.seq, 0, total))) break;
+            if (!(alive = run_barrier(c, c->bar, sh, run.seq, 0, total))) break;
             const uint32_t V2 = T + *(volatile uint32_t *)&c->xcnt.v, na2 = *(volatile uint32_t *)&c->acnt.v;
             uint32_t *const ps = pool_set(a, set ^ 1);
             uint4 *const meta2 = reinterpret_cast<uint4 *>(ps);
@@ -729,7 +732,7 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
                     for (int j = 0; j < RUN_P; ++j)
                         if (live[j]) rc2[first + pair[j]] = __ldcg(a.rank + run.id_of(__ldcg(sp.rc + pos[j]))) - 1;
                 });
-            if (!(alive = run_barrier(c, sh, run.seq, over ? 1 : 0, total))) break;
+            if (!(alive = run_barrier(c, c->bar, sh, run.seq, over ? 1 : 0, total))) break;
             if (lead) *(volatile uint32_t *)&c->xcnt.v = *(volatile uint32_t *)&c->ecnt.v = 0;
             if (total & RUN_COUNT) { // too many readers for the pool: stay in the whole graph
                 compactable = false;
@@ -744,7 +747,7 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
                 uint32_t *const t = alist;
                 alist = la;
                 la = t;
-                if (!BATCH && V2 <= a.tail_cap) { // small enough for one cluster
+                if (!BATCH && V2 <= max(a.tail_cap, a.own_cap)) { // small enough for one of the kernels below
                     hand = true;
                     break;
                 }
@@ -773,11 +776,11 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
             c->ph_rounds = ph_rounds;
             c->ph_check = ph_check;
             c->t0 = t0;
-            c->hand = 1;
+            c->hand = sp.V <= a.tail_cap ? 2u : 1u;
         }
         return;
     }
-    if (alive) alive = run_barrier(c, sh, run.seq, 0, total);
+    if (alive) alive = run_barrier(c, c->bar, sh, run.seq, 0, total);
     if (lead) {
         RunRes *R = a.res;
         R->verdict = verdict;
@@ -812,6 +815,9 @@ constexpr int TT = 1024;             // threads per block
 constexpr uint32_t TAIL_N = 8704;    // vertices per block: 26 bytes of shared memory each
 constexpr uint32_t TAIL_C = 16;      // blocks at most
 constexpr size_t TAIL_SMEM = (size_t)TAIL_N * 26;
+// graphs up to here run in the cluster, larger ones over the grid (k_own).  Layered graphs, synchronous, us per
+// run with k_tail / k_own: 16,000 vertices 166 / 205, 30,000 262 / 235, 60,000 317 / 238, 130,000 470 / 263
+constexpr uint32_t TAIL_BEST = 16384;
 constexpr uint32_t TAIL_LONG = 16;   // reader lists longer than this are walked by a whole warp
 
 __device__ __forceinline__ uint32_t cluster_rank()
@@ -852,7 +858,7 @@ __global__ void __launch_bounds__(TT, 1) k_tail(const __grid_constant__ RunArgs 
     __shared__ unsigned long long s_word[2][TAIL_C], s_part[TT / 32], s_sum;
     __shared__ uint32_t s_min[TT / 32], s_n, s_late;
     RunCtl *c = a.ctl;
-    if (!whole && !*(volatile uint32_t *)&c->hand) return; // k_run finished the run (every block returns)
+    if (!whole && *(volatile uint32_t *)&c->hand != 2) return; // the run is finished (every block returns)
     if (a.prep && a.prep[0]) return;                        // k_prepare refused the graph
     const uint32_t nacc0 = a.prep ? a.prep[1] : a.nacc0;
     const uint64_t m = a.prep ? a.prep[2] : a.m;
@@ -1136,6 +1142,460 @@ __global__ void __launch_bounds__(TT, 1) k_tail(const __grid_constant__ RunArgs 
         R->ph_check = ph_check;
     }
     cluster_barrier(); // no block leaves while another may still write into its shared memory
+}
+
+// -------------------------------------------------------- medium graphs --
+//
+// k_own: the same run over the grid for a whole graph, or the compact graph k_run leaves, of at most OWN_N
+// vertices per SM.  Block b owns a contiguous share of the vertices and keeps their reader ranges, own offers
+// and last values in shared memory, and their reader lists too where they fit.  A push is a maximum
+// on the reader's word in global memory that nothing waits for; every round the owner reads its share's
+// words (coalesced) and pushes for those that changed.  So a round is one coalesced read, the reader ids,
+// and the barrier, where k_run's lists take seven dependent accesses (list, state, reader range, reader,
+// returning atomic, list position, barrier) and 1.3 us more.  Reading the whole share costs V * 4 bytes a round
+// from L2, about 1 us at the largest size.
+//   asynchronous  in[0] / in[1] = the values, by outer iteration mod 2; last = the value pushed last
+//   synchronous   in[0] / in[1] = the inboxes, by round mod 2 (as in k_tail); last = the value
+constexpr uint32_t OWN_N = 12288;              // vertices per block: 18 bytes of shared memory each
+constexpr uint32_t OWN_SMEM = 224 * 1024;      // the rest holds reader lists
+constexpr int OWN_U = 4;                       // words read ahead per thread
+constexpr uint32_t OWN_HUB = 2048;             // reader lists longer than this are walked by the whole block
+
+struct OwnSmem {
+    unsigned long long word;
+    uint32_t ok, n, hubs, late, ebase, xbase;
+    uint32_t scan[TT / 32], scan2[TT / 32], mins[TT / 32], sums[TT / 32];
+    uint32_t hub[32];
+    unsigned long long part[TT / 32];
+};
+
+// exclusive prefix of x over the block (TT threads), *total its sum
+__device__ __forceinline__ uint32_t own_scan(uint32_t x, uint32_t *s, uint32_t &total)
+{
+    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+    const uint32_t incl = warp_inclusive_scan(x);
+    __syncthreads(); // (s is free)
+    if (lane == 31) s[warp] = incl;
+    __syncthreads();
+    if (warp == 0) s[lane] = warp_inclusive_scan(s[lane]);
+    __syncthreads();
+    total = s[TT / 32 - 1];
+    return incl - x + (warp ? s[warp - 1] : 0u);
+}
+
+template <bool SYNC>
+__global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a, uint32_t whole)
+{
+    extern __shared__ uint32_t s_mem[];
+    __shared__ OwnSmem sh;
+    RunCtl *c = a.ctl;
+    if (!whole && *(volatile uint32_t *)&c->hand != 1) return; // finished, or left to k_tail (every block returns)
+    const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+    const bool lead = blockIdx.x == 0 && tid == 0;
+    const uint32_t n = a.n, V = whole ? n : *(volatile uint32_t *)&c->V;
+    const uint32_t share = (V + gridDim.x - 1) / gridDim.x, v0 = min(V, blockIdx.x * share), mine = min(V, v0 + share) - v0;
+    const uint32_t stride = (share + 3) & ~3u;
+    uint32_t *const last = s_mem, *const own = last + stride, *const beg = own + stride, *const end = beg + stride;
+    uint16_t *const queue = reinterpret_cast<uint16_t *>(end + stride);
+    uint32_t *const s_rc = end + stride + stride / 2;
+    const uint32_t rc_room = OWN_SMEM / 4 - (4 * stride + stride / 2);
+    uint32_t set = whole ? 1u : *(volatile uint32_t *)&c->set;
+    const uint32_t cap = pool_cap(n);
+    uint32_t *const ps = pool_set(a, set);
+    const uint4 *meta = reinterpret_cast<const uint4 *>(ps);
+    const uint32_t *row = ps + 4ull * cap, *rc = whole ? a.rcol : ps + 6ull * cap;
+    uint32_t *const in0 = reinterpret_cast<uint32_t *>(a.W), *const in1 = in0 + n;
+    const uint64_t t0 = whole ? global_ns() : *(volatile unsigned long long *)&c->t0;
+    uint64_t mark = global_ns(), ph_rounds = 0, ph_check = 0;
+    auto phase = [&](uint64_t &acc) {
+        const uint64_t now = global_ns();
+        if ((int64_t)(now - mark) > 0) {
+            acc += now - mark;
+            mark = now;
+        }
+    };
+    auto late = [&] { return lead && (int64_t)(global_ns() - t0) > (int64_t)a.timeout_ns; };
+
+    // ---- the share's readers, offers and (where they fit) reader lists
+    uint32_t entries = 0; // reader entries of the share so far
+    bool cached = true;
+    for (uint32_t i0 = 0; i0 < mine; i0 += TT) { // (block-uniform)
+        const uint32_t i = i0 + tid;
+        uint32_t b = 0, e = 0;
+        if (i < mine) {
+            const uint32_t v = v0 + i;
+            uint32_t o;
+            if (whole) {
+                b = __ldg(a.rrowptr + v);
+                e = __ldg(a.rrowptr + v + 1);
+                o = ((__ldg(a.acc0 + (v >> 5)) >> (v & 31u)) & 1u) ? v + 1 : 0u;
+            } else {
+                const uint4 q = __ldg(meta + v);
+                b = q.x;
+                e = q.y;
+                o = q.z;
+            }
+            last[i] = 0;
+            own[i] = o;
+            beg[i] = b;
+            end[i] = e;
+        }
+        uint32_t total;
+        const uint32_t at = entries + own_scan(e - b, sh.scan, total);
+        cached = cached && total <= rc_room - min(rc_room, entries) && entries <= rc_room;
+        entries += total; // (a wrapped sum: not cached any more)
+        if (cached) { // (a list that no thread copies alone in reasonable time: the warp does)
+            for (unsigned m = __ballot_sync(0xFFFFFFFFu, e - b > TAIL_LONG); m; m &= m - 1) {
+                const int src = __ffs(m) - 1;
+                const uint32_t bb = __shfl_sync(0xFFFFFFFFu, b, src), ll = __shfl_sync(0xFFFFFFFFu, e - b, src),
+                               aa = __shfl_sync(0xFFFFFFFFu, at, src);
+                for (uint32_t j = lane; j < ll; j += 32) s_rc[aa + j] = __ldg(rc + bb + j);
+            }
+            if (e - b <= TAIL_LONG)
+                for (uint32_t j = 0; j < e - b; ++j) s_rc[at + j] = __ldg(rc + b + j);
+        }
+    }
+    __syncthreads();
+    if (cached) { // ranges into the copy
+        uint32_t done = 0;
+        for (uint32_t i0 = 0; i0 < mine; i0 += TT) {
+            const uint32_t i = i0 + tid, len = i < mine ? end[i] - beg[i] : 0u;
+            uint32_t total;
+            const uint32_t at = done + own_scan(len, sh.scan, total);
+            done += total;
+            if (i < mine) {
+                beg[i] = at;
+                end[i] = at + len;
+            }
+        }
+    }
+    if (whole) { // the run's accepting set, and an empty map
+        const uint64_t gid = (uint64_t)blockIdx.x * TT + tid, threads = (uint64_t)gridDim.x * TT;
+        for (uint64_t i = gid; i < a.words; i += threads) a.acc[i] = __ldg(a.acc0 + i);
+    }
+    if (tid == 0) sh.late = 0;
+    __syncthreads();
+
+    uint32_t outer = whole ? 0u : *(volatile uint32_t *)&c->outer, nacc = whole ? a.nacc0 : *(volatile uint32_t *)&c->nacc;
+    uint32_t status = ST_OK, verdict = 0, witness = NONE, seq = 0, gate = a.tail_cap / 2;
+    unsigned long long relax = 0, frows = 0, inner_total = 0, total = 0;
+    bool go = nacc != 0, alive = true, hand = false;
+    const auto reader = [&](uint32_t j) { return cached ? s_rc[j] : __ldg(rc + j); };
+    while (go) {
+        ++outer;
+        uint32_t *const val = (outer & 1) ? in1 : in0; // (asynchronous)
+        if (lead && (SYNC || !a.count_round1)) relax += a.m; // round 1 covers every row
+        uint32_t r = 0;
+        for (;;) {
+            ++r;
+            uint32_t *const inbox = (r & 1) ? in0 : in1; // what came in round r - 1 (synchronous)
+            uint32_t *const to = SYNC ? ((r & 1) ? in1 : in0) : val;
+            const bool pushes = r <= a.max_inner; // (past the limit the last round's values are only taken)
+            uint32_t hits = 0;
+            for (uint32_t pass = 0;; ++pass) { // (asynchronous: the share once more, lc_passes times while it changes)
+                if (tid == 0) sh.n = sh.hubs = 0;
+                __syncthreads();
+                const bool start = r == 1 && pass == 0;
+                const uint32_t *const words = (SYNC ? inbox : val) + v0;
+                for (uint32_t i0 = 0; i0 < mine; i0 += TT * OWN_U) { // (block-uniform) OWN_U words in flight per thread
+                    uint32_t y[OWN_U];
+#pragma unroll
+                    for (int k = 0; k < OWN_U; ++k) {
+                        const uint32_t i = i0 + k * TT + tid;
+                        y[k] = i >= mine ? 0u : start ? own[i] : __ldcg(words + i);
+                    }
+#pragma unroll
+                    for (int k = 0; k < OWN_U; ++k) {
+                        const uint32_t i = i0 + k * TT + tid;
+                        if (i0 + k * TT >= mine) break; // (block-uniform)
+                        const unsigned some = __ballot_sync(0xFFFFFFFFu, y[k] != 0);
+                        if (!some) continue; // (warp-uniform: nothing here)
+                        bool hit = y[k] != 0;
+                        if (!start) {
+                            if (SYNC) {
+                                if (i < mine) inbox[v0 + i] = 0; // (whole lines)
+                                if (hit && r > 2) {              // a frontier row of round r - 1
+                                    const uint32_t v = v0 + i;
+                                    relax += whole ? __ldg(a.rowptr + v + 1) - __ldg(a.rowptr + v) : __ldg(row + v);
+                                    ++frows;
+                                }
+                            }
+                            hit = hit && y[k] > last[i];
+                            if (hit) last[i] = y[k];
+                        }
+                        const unsigned m = __ballot_sync(0xFFFFFFFFu, hit);
+                        if (!m) continue;
+                        uint32_t at = 0;
+                        if (lane == 0) at = atomicAdd(&sh.n, (uint32_t)__popc(m));
+                        at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(m & ((1u << lane) - 1u));
+                        if (hit) queue[at] = (uint16_t)i;
+                    }
+                }
+                __syncthreads();
+                const uint32_t nq = sh.n;
+                hits += nq;
+                if (!nq || !pushes) break;
+                for (uint32_t q0 = 0; q0 < nq; q0 += TT) { // (block-uniform)
+                    const uint32_t q = q0 + tid;
+                    uint32_t o = 0, b = 0, e = 0;
+                    if (q < nq) {
+                        const uint32_t i = queue[q];
+                        o = start ? own[i] : max(last[i], own[i]);
+                        b = beg[i];
+                        e = end[i];
+                        if (!SYNC) {
+                            if (r > 1 || pass || a.count_round1) relax += e - b;
+                            if (r > 1) ++frows;
+                        }
+                        if (e - b > OWN_HUB) { // the whole block's, below (the first 32 of a pass)
+                            const uint32_t h = atomicAdd(&sh.hubs, 1u);
+                            if (h < 32) {
+                                sh.hub[h] = i;
+                                b = e;
+                            }
+                        }
+                    }
+                    for (unsigned m = __ballot_sync(0xFFFFFFFFu, e - b > TAIL_LONG); m; m &= m - 1) {
+                        const int src = __ffs(m) - 1;
+                        const uint32_t ob = __shfl_sync(0xFFFFFFFFu, o, src), bb = __shfl_sync(0xFFFFFFFFu, b, src),
+                                       ll = __shfl_sync(0xFFFFFFFFu, e - b, src);
+#pragma unroll 4
+                        for (uint32_t j = lane; j < ll; j += 32) atomicMax(to + reader(bb + j), ob);
+                        if ((int)lane == src) b = e;
+                    }
+                    for (uint32_t j = 0; j < e - b; j += 4) { // up to four readers in flight
+                        uint32_t w[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) w[k] = j + k < e - b ? reader(b + j + k) : NONE;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            if (w[k] != NONE) atomicMax(to + w[k], o);
+                    }
+                }
+                __syncthreads();
+                for (uint32_t h = 0; h < min(sh.hubs, 32u); ++h) {
+                    const uint32_t i = sh.hub[h], b = beg[i], ll = end[i] - b;
+                    const uint32_t o = start ? own[i] : max(last[i], own[i]);
+#pragma unroll 4
+                    for (uint32_t j = tid; j < ll; j += TT) atomicMax(to + reader(b + j), o);
+                }
+                __syncthreads(); // (the queue and the hubs are read)
+                if (SYNC || pass >= a.lc_passes) break;
+            }
+            alive = run_barrier(c, c->obar, sh, seq, (unsigned long long)hits + ((r & 3u) == 0 && late() ? RUN_STOP : 0ull), total);
+            if (!alive) break;
+            if (r == 1) continue; // (the limit and the end of the rounds: once round 1's values are taken)
+            if (total & RUN_STOP) status = ST_TIMEOUT;
+            else if ((total & RUN_COUNT) && !pushes) status = ST_LIMIT;
+            if (!(total & RUN_COUNT) || status != ST_OK) break;
+        }
+        if (!alive) break;
+        const uint32_t rounds = status == ST_TIMEOUT ? r : r - 1;
+        inner_total += rounds;
+        if (lead) {
+            if (outer - 1 < a.hist_cap) a.hist[outer - 1] = rounds;
+            if (outer - 1 < RUN_HIST) a.res->hist[outer - 1] = rounds;
+            phase(ph_rounds);
+        }
+        if (status != ST_OK) break;
+        // ---- self-map test and elimination (last[] holds the values)
+        uint32_t wit = NONE, elim = 0, have = 0, settled = 0;
+        for (uint32_t i0 = 0; i0 < mine; i0 += TT) {
+            const uint32_t i = i0 + tid, x = i < mine ? last[i] : 0u;
+            if (x) {
+                ++have;
+                if (x - 1 == (whole ? v0 + i : __ldg(&meta[v0 + i].w))) wit = min(wit, x - 1);
+            }
+            const unsigned same = __match_any_sync(0xFFFFFFFFu, x); // (many vertices share a few values)
+            if (x && x != settled && lane == (unsigned)(__ffs(same) - 1)) {
+                const uint32_t u = x - 1, bit = 1u << (u & 31u);
+                if ((__ldcg(a.acc + (u >> 5)) & bit) && (atomicAnd(a.acc + (u >> 5), ~bit) & bit)) ++elim;
+            }
+            settled = x;
+        }
+        wit = __reduce_min_sync(0xFFFFFFFFu, wit);
+        elim = __reduce_add_sync(0xFFFFFFFFu, elim);
+        have = __reduce_add_sync(0xFFFFFFFFu, have);
+        if (lane == 0) {
+            sh.mins[warp] = wit;
+            sh.sums[warp] = elim;
+            sh.scan[warp] = have;
+        }
+        __syncthreads();
+        if (tid < 32) {
+            wit = __reduce_min_sync(0xFFFFFFFFu, sh.mins[tid]);
+            elim = __reduce_add_sync(0xFFFFFFFFu, sh.sums[tid]);
+            have = __reduce_add_sync(0xFFFFFFFFu, sh.scan[tid]);
+        }
+        if (tid == 0) {
+            if (wit != NONE) atomicMax(&c->witness.v, NONE - wit);
+            if (have) atomicAdd(&c->ocnt[outer & 1].v, have);
+            if (lead) *(volatile uint32_t *)&c->ocnt[(outer + 1) & 1].v = 0;
+        }
+        alive = run_barrier(c, c->obar, sh, seq,
+                            (unsigned long long)elim + (wit != NONE ? RUN_FOUND : 0ull) + (late() ? RUN_STOP : 0ull), total);
+        if (!alive) break;
+        const uint32_t T = *(volatile uint32_t *)&c->ocnt[outer & 1].v;
+        if (lead) phase(ph_check);
+        if (total & (RUN_STOP - RUN_FOUND)) {
+            verdict = 1;
+            witness = NONE - *(volatile uint32_t *)&c->witness.v;
+            go = false;
+        } else if (T == 0) {
+            go = false; // nothing reaches a remaining accepting vertex
+        } else {
+            nacc -= (uint32_t)(total & RUN_COUNT);
+            if (nacc == 0) go = false;
+            else if ((a.max_outer && outer >= a.max_outer) || outer > a.nacc0) {
+                status = ST_LIMIT;
+                go = false;
+            } else if (total & RUN_STOP) {
+                status = ST_TIMEOUT;
+                go = false;
+            }
+        }
+        if (!go) break;
+        // ---- the next iteration: eliminated vertices offer nothing, values back to none
+        const bool pack = T <= gate;
+        uint32_t V2 = 0, E2 = 0;
+        const uint32_t lim = min(a.tail_cap, cap);
+        const uint64_t ecap = (uint64_t)n * 3 / 4 - 8;
+        uint32_t *const ps2 = pool_set(a, set ^ 1);
+        uint4 *const meta2 = reinterpret_cast<uint4 *>(ps2);
+        uint32_t *const row2 = ps2 + 4ull * cap, *const rc2 = ps2 + 6ull * cap;
+        bool over = false;
+        for (uint32_t i0 = 0; i0 < mine; i0 += TT) { // (block-uniform)
+            const uint32_t i = i0 + tid;
+            uint32_t x = 0, o = 0, len = 0;
+            if (i < mine) {
+                x = last[i];
+                o = own[i];
+                if (o && !((__ldcg(a.acc + ((o - 1) >> 5)) >> ((o - 1) & 31u)) & 1u)) own[i] = o = 0;
+                len = end[i] - beg[i];
+                if (!SYNC && x) val[v0 + i] = 0; // (the next iteration's pushes go to the other array)
+                last[i] = 0;
+            }
+            if (!pack) continue;
+            // compaction into the graph of the vertices that had a value and the accepting ones, as in k_run
+            const bool member = x != 0 || (o != 0 && len != 0);
+            uint32_t nm, ne;
+            const uint32_t at = own_scan(member ? 1u : 0u, sh.scan, nm), ea = own_scan(member ? len : 0u, sh.scan2, ne);
+            if (tid == 0) {
+                sh.xbase = nm ? atomicAdd(&c->xcnt.v, nm) : 0u;
+                sh.ebase = ne ? atomicAdd(&c->ecnt.v, ne) : 0u;
+            }
+            __syncthreads();
+            const uint32_t xb = sh.xbase, eb = sh.ebase;
+            if ((uint64_t)xb + nm > lim || (uint64_t)eb + ne > ecap) over = true;
+            if (member && !over) {
+                const uint32_t v = v0 + i, id = whole ? v : __ldg(&meta[v].w), k = xb + at;
+                meta2[k] = make_uint4(eb + ea, eb + ea + len, o, id);
+                if (SYNC) row2[k] = whole ? __ldg(a.rowptr + v + 1) - __ldg(a.rowptr + v) : __ldg(row + v);
+                a.rank[id] = k + 1;
+                last[i] = k + 1; // (for the reader lists below)
+            }
+            __syncthreads(); // (the bases are read)
+        }
+        if (!pack) continue;
+        alive = run_barrier(c, c->obar, sh, seq, over ? 1u : 0u, total);
+        if (!alive) break;
+        V2 = *(volatile uint32_t *)&c->xcnt.v;
+        E2 = *(volatile uint32_t *)&c->ecnt.v;
+        const bool fits = (total & RUN_COUNT) == 0;
+        for (uint32_t i0 = 0; i0 < mine; i0 += TT) {
+            const uint32_t i = i0 + tid, k = i < mine ? last[i] : 0u;
+            uint32_t b = 0, e = 0, at = 0;
+            if (fits && k) {
+                b = beg[i];
+                e = end[i];
+                at = meta2[k - 1].x;
+            }
+            if (i < mine) last[i] = 0;
+            auto number = [&](uint32_t w) { return __ldcg(a.rank + (whole ? w : __ldg(&meta[w].w))) - 1; };
+            for (unsigned m = __ballot_sync(0xFFFFFFFFu, e - b > TAIL_LONG); m; m &= m - 1) {
+                const int src = __ffs(m) - 1;
+                const uint32_t bb = __shfl_sync(0xFFFFFFFFu, b, src), ll = __shfl_sync(0xFFFFFFFFu, e - b, src),
+                               aa = __shfl_sync(0xFFFFFFFFu, at, src);
+                for (uint32_t j = lane; j < ll; j += 32) rc2[aa + j] = number(reader(bb + j));
+                if ((int)lane == src) b = e;
+            }
+            for (uint32_t j = 0; j < e - b; ++j) rc2[at + j] = number(reader(b + j));
+        }
+        if (fits) {
+            if (lead) {
+                c->V = V2;
+                c->set = set ^ 1;
+            }
+            hand = true;
+            break;
+        }
+        // too many vertices or readers: try again once half as many have a value
+        gate = min(gate, T) / 2;
+        alive = run_barrier(c, c->obar, sh, seq, 0, total); // (every block has read the counts)
+        if (!alive) break;
+        if (lead) *(volatile uint32_t *)&c->xcnt.v = *(volatile uint32_t *)&c->ecnt.v = 0;
+        (void)E2;
+    }
+    // ---- the map of the last iteration; the state back to zero
+    if (alive && !hand) {
+        uint32_t *const val = (outer & 1) ? in1 : in0;
+        for (uint32_t i = tid; i < mine; i += TT) {
+            uint32_t x = last[i];
+            if (SYNC) {
+                if (status != ST_OK) in0[v0 + i] = in1[v0 + i] = 0; // (at the fix-point the inboxes are empty)
+            } else {
+                if (status != ST_OK) x = max(x, __ldcg(val + v0 + i));
+                if (x) val[v0 + i] = 0;
+            }
+            if (a.out) {
+                if (whole) a.out[v0 + i] = x - 1u; // (no value: MAP_NONE)
+                else if (x) a.out[__ldg(&meta[v0 + i].w)] = x - 1u;
+            }
+        }
+    } else if (hand && whole && a.out) { // k_tail writes the values of the last iteration over this
+        for (uint32_t i = tid; i < mine; i += TT) a.out[v0 + i] = NONE;
+    }
+    for (int q = 0; q < 2; ++q) {
+        const unsigned long long s = warp_sum64(q ? frows : relax);
+        __syncthreads();
+        if (lane == 0) sh.part[warp] = s;
+        __syncthreads();
+        if (tid == 0) {
+            unsigned long long t = 0;
+            for (int w = 0; w < TT / 32; ++w) t += sh.part[w];
+            if (t) atomicAdd(q ? &c->frows.v : &c->relax.v, t);
+        }
+    }
+    if (alive) alive = run_barrier(c, c->obar, sh, seq, 0, total);
+    if (!lead) return;
+    if (!whole) { // and what k_run had counted
+        inner_total += c->inner_total;
+        ph_rounds += c->ph_rounds;
+        ph_check += c->ph_check;
+    }
+    if (hand) {
+        c->outer = outer;
+        c->nacc = nacc;
+        c->inner_total = inner_total;
+        c->ph_rounds = ph_rounds;
+        c->ph_check = ph_check;
+        c->t0 = t0;
+        c->hand = 2;
+        return;
+    }
+    RunRes *R = a.res;
+    R->verdict = verdict;
+    R->witness = witness;
+    R->outer = outer;
+    R->status = alive ? status : ST_TIMEOUT;
+    R->gave_up = alive ? 0u : 1u;
+    R->nacc = nacc;
+    R->inner_total = inner_total;
+    R->relax = *(volatile unsigned long long *)&c->relax.v;
+    R->frontier_rows = *(volatile unsigned long long *)&c->frows.v;
+    R->ph_rounds = ph_rounds;
+    R->ph_check = ph_check;
+    if (!whole) c->hand = 0;
 }
 
 // Set-up of a small graph in one cluster (before k_tail): bounds and validity of the CSR, the accepting set

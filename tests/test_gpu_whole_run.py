@@ -172,3 +172,19 @@ def test_static_refuses_what_it_refused(pkg, rowptr, col, code, on_device):
         pkg.map_run_static(2, to(rowptr), to(col), to([1]), map_out=out)
     assert e.value.code == getattr(pkg, f"MAP_ERR_{code}")
     assert out.tolist() == [9, 9]
+
+
+@pytest.mark.parametrize("n", [16384, 16385, 152 * 1024 + 1, 152 * 12288, 152 * 12288 + 1])
+def test_sizes_around_the_grid_kernel(pkg, n):
+    """k_own between the cluster and k_run: a vertex more than the cluster takes, than a thread holds, and at
+    its capacity (12,288 per block on 152 SMs); dense accepting sets, a planted cycle."""
+    compare(pkg, mapgen.layered_graph(n, max(8, n // 9000), seed=3), runs=1)
+    compare(pkg, mapgen.layered_graph(n, max(8, n // 9000), seed=4, plant=True, acc_p=0.2), runs=1)
+
+
+@pytest.mark.parametrize("acc_p", [0.001, 0.5, 1.0])
+def test_interleaved_products_and_dense_accepting_sets(pkg, acc_p):
+    g = mapgen.product_graph(6, 6, True)
+    compare(pkg, g)
+    r = mapgen.random_graph(200_000, 1, 6, acc_p, seed=8, variant="plain")
+    compare(pkg, r, pkg.MAP_FLAG_FRONTIER_START)
