@@ -264,6 +264,16 @@ int tail_blocks()
     return best;
 }
 
+int lasso_occupancy()
+{
+    int o = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, mapk::k_lasso, mapk::RT, 0) != cudaSuccess) {
+        cudaGetLastError();
+        o = 1;
+    }
+    return std::max(1, o);
+}
+
 // whether k_own's blocks fit on the current device (one per SM, a cooperative launch).  Asked once per device.
 bool own_fits()
 {
@@ -1007,13 +1017,39 @@ static int take_result(const mapk::RunRes &R, const map_opts &opts, uint64_t m, 
     return MAP_OK;
 }
 
+// the control block of whole-run launches, allocated on first use
+static int ensure_run_ctl(map_graph *g)
+{
+    if (!g->run_ctl) CK(cudaMallocAsync((void **)&g->run_ctl, sizeof(mapk::RunCtl) + sizeof(mapk::RunRes), g->stream));
+    return MAP_OK;
+}
+
+// where a launch leaves its result: the handle's page-locked slot, or (without one) behind its control block
+static mapk::RunRes *run_result(const map_graph *g)
+{
+    return g->h_ctl_pinned ? reinterpret_cast<mapk::RunRes *>(reinterpret_cast<uint8_t *>(g->h_ctl) + PinnedSlots::RES)
+                           : reinterpret_cast<mapk::RunRes *>(g->run_ctl + 1);
+}
+
+// wait for the stream; *R: the result, copied to *pageable where there is no page-locked slot
+static int await_result(const map_graph *g, cudaStream_t s, mapk::RunRes *pageable, const mapk::RunRes **R)
+{
+    *R = run_result(g);
+    if (!g->h_ctl_pinned) {
+        CK(cudaMemcpyAsync(pageable, *R, sizeof *pageable, cudaMemcpyDeviceToHost, s));
+        *R = pageable;
+    }
+    CK(cudaStreamSynchronize(s));
+    return MAP_OK;
+}
+
 // Queue one whole run as a single launch (k_run) and fill in the result from where the kernel left it.
 static int launch_run(map_graph *g, cudaStream_t s, const map_opts &opts, const Ctl &init, bool count_round1,
                       uint32_t *out)
 {
     static const int occ = run_occupancy();
     const size_t n = g->n;
-    if (!g->run_ctl) CK(cudaMallocAsync((void **)&g->run_ctl, sizeof(mapk::RunCtl) + sizeof(mapk::RunRes), s));
+    if (const int rc = ensure_run_ctl(g)) return rc;
     mapk::RunArgs a;
     memset(&a, 0, sizeof a);
     a.n = g->n;
@@ -1032,8 +1068,7 @@ static int launch_run(map_graph *g, cudaStream_t s, const map_opts &opts, const 
     a.rank = g->mval;
     a.pool = g->flist;
     a.ctl = g->run_ctl;
-    a.res = g->h_ctl_pinned ? reinterpret_cast<mapk::RunRes *>(reinterpret_cast<uint8_t *>(g->h_ctl) + PinnedSlots::RES)
-                            : reinterpret_cast<mapk::RunRes *>(g->run_ctl + 1);
+    a.res = run_result(g);
     a.hist = g->hist;
     a.hist_cap = g->hist_cap;
     a.out = out;
@@ -1184,15 +1219,10 @@ static int run_impl(map_graph *g, const map_opts *opts_in, map_result *res, uint
         for (uint32_t k = 0; k < reps; ++k)
             if ((rc = launch_run(g, s, opts, init, asked || g->tuned, map_out ? init.out : nullptr))) return rc;
         CK(cudaEventRecord(g->ev[1], s));
-        mapk::RunRes pageable; // (without a page-locked slot the result is copied from the device)
-        const mapk::RunRes *R = &pageable;
-        if (g->h_ctl_pinned) {
-            R = reinterpret_cast<const mapk::RunRes *>(reinterpret_cast<const uint8_t *>(g->h_ctl) + PinnedSlots::RES);
-        } else {
-            CK(cudaMemcpyAsync(&pageable, g->run_ctl + 1, sizeof pageable, cudaMemcpyDeviceToHost, s));
-        }
+        mapk::RunRes pageable;
+        const mapk::RunRes *R = nullptr;
         if (map_out && !out_dev) CK(cudaMemcpyAsync(map_out, g->xbuf, (size_t)n * 4, cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
+        if ((rc = await_result(g, s, &pageable, &R))) return rc;
         float ms = 0.f;
         CK(cudaEventElapsedTime(&ms, g->ev[0], g->ev[1]));
         if ((rc = take_result(*R, opts, g->m, sync_sched, g->hist, g->hist_cap, s, res))) return rc;
@@ -1503,52 +1533,6 @@ int map_autotune(map_graph *g, uint32_t sched, map_tune_result *out)
     return MAP_OK;
 }
 
-// shortest path source -> target along rows (at least one edge) into host path[0..cap); *len = vertices
-static int bfs_path(map_graph *g, uint32_t source, uint32_t target, uint32_t *path, uint32_t cap, uint32_t *len)
-{
-    cudaStream_t s = g->stream;
-    const uint32_t n = g->n;
-    uint32_t *parent = g->xbuf, *q0 = g->list, *q1 = g->list + n; // list holds 3n entries
-    uint32_t *cnt = &g->ctl->lcnt[0].v, *cnt2 = &g->ctl->lcnt[1].v, *found = &g->ctl->lcnt[2].v;
-    mapk::k_fill<<<grid_for(g, n, 1), 256, 0, s>>>(parent, n, mapk::NONE);
-    CK(cudaGetLastError());
-    if (source != target) { // the source is reached from the start
-        CK(cudaMemcpyAsync(parent + source, &source, 4, cudaMemcpyHostToDevice, s));
-    }
-    uint32_t one = 1, zero = 0;
-    CK(cudaMemcpyAsync(q0, &source, 4, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(cnt, &one, 4, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(found, &zero, 4, cudaMemcpyHostToDevice, s));
-    uint32_t h[2] = {1, 0};
-    for (uint32_t level = 0; level <= n && h[0]; ++level) {
-        CK(cudaMemcpyAsync(cnt2, &zero, 4, cudaMemcpyHostToDevice, s));
-        mapk::k_bfs_level<<<grid_for(g, h[0], 1), 256, 0, s>>>(q0, cnt, g->rowptr, g->colidx, parent, q1, cnt2,
-                                                                 target, found);
-        CK(cudaGetLastError());
-        CK(cudaMemcpyAsync(&h[0], cnt2, 4, cudaMemcpyDeviceToHost, s));
-        CK(cudaMemcpyAsync(&h[1], found, 4, cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
-        if (h[1]) break;
-        std::swap(q0, q1);
-        std::swap(cnt, cnt2);
-    }
-    if (!h[1]) return fail(MAP_ERR_ARG, "map_lasso: vertex %u is not reachable from %u", target, source);
-    // a parent chain visits distinct vertices (target twice when it is the source): <= n + 1 entries
-    uint32_t k = 0, *out = g->list;
-    const uint32_t dcap = cap < n + 1 ? cap : n + 1;
-    mapk::k_walk_back<<<1, 32, 0, s>>>(parent, source, target, out, dcap, n + 1, found);
-    CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(&k, found, 4, cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    if (k == 0xFFFFFFFFu || k > cap) return fail(MAP_ERR_LIMIT, "map_lasso: the path does not fit into %u entries", cap);
-    std::vector<uint32_t> rev(k);
-    CK(cudaMemcpyAsync(rev.data(), out, (size_t)k * 4, cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    for (uint32_t i = 0; i < k; ++i) path[i] = rev[k - 1 - i];
-    *len = k;
-    return MAP_OK;
-}
-
 int map_lasso(map_graph *g, uint32_t init, uint32_t witness, uint32_t *path, uint32_t cap, uint32_t *prefix_len,
               uint32_t *cycle_len)
 {
@@ -1557,17 +1541,63 @@ int map_lasso(map_graph *g, uint32_t init, uint32_t witness, uint32_t *path, uin
     if (g->comp) return fail(MAP_ERR_ARG, "map_lasso: single graphs only");
     if (witness >= g->n || (init != MAP_NONE && init >= g->n)) return fail(MAP_ERR_ARG, "map_lasso: vertex out of range");
     *prefix_len = *cycle_len = 0;
+    cudaStream_t s = g->stream;
+    const size_t n = g->n;
+    int rc = ensure_run_ctl(g);
+    if (rc) return rc;
+    mapk::LassoArgs a;
+    a.n = g->n;
+    a.rowptr = g->rowptr;
+    a.colidx = g->colidx;
+    const bool prefix = init != MAP_NONE && init != witness;
+    a.from[0] = prefix ? init : mapk::NONE;
+    a.from[1] = a.to[0] = a.to[1] = witness;
+    a.parent[0] = g->xbuf;
+    a.parent[1] = g->touched;
+    a.qa = g->list;
+    a.qb = g->list + n;
+    a.path[0] = g->elog;
+    a.path[1] = g->list + 2 * n; // (n entries and the slack behind them)
+    a.ctl = g->run_ctl;
+    a.res = run_result(g);
+    CK(cudaMemsetAsync(g->run_ctl, 0, sizeof(mapk::RunCtl), s));
+    static const int occ = lasso_occupancy();
+    cudaLaunchConfig_t cfg = {};
+    // (at least two blocks: each walks one path back)
+    cfg.gridDim = dim3((unsigned)std::max<uint64_t>(2, std::min<uint64_t>((uint64_t)g->sms * occ, (n + mapk::RT - 1) / mapk::RT)));
+    cfg.blockDim = dim3(mapk::RT);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    CK(cudaLaunchKernelEx(&cfg, mapk::k_lasso, a));
+    mapk::RunRes pageable;
+    const mapk::RunRes *R = nullptr;
+    if ((rc = await_result(g, s, &pageable, &R))) return rc;
+    if (R->gave_up) return fail(MAP_ERR_TIMEOUT, "map_lasso: a bounded device wait (grid barrier) gave up after seconds without progress");
+    // path q (len vertices, backwards) into path[at ..], forwards
+    const auto take = [&](int q, uint32_t source, uint32_t len, uint32_t at) -> int {
+        if (!len) return fail(MAP_ERR_ARG, "map_lasso: vertex %u is not reachable from %u", witness, source);
+        if (len > cap - at) return fail(MAP_ERR_LIMIT, "map_lasso: the path does not fit into %u entries", cap - at);
+        if (len <= mapk::RUN_HIST / 2) {
+            memcpy(path + at, R->hist + q * (mapk::RUN_HIST / 2), (size_t)len * 4);
+        } else {
+            CK(cudaMemcpyAsync(path + at, a.path[q], (size_t)len * 4, cudaMemcpyDeviceToHost, s));
+            CK(cudaStreamSynchronize(s));
+        }
+        std::reverse(path + at, path + at + len);
+        return MAP_OK;
+    };
     uint32_t used = 0;
-    int rc = MAP_OK;
-    if (init != MAP_NONE && init != witness) { // init -> ... -> witness
-        uint32_t k = 0;
-        if ((rc = bfs_path(g, init, witness, path, cap, &k))) return rc;
-        used = k - 1; // the witness opens the cycle part
+    if (prefix) { // init -> ... -> witness
+        if ((rc = take(0, init, R->verdict, 0))) return rc;
+        used = R->verdict - 1; // the witness opens the cycle part
         *prefix_len = used;
     }
-    uint32_t k = 0; // witness -> ... -> witness
-    if ((rc = bfs_path(g, witness, witness, path + used, cap - used, &k))) return rc;
-    *cycle_len = k;
+    if ((rc = take(1, witness, R->witness, used))) return rc; // witness -> ... -> witness
+    *cycle_len = R->witness;
     return MAP_OK;
 }
 

@@ -168,45 +168,8 @@ __device__ __forceinline__ bool run_barrier(RunCtl *c, Line64 *bar, Smem &sh, ui
     return sh.ok != 0;
 }
 
-// the space a run works in: the whole graph, or the compact graph of a later iteration
-struct Space {
-    uint32_t V, na;          // vertices, accepting vertices listed
-    const uint4 *meta;       // compact: (first reader, end, own offer, original id); NULL: the whole graph
-    const uint32_t *rc;      // readers
-    const uint32_t *row;     // compact: row lengths (NULL: from rowptr)
-    const uint32_t *comp;    // batched: graph of each vertex
-};
-
-// compact arrays, set h (0 or 1) in the pool of 3n words
-__device__ __forceinline__ uint32_t pool_cap(uint32_t n) { return (n / 8) & ~3u; }
-__device__ __forceinline__ uint32_t *pool_set(const RunArgs &a, uint32_t h) { return a.pool + (uint64_t)h * ((a.n + a.n / 2) & ~3u); }
-
-template <bool SYNC, bool BATCH> struct Run {
-    static constexpr uint32_t S = (SYNC || BATCH) ? 2 : 1; // state words per vertex
-
-    const RunArgs &a;
-    RunSmem &sh;
-    Space sp;
-    uint32_t seq = 0, lseq = 0; // barriers and rounds of the whole run so far
-    unsigned long long relax = 0, frows = 0;
-
-    __device__ Run(const RunArgs &a_, RunSmem &s_) : a(a_), sh(s_) {}
-
-    __device__ __forceinline__ uint32_t id_of(uint32_t v) const { return sp.meta ? __ldcg(&sp.meta[v].w) : v; }
-    __device__ __forceinline__ bool accepting(uint32_t v) const
-    {
-        return sp.meta ? __ldcg(&sp.meta[v].z) != 0 : ((__ldcg(a.acc + (v >> 5)) >> (v & 31u)) & 1u) != 0;
-    }
-
-    __device__ __forceinline__ uint32_t readers(uint32_t v) const
-    {
-        if (!sp.meta) return __ldg(a.rrowptr + v + 1) - __ldg(a.rrowptr + v);
-        const uint4 q = __ldcg(sp.meta + v);
-        return q.y - q.x;
-    }
-
     // append w (where flag) to the staged list s_buf (count *s_cnt); what does not fit goes to g directly
-    __device__ __forceinline__ void emit(bool flag, uint32_t w, uint32_t *s_buf, uint32_t *s_cnt, uint32_t *g, uint32_t *gcnt)
+    __device__ __forceinline__ void stage_emit(bool flag, uint32_t w, uint32_t *s_buf, uint32_t *s_cnt, uint32_t *g, uint32_t *gcnt)
     {
         const unsigned mask = __ballot_sync(0xFFFFFFFFu, flag);
         if (!mask) return;
@@ -230,7 +193,7 @@ template <bool SYNC, bool BATCH> struct Run {
     // range, begin(total) runs once per chunk, and the (offer, reader position) pairs are spread
     // evenly over the block's threads, RUN_P per thread and step: act(live, o, pos) for RUN_P pairs
     template <class Get, class Begin, class Act>
-    __device__ __forceinline__ void expand(uint64_t beg, uint64_t end, Get get, Begin begin, Act act)
+    __device__ __forceinline__ void expand(RunSmem &sh, uint64_t beg, uint64_t end, Get get, Begin begin, Act act)
     {
         for (uint64_t c0 = beg; c0 < end; c0 += RT) {
             const uint64_t i = c0 + threadIdx.x;
@@ -268,6 +231,43 @@ template <bool SYNC, bool BATCH> struct Run {
             }
             __syncthreads(); // before the shared arrays are refilled
         }
+    }
+
+// the space a run works in: the whole graph, or the compact graph of a later iteration
+struct Space {
+    uint32_t V, na;          // vertices, accepting vertices listed
+    const uint4 *meta;       // compact: (first reader, end, own offer, original id); NULL: the whole graph
+    const uint32_t *rc;      // readers
+    const uint32_t *row;     // compact: row lengths (NULL: from rowptr)
+    const uint32_t *comp;    // batched: graph of each vertex
+};
+
+// compact arrays, set h (0 or 1) in the pool of 3n words
+__device__ __forceinline__ uint32_t pool_cap(uint32_t n) { return (n / 8) & ~3u; }
+__device__ __forceinline__ uint32_t *pool_set(const RunArgs &a, uint32_t h) { return a.pool + (uint64_t)h * ((a.n + a.n / 2) & ~3u); }
+
+template <bool SYNC, bool BATCH> struct Run {
+    static constexpr uint32_t S = (SYNC || BATCH) ? 2 : 1; // state words per vertex
+
+    const RunArgs &a;
+    RunSmem &sh;
+    Space sp;
+    uint32_t seq = 0, lseq = 0; // barriers and rounds of the whole run so far
+    unsigned long long relax = 0, frows = 0;
+
+    __device__ Run(const RunArgs &a_, RunSmem &s_) : a(a_), sh(s_) {}
+
+    __device__ __forceinline__ uint32_t id_of(uint32_t v) const { return sp.meta ? __ldcg(&sp.meta[v].w) : v; }
+    __device__ __forceinline__ bool accepting(uint32_t v) const
+    {
+        return sp.meta ? __ldcg(&sp.meta[v].z) != 0 : ((__ldcg(a.acc + (v >> 5)) >> (v & 31u)) & 1u) != 0;
+    }
+
+    __device__ __forceinline__ uint32_t readers(uint32_t v) const
+    {
+        if (!sp.meta) return __ldg(a.rrowptr + v + 1) - __ldg(a.rrowptr + v);
+        const uint4 q = __ldcg(sp.meta + v);
+        return q.y - q.x;
     }
 
     // one push of offer o to reader w in round r: raised first in this round, with no value
@@ -412,11 +412,11 @@ template <bool SYNC, bool BATCH> struct Run {
                     CompState &s = a.cs[__ldcg(sp.comp + w[j])];
                     if (*(volatile uint32_t *)&s.last_change < r) atomicMax(&s.last_change, r);
                 }
-                emit(done[j].listed, w[j], sh.list, &sh.ln, next, lcnt);
-                emit(done[j].fresh, w[j], sh.touch, &sh.tn, a.touched, tcnt);
+                stage_emit(done[j].listed, w[j], sh.list, &sh.ln, next, lcnt);
+                stage_emit(done[j].fresh, w[j], sh.touch, &sh.tn, a.touched, tcnt);
             }
         };
-        expand(beg, end, get, begin, act);
+        expand(sh, beg, end, get, begin, act);
         if (!SYNC && !BATCH) {
             // the block pushes the live values of the vertices it listed itself once more (lc_passes
             // times), so that values travel several edges per barrier; they stay listed
@@ -426,7 +426,7 @@ template <bool SYNC, bool BATCH> struct Run {
                 const uint32_t e = min(sh.ln, RUN_CAP); // final: a block barrier ended the last chunk
                 __syncthreads();                        // (read by every thread before it grows)
                 if (e == q) break;
-                expand(q, e, get, begin, act);
+                expand(sh, q, e, get, begin, act);
                 q = e;
             }
         }
@@ -699,8 +699,8 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
             const uint64_t per = ((uint64_t)V2 + gridDim.x - 1) / gridDim.x;
             const uint64_t beg = min((uint64_t)V2, blockIdx.x * per), end = min((uint64_t)V2, beg + per);
             uint32_t first = 0; // this chunk's first entry in rc2
-            run.expand(
-                beg, end,
+            expand(
+                sh, beg, end,
                 [&](uint64_t i, uint32_t &, uint32_t &b, uint32_t &len) {
                     const uint32_t v = __ldcg(a.touched + i);
                     if (sp.meta) {
@@ -794,6 +794,102 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
         R->frontier_rows = *(volatile unsigned long long *)&c->frows.v;
         R->ph_rounds = ph_rounds;
         R->ph_check = ph_check;
+    }
+}
+
+// ---------------------------------------------------------- counterexample --
+//
+// k_lasso: the shortest paths from[q] -> to[q] along rows (at least one edge), q = 0 and 1 (from NONE: none
+// asked for), by breadth-first search with parent pointers, all levels in one cooperative launch.  A level
+// is a handful of dependent accesses; stepped from the host, each cost a launch, two pageable copies and a wait
+// besides (10^6 vertices, two searches of about ten levels: 1.0 ms, here 0.1 ms).  The path is left backwards
+// in path[q] (its first 256 vertices in res->hist[256 q ..] too) and its length in res->verdict and
+// res->witness (0: not reachable).
+struct LassoArgs {
+    uint32_t n;
+    const uint32_t *rowptr, *colidx;
+    uint32_t from[2], to[2];
+    uint32_t *parent[2], *path[2], *qa, *qb; // n entries each (path[1]: n + 1)
+    RunCtl *ctl;
+    RunRes *res;
+};
+
+__global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_lasso(const __grid_constant__ LassoArgs a)
+{
+    __shared__ RunSmem sh;
+    RunCtl *c = a.ctl;
+    const uint64_t tid = (uint64_t)blockIdx.x * RT + threadIdx.x, nthreads = (uint64_t)gridDim.x * RT;
+    uint32_t seq = 0, lseq = 0;
+    unsigned long long total = 0;
+    for (int q = 0; q < 2; ++q)
+        if (a.from[q] != NONE)
+            for (uint64_t i = tid; i < a.n; i += nthreads) // (a source that is not the target is reached from the start)
+                a.parent[q][i] = i == a.from[q] && a.from[q] != a.to[q] ? a.from[q] : NONE;
+    bool alive = run_barrier(c, c->bar, sh, seq, 0, total), found[2] = {false, false};
+    for (int q = 0; q < 2 && alive; ++q) {
+        if (a.from[q] == NONE) continue;
+        uint32_t *const parent = a.parent[q];
+        uint32_t nl = 1;
+        for (uint32_t level = 0; nl && !found[q] && alive; ++level) {
+            ++lseq;
+            const uint32_t *const in = (lseq & 1) ? a.qa : a.qb;
+            uint32_t *const out = (lseq & 1) ? a.qb : a.qa;
+            uint32_t *const cnt = &c->lcnt[lseq % 3].v;
+            __syncthreads(); // (the staged list of the last level is read)
+            if (threadIdx.x == 0) {
+                sh.ln = sh.tn = 0;
+                if (blockIdx.x == 0) *(volatile uint32_t *)&c->lcnt[(lseq + 1) % 3].v = 0;
+            }
+            __syncthreads();
+            const uint64_t per = ((uint64_t)nl + gridDim.x - 1) / gridDim.x;
+            const uint64_t beg = min((uint64_t)nl, blockIdx.x * per), end = min((uint64_t)nl, beg + per);
+            expand(
+                sh, beg, end,
+                [&](uint64_t i, uint32_t &o, uint32_t &b, uint32_t &len) {
+                    o = level ? __ldcg(in + i) : a.from[q];
+                    b = __ldg(a.rowptr + o);
+                    len = __ldg(a.rowptr + o + 1) - b;
+                },
+                [](bool, uint64_t, uint32_t, uint32_t, uint32_t) {},
+                [&](const bool (&live)[RUN_P], const uint32_t (&u)[RUN_P], const uint32_t (&pos)[RUN_P], const uint32_t (&)[RUN_P]) {
+#pragma unroll
+                    for (int j = 0; j < RUN_P; ++j) {
+                        bool fresh = false;
+                        uint32_t v = 0;
+                        if (live[j]) {
+                            v = __ldg(a.colidx + pos[j]) & 0x7FFFFFFFu; // bit 31 is the accepting flag
+                            fresh = __ldcg(parent + v) == NONE && atomicCAS(parent + v, NONE, u[j]) == NONE;
+                            if (fresh && v == a.to[q]) sh.tn = 1;
+                        }
+                        stage_emit(fresh, v, sh.list, &sh.ln, out, cnt);
+                    }
+                });
+            __syncthreads();
+            const uint32_t ln = sh.ln, kept = min(ln, RUN_CAP);
+            if (threadIdx.x == 0 && kept) sh.lbase = atomicAdd(cnt, kept);
+            __syncthreads();
+            for (uint32_t i = threadIdx.x; i < kept; i += RT) out[sh.lbase + i] = sh.list[i];
+            alive = run_barrier(c, c->bar, sh, seq, (unsigned long long)ln + (sh.tn ? RUN_FOUND : 0ull), total);
+            nl = (uint32_t)(total & RUN_COUNT);
+            found[q] = (total >> 32) != 0;
+        }
+    }
+    // walked back by one thread each
+    const uint32_t q = blockIdx.x;
+    if (threadIdx.x == 0 && q < 2) {
+        uint32_t k = 0;
+        if (alive && a.from[q] != NONE && found[q]) {
+            uint32_t v = a.to[q];
+            do { // (a parent chain visits distinct vertices, the target twice when it is the source)
+                if (k) v = __ldcg(a.parent[q] + v);
+                a.path[q][k] = v;
+                if (k < RUN_HIST / 2) a.res->hist[q * (RUN_HIST / 2) + k] = v;
+                ++k;
+            } while ((k == 1 || v != a.from[q]) && k <= a.n);
+        }
+        if (q == 0) a.res->verdict = k;
+        else a.res->witness = k;
+        if (q == 0) a.res->gave_up = alive ? 0u : 1u;
     }
 }
 
