@@ -168,70 +168,70 @@ __device__ __forceinline__ bool run_barrier(RunCtl *c, Line64 *bar, Smem &sh, ui
     return sh.ok != 0;
 }
 
-    // append w (where flag) to the staged list s_buf (count *s_cnt); what does not fit goes to g directly
-    __device__ __forceinline__ void stage_emit(bool flag, uint32_t w, uint32_t *s_buf, uint32_t *s_cnt, uint32_t *g, uint32_t *gcnt)
-    {
-        const unsigned mask = __ballot_sync(0xFFFFFFFFu, flag);
-        if (!mask) return;
-        const unsigned lane = lane_id(), leader = __ffs(mask) - 1;
-        uint32_t pos = 0;
-        if (lane == leader) pos = atomicAdd(s_cnt, (uint32_t)__popc(mask));
-        pos = __shfl_sync(0xFFFFFFFFu, pos, leader) + __popc(mask & ((1u << lane) - 1u));
-        const bool over = flag && pos >= RUN_CAP;
-        if (flag && !over) s_buf[pos] = w;
-        if (__any_sync(0xFFFFFFFFu, over)) {
-            const unsigned om = __ballot_sync(0xFFFFFFFFu, over);
-            uint32_t at = 0;
-            const unsigned ol = __ffs(om) - 1;
-            if (lane == ol) at = atomicAdd(gcnt, (uint32_t)__popc(om));
-            at = __shfl_sync(0xFFFFFFFFu, at, ol) + __popc(om & ((1u << lane) - 1u));
-            if (over) g[at] = w;
-        }
+// append w (where flag) to the staged list s_buf (count *s_cnt); what does not fit goes to g directly
+__device__ __forceinline__ void stage_emit(bool flag, uint32_t w, uint32_t *s_buf, uint32_t *s_cnt, uint32_t *g, uint32_t *gcnt)
+{
+    const unsigned mask = __ballot_sync(0xFFFFFFFFu, flag);
+    if (!mask) return;
+    const unsigned lane = lane_id(), leader = __ffs(mask) - 1;
+    uint32_t pos = 0;
+    if (lane == leader) pos = atomicAdd(s_cnt, (uint32_t)__popc(mask));
+    pos = __shfl_sync(0xFFFFFFFFu, pos, leader) + __popc(mask & ((1u << lane) - 1u));
+    const bool over = flag && pos >= RUN_CAP;
+    if (flag && !over) s_buf[pos] = w;
+    if (__any_sync(0xFFFFFFFFu, over)) {
+        const unsigned om = __ballot_sync(0xFFFFFFFFu, over);
+        uint32_t at = 0;
+        const unsigned ol = __ffs(om) - 1;
+        if (lane == ol) at = atomicAdd(gcnt, (uint32_t)__popc(om));
+        at = __shfl_sync(0xFFFFFFFFu, at, ol) + __popc(om & ((1u << lane) - 1u));
+        if (over) g[at] = w;
     }
+}
 
-    // entries [beg, end) in chunks of RT per block: get(i, o, b, len) gives an entry's offer and reader
-    // range, begin(total) runs once per chunk, and the (offer, reader position) pairs are spread
-    // evenly over the block's threads, RUN_P per thread and step: act(live, o, pos) for RUN_P pairs
-    template <class Get, class Begin, class Act>
-    __device__ __forceinline__ void expand(RunSmem &sh, uint64_t beg, uint64_t end, Get get, Begin begin, Act act)
-    {
-        for (uint64_t c0 = beg; c0 < end; c0 += RT) {
-            const uint64_t i = c0 + threadIdx.x;
-            uint32_t o = 0, b = 0, len = 0;
-            if (i < end) get(i, o, b, len);
-            const uint32_t incl = run_block_scan(len, sh.scan);
-            sh.o[threadIdx.x] = o;
-            sh.b[threadIdx.x] = b - (incl - len); // reader position of pair p: b[owner] + p (32-bit wrap intended)
-            sh.incl[threadIdx.x] = incl;
-            __syncthreads();
-            const uint32_t total = sh.incl[RT - 1];
-            begin(i < end, i, incl - len, len, total);
-            for (uint64_t p0 = 0; p0 < total; p0 += RT * RUN_P) {
-                bool live[RUN_P];
-                uint32_t off[RUN_P], pos[RUN_P], pair[RUN_P];
+// entries [beg, end) in chunks of RT per block: get(i, o, b, len) gives an entry's offer and reader
+// range, begin(total) runs once per chunk, and the (offer, reader position) pairs are spread
+// evenly over the block's threads, RUN_P per thread and step: act(live, o, pos) for RUN_P pairs
+template <class Get, class Begin, class Act>
+__device__ __forceinline__ void expand(RunSmem &sh, uint64_t beg, uint64_t end, Get get, Begin begin, Act act)
+{
+    for (uint64_t c0 = beg; c0 < end; c0 += RT) {
+        const uint64_t i = c0 + threadIdx.x;
+        uint32_t o = 0, b = 0, len = 0;
+        if (i < end) get(i, o, b, len);
+        const uint32_t incl = run_block_scan(len, sh.scan);
+        sh.o[threadIdx.x] = o;
+        sh.b[threadIdx.x] = b - (incl - len); // reader position of pair p: b[owner] + p (32-bit wrap intended)
+        sh.incl[threadIdx.x] = incl;
+        __syncthreads();
+        const uint32_t total = sh.incl[RT - 1];
+        begin(i < end, i, incl - len, len, total);
+        for (uint64_t p0 = 0; p0 < total; p0 += RT * RUN_P) {
+            bool live[RUN_P];
+            uint32_t off[RUN_P], pos[RUN_P], pair[RUN_P];
 #pragma unroll
-                for (int j = 0; j < RUN_P; ++j) {
-                    const uint64_t p = p0 + j * RT + threadIdx.x;
-                    live[j] = p < total;
-                    off[j] = pos[j] = 0;
-                    pair[j] = (uint32_t)p;
-                    if (live[j]) {
-                        uint32_t lo = 0, hi = RT - 1; // the owner: first entry with incl > p
+            for (int j = 0; j < RUN_P; ++j) {
+                const uint64_t p = p0 + j * RT + threadIdx.x;
+                live[j] = p < total;
+                off[j] = pos[j] = 0;
+                pair[j] = (uint32_t)p;
+                if (live[j]) {
+                    uint32_t lo = 0, hi = RT - 1; // the owner: first entry with incl > p
 #pragma unroll
-                        for (int st = 0; st < 9; ++st) {
-                            const uint32_t mid = (lo + hi) >> 1;
-                            if (sh.incl[mid] > (uint32_t)p) hi = mid;
-                            else lo = min(mid + 1, hi);
-                        }
-                        off[j] = sh.o[lo];
-                        pos[j] = sh.b[lo] + (uint32_t)p;
+                    for (int st = 0; st < 9; ++st) {
+                        const uint32_t mid = (lo + hi) >> 1;
+                        if (sh.incl[mid] > (uint32_t)p) hi = mid;
+                        else lo = min(mid + 1, hi);
                     }
+                    off[j] = sh.o[lo];
+                    pos[j] = sh.b[lo] + (uint32_t)p;
                 }
-                act(live, off, pos, pair);
             }
-            __syncthreads(); // before the shared arrays are refilled
+            act(live, off, pos, pair);
         }
+        __syncthreads(); // before the shared arrays are refilled
     }
+}
 
 // the space a run works in: the whole graph, or the compact graph of a later iteration
 struct Space {
