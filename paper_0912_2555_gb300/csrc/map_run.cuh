@@ -28,6 +28,11 @@
 // accesses over the full arrays are bound by address translation (measured: 42 G/s over 2 GB against
 // 128 G atomics/s and 300 G loads/s over a packed array), and the compact arrays stay in L2.
 //
+// Floods.  When a list holds a large share of the whole graph's vertices (one value sweeping a giant
+// component), its random accesses cost more than reading everything in order: from there on the iteration
+// runs in scan mode (Run::scan_round), with 4-byte state arrays, pushes that nothing waits for and each block
+// reading its contiguous share of the vertices every round.
+//
 // What it measured, ms per run (dense start in a CUDA graph -> here, k_tail included): layered 2^26
 // asynchronous 16.35 -> 3.4, 2^24 synchronous 7.3 -> 2.6, 10^6 asynchronous 2.82 -> 0.89, the 16,384-vertex
 // random graph 0.44 -> 0.12.
@@ -44,7 +49,13 @@ constexpr int RT = 512; // threads per block
 #define MAPGPU_RUN_P 1 // pushes per thread and step, all in flight together
 #endif
 constexpr int RUN_P = MAPGPU_RUN_P;
-constexpr uint32_t RUN_CAP = 2048;  // entries a block stages per round and list
+// a list of at least 1/16 of the whole graph (and RUN_SCAN_MIN entries) goes to scan mode, and back to lists below
+// 1/64.  Layered graphs with a planted cycle, ms per synchronous / asynchronous run, lists only -> with scans:
+// 2 M vertices 1.22 / 0.71 -> 0.57 / 0.41, 5 M 10.0 / 3.2 -> 3.2 / 1.6, 64-graph batch 6.4 / 5.1 -> 5.6 / 5.3 (shares
+// 32 and 128: 5 M 3.2 / 2.4; 8 and 32: 14 M async 3.2 instead of 2.85)
+constexpr uint32_t RUN_SCAN_SHARE = 16, RUN_LIST_SHARE = 64;
+constexpr uint32_t RUN_SCAN_MIN = 8192;
+constexpr uint32_t RUN_CAP = 8 * RT; // entries a block stages per round and list
 constexpr uint32_t RUN_HIST = 512;  // outer iterations whose rounds come back with the result
 
 struct alignas(128) Line64 {
@@ -218,7 +229,7 @@ __device__ __forceinline__ void expand(RunSmem &sh, uint64_t beg, uint64_t end, 
                 if (live[j]) {
                     uint32_t lo = 0, hi = RT - 1; // the owner: first entry with incl > p
 #pragma unroll
-                    for (int st = 0; st < 9; ++st) {
+                    for (int st = 1; st < RT; st *= 2) {
                         const uint32_t mid = (lo + hi) >> 1;
                         if (sh.incl[mid] > (uint32_t)p) hi = mid;
                         else lo = min(mid + 1, hi);
@@ -357,23 +368,31 @@ template <bool SYNC, bool BATCH> struct Run {
         len = idle ? 0u : e - b;
     }
 
-    __device__ __forceinline__ void add_row(bool row, uint32_t w)
-    { // a frontier row: its length to the relaxation count (batched: of its graph)
-        unsigned long long len = 0;
+    // a frontier row: its length to the relaxation count (batched: of its graph g too); the whole warp calls it
+    __device__ __forceinline__ void count_row(bool row, uint32_t len, uint32_t g)
+    {
         if (row) {
-            len = sp.row ? __ldcg(sp.row + w) : __ldg(a.rowptr + w + 1) - __ldg(a.rowptr + w);
             relax += len;
             ++frows;
         }
         if constexpr (BATCH) {
-            const uint32_t c = row ? __ldcg(sp.comp + w) : NONE;
+            const uint32_t c = row ? g : NONE, l = row ? len : 0u;
             const unsigned same = __match_any_sync(0xFFFFFFFFu, c);
-            const unsigned lo = __reduce_add_sync(same, (unsigned)(len & 0xFFFFu));
-            const unsigned hi = __reduce_add_sync(same, (unsigned)(len >> 16));
+            const unsigned lo = __reduce_add_sync(same, l & 0xFFFFu);
+            const unsigned hi = __reduce_add_sync(same, l >> 16);
             const unsigned long long sum = (unsigned long long)lo + ((unsigned long long)hi << 16);
             if (c != NONE && lane_id() == (unsigned)(__ffs(same) - 1) && sum)
                 atomicAdd((unsigned long long *)&a.cs[c].relax, sum);
         }
+    }
+    __device__ __forceinline__ void add_row(bool row, uint32_t w)
+    {
+        uint32_t len = 0, g = NONE;
+        if (row) {
+            len = sp.row ? __ldcg(sp.row + w) : __ldg(a.rowptr + w + 1) - __ldg(a.rowptr + w);
+            if (BATCH) g = __ldcg(sp.comp + w);
+        }
+        count_row(row, len, g);
     }
 
     // one round over `list` (nl entries); returns false if a wait gave up
@@ -408,10 +427,7 @@ template <bool SYNC, bool BATCH> struct Run {
 #pragma unroll
             for (int j = 0; j < RUN_P; ++j) {
                 if ((SYNC || BATCH) && r > 1) add_row(done[j].row, w[j]);
-                if (BATCH && done[j].listed) {
-                    CompState &s = a.cs[__ldcg(sp.comp + w[j])];
-                    if (*(volatile uint32_t *)&s.last_change < r) atomicMax(&s.last_change, r);
-                }
+                if (BATCH && done[j].listed) changed(w[j], r);
                 stage_emit(done[j].listed, w[j], sh.list, &sh.ln, next, lcnt);
                 stage_emit(done[j].fresh, w[j], sh.touch, &sh.tn, a.touched, tcnt);
             }
@@ -438,6 +454,212 @@ template <bool SYNC, bool BATCH> struct Run {
         for (uint32_t i = threadIdx.x; i < kept; i += RT) next[sh.lbase + i] = sh.list[i];
         for (uint32_t i = threadIdx.x; i < tkept; i += RT) a.touched[sh.tbase + i] = sh.touch[i];
         return run_barrier(c, c->bar, sh, seq, (unsigned long long)ln + (timing ? RUN_STOP : 0ull), total);
+    }
+
+    // ---- scan mode (whole graph): three arrays of n words in the pool.
+    //   synchronous   A / B = the inboxes of even / odd rounds, val = the values (as in k_tail)
+    //   asynchronous  val = the values, A = the value pushed last, B = (batched) the last round a row was reached in
+    __device__ __forceinline__ uint32_t *scan_val() const { return a.pool; }
+    __device__ __forceinline__ uint32_t *scan_a() const { return a.pool + a.n; }
+    __device__ __forceinline__ uint32_t *scan_b() const { return a.pool + 2ull * a.n; }
+
+    // from lists to scans after round r: the state words into the arrays and back to zero; a vertex of round r's
+    // list looks as if its value had just come in
+    __device__ __forceinline__ bool enter_scan(uint32_t r, unsigned long long &total)
+    {
+        const uint64_t nthreads = (uint64_t)gridDim.x * RT;
+        for (uint64_t v = (uint64_t)blockIdx.x * RT + threadIdx.x; v < a.n; v += nthreads) {
+            uint32_t x, in;
+            if constexpr (SYNC) {
+                ulonglong2 *p = reinterpret_cast<ulonglong2 *>(a.W) + v;
+                const ulonglong2 q = __ldcg(p);
+                if (q.x | q.y) *p = make_ulonglong2(0, 0);
+                const unsigned long long cur = (r & 1) ? q.y : q.x;
+                x = max((uint32_t)q.x, (uint32_t)q.y);
+                in = (cur >> 33) == r && ((cur >> 32) & 1u) ? x : 0u;
+                scan_val()[v] = in ? 0u : x;
+                ((r & 1) ? scan_b() : scan_a())[v] = in;
+                ((r & 1) ? scan_a() : scan_b())[v] = 0;
+            } else {
+                const unsigned long long q = __ldcg(a.W + (uint64_t)S * v);
+                if (q) a.W[(uint64_t)S * v] = 0;
+                if (BATCH && q) a.W[2ull * v + 1] = 0;
+                x = (uint32_t)(q >> 32);
+                scan_val()[v] = x;
+                scan_a()[v] = (uint32_t)q == (uint32_t)~r ? 0u : x;
+                if (BATCH) scan_b()[v] = 0;
+            }
+        }
+        if (blockIdx.x == 0 && threadIdx.x == 0) *(volatile uint32_t *)&a.ctl->ocnt[0].v = 0;
+        return run_barrier(a.ctl, a.ctl->bar, sh, seq, 0, total);
+    }
+
+    // round r: what came in in round r - 1 is taken (first: from the list of round r - 1, whose rows are counted
+    // already) and, unless past the limit, pushed on; total = the vertices that changed in round r - 1
+    __device__ __forceinline__ bool scan_round(uint32_t r, bool first, bool pushes, bool timing, unsigned long long &total)
+    {
+        constexpr uint32_t U = 4, CHUNK = RT * U; // words in flight per thread
+        uint32_t *const val = scan_val(), *const in = (r & 1) ? scan_a() : scan_b(), *const to = SYNC ? ((r & 1) ? scan_b() : scan_a()) : val;
+        // pieces of RT vertices go round the blocks: a wave through consecutive vertices (layers) is everybody's
+        const uint64_t step = (uint64_t)gridDim.x * RT, v0 = (uint64_t)blockIdx.x * RT, v1 = a.n;
+        uint32_t hits = 0;
+        __syncthreads();
+        if (threadIdx.x == 0) sh.ln = 0;
+        __syncthreads();
+        for (uint64_t c0 = v0; c0 < v1; c0 += step * U) { // (block-uniform)
+            // three steps with U loads in flight each: what came in; for the warps' words with something in
+            // them what the vertex holds, its row and graph; the rest
+            uint32_t y[U], z[U], len[U], g[U];
+            bool row[U];
+#pragma unroll
+            for (uint32_t k = 0; k < U; ++k) {
+                const uint64_t v = c0 + k * step + threadIdx.x;
+                y[k] = v < v1 ? __ldcg((SYNC ? in : val) + v) : 0u;
+                if (!SYNC) z[k] = v < v1 ? __ldcg(scan_a() + v) : 0u;
+                row[k] = !SYNC && BATCH && v < v1 && __ldcg(scan_b() + v) == r - 1;
+            }
+            uint32_t some = 0; // (warp-uniform) bit k: something in the warp's word k
+#pragma unroll
+            for (uint32_t k = 0; k < U; ++k) {
+                const uint32_t v = (uint32_t)(c0 + k * step + threadIdx.x);
+                if (SYNC) row[k] = y[k] != 0;
+                len[k] = 0;
+                g[k] = NONE;
+                if (!__any_sync(0xFFFFFFFFu, row[k] || (!SYNC && y[k] > z[k]))) continue;
+                some |= 1u << k;
+                if (c0 + k * step + threadIdx.x >= v1) continue;
+                if (SYNC) z[k] = __ldcg(val + v);
+                if (SYNC || BATCH) len[k] = __ldg(a.rowptr + v + 1) - __ldg(a.rowptr + v);
+                if (BATCH) g[k] = __ldcg(sp.comp + v);
+            }
+#pragma unroll
+            for (uint32_t k = 0; k < U; ++k) {
+                if (!((some >> k) & 1u)) continue;
+                const uint32_t v = (uint32_t)(c0 + k * step + threadIdx.x);
+                if (SYNC && c0 + k * step + threadIdx.x < v1) in[v] = 0; // (whole lines)
+                const bool hit = y[k] != 0 && y[k] > z[k];
+                if (hit) (SYNC ? val : scan_a())[v] = y[k];
+                if ((SYNC || BATCH) && !first && r > 2) count_row(row[k], len[k], g[k]); // frontier rows of round r - 1
+                if (BATCH && hit) changed_graph(g[k], r - 1);
+                const unsigned m = __ballot_sync(0xFFFFFFFFu, hit);
+                if (!m) continue;
+                uint32_t at = 0;
+                if (lane_id() == 0) at = atomicAdd(&sh.ln, (uint32_t)__popc(m));
+                at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(m & ((1u << lane_id()) - 1u));
+                if (hit) {
+                    sh.list[at] = v;
+                    sh.touch[at] = y[k];
+                }
+            }
+            __syncthreads();
+            const uint32_t nq = sh.ln; // (the hits of several chunks are pushed together)
+            if (nq + CHUNK <= RUN_CAP && c0 + step * U < v1) continue;
+            hits += nq;
+            if (pushes)
+                expand(
+                    sh, 0, nq,
+                    [&](uint64_t i, uint32_t &o, uint32_t &b, uint32_t &len) {
+                        const uint32_t u = sh.list[i];
+                        b = __ldg(a.rrowptr + u);
+                        len = __ldg(a.rrowptr + u + 1) - b;
+                        o = max(sh.touch[i], ((__ldcg(a.acc + (u >> 5)) >> (u & 31u)) & 1u) ? u + 1 : 0u);
+                    },
+                    [&](bool, uint64_t, uint32_t, uint32_t, uint32_t tot) {
+                        if (!SYNC && !BATCH && threadIdx.x == 0) relax += tot;
+                    },
+                    [&](const bool (&live)[RUN_P], const uint32_t (&o)[RUN_P], const uint32_t (&pos)[RUN_P], const uint32_t (&)[RUN_P]) {
+#pragma unroll
+                        for (int j = 0; j < RUN_P; ++j) {
+                            if (!live[j]) continue;
+                            const uint32_t w = __ldcg(sp.rc + pos[j]);
+                            atomicMax(to + w, o[j]);
+                            if (!SYNC && BATCH) atomicMax(scan_b() + w, r);
+                        }
+                    });
+            __syncthreads();
+            if (threadIdx.x == 0) sh.ln = 0;
+            __syncthreads();
+        }
+        return run_barrier(a.ctl, a.ctl->bar, sh, seq, (unsigned long long)hits + (timing ? RUN_STOP : 0ull), total);
+    }
+
+    // from scans back to lists after round r, in the place of the scan that would take what round r pushed: the
+    // values into the state words, the vertices that changed in round r to `list`, those with a value to the
+    // touched list; total = the length of `list`
+    __device__ __forceinline__ bool leave_scan(uint32_t r, uint32_t outer, uint32_t *list, unsigned long long &total)
+    {
+        constexpr uint32_t U = 4, CHUNK = RT * U;
+        RunCtl *c = a.ctl;
+        ++lseq;
+        uint32_t *const lcnt = &c->lcnt[lseq % 3].v, *const tcnt = &c->tcnt[outer & 1].v;
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            *(volatile uint32_t *)&c->lcnt[(lseq + 1) % 3].v = 0;
+            *(volatile uint32_t *)tcnt = 0; // (the touched list is made anew)
+        }
+        if (!run_barrier(c, c->bar, sh, seq, 0, total)) return false;
+        uint32_t *const val = scan_val(), *const in = (r & 1) ? scan_b() : scan_a();
+        uint32_t listed = 0;
+        for (uint64_t c0 = (uint64_t)blockIdx.x * CHUNK; c0 < a.n; c0 += (uint64_t)gridDim.x * CHUNK) { // (block-uniform)
+            uint32_t x[U], got = 0; // per vertex: its value; got: bits 0-3 = changed in round r
+            uint32_t nt = 0, nl = 0;
+#pragma unroll
+            for (uint32_t k = 0; k < U; ++k) {
+                const uint64_t v = c0 + k * RT + threadIdx.x;
+                x[k] = v < a.n ? __ldcg(val + v) : 0u;
+                bool row = false, ch = false;
+                if constexpr (SYNC) {
+                    const uint32_t y = v < a.n ? __ldcg(in + v) : 0u;
+                    row = y != 0;
+                    ch = y > x[k];
+                    x[k] = max(x[k], y);
+                } else if (v < a.n) {
+                    ch = x[k] > __ldcg(scan_a() + v);
+                    row = BATCH && __ldcg(scan_b() + v) == r;
+                }
+                if ((SYNC || BATCH) && r > 1 && __any_sync(0xFFFFFFFFu, row)) add_row(row, (uint32_t)v);
+                if (ch) {
+                    got |= 1u << k;
+                    ++nl;
+                    if (BATCH) changed((uint32_t)v, r);
+                }
+                if (x[k]) {
+                    ++nt;
+                    if constexpr (SYNC) {
+                        const unsigned long long w = ch ? (unsigned long long)r << 33 | 1ull << 32 | x[k] : x[k];
+                        reinterpret_cast<ulonglong2 *>(a.W)[v] = (r & 1) ? make_ulonglong2(0, w) : make_ulonglong2(w, 0);
+                    } else {
+                        a.W[(uint64_t)S * v] = (unsigned long long)x[k] << 32 | (uint32_t)~(ch ? r : 0u);
+                        if (BATCH) a.W[2ull * v + 1] = row ? r : 0u;
+                    }
+                }
+            }
+            const uint32_t both = run_block_scan(nt << 16 | nl, sh.scan); // (at most 2,048 each)
+            if (threadIdx.x == RT - 1) {
+                sh.tbase = atomicAdd(tcnt, both >> 16);
+                sh.lbase = atomicAdd(lcnt, both & 0xFFFFu);
+                listed += both & 0xFFFFu;
+            }
+            __syncthreads();
+            uint32_t ta = sh.tbase + (both >> 16) - nt, la = sh.lbase + (both & 0xFFFFu) - nl;
+#pragma unroll
+            for (uint32_t k = 0; k < U; ++k) {
+                const uint32_t v = (uint32_t)c0 + k * RT + threadIdx.x;
+                if (x[k]) a.touched[ta++] = v;
+                if ((got >> k) & 1u) list[la++] = v;
+            }
+            __syncthreads(); // (the bases are read)
+        }
+        if (threadIdx.x == RT - 1) sh.ln = listed;
+        __syncthreads();
+        return run_barrier(c, c->bar, sh, seq, sh.ln, total);
+    }
+
+    // batched: vertex v's graph changed in round r
+    __device__ __forceinline__ void changed(uint32_t v, uint32_t r) { changed_graph(__ldcg(sp.comp + v), r); }
+    __device__ __forceinline__ void changed_graph(uint32_t g, uint32_t r)
+    {
+        CompState &s = a.cs[g];
+        if (*(volatile uint32_t *)&s.last_change < r) atomicMax(&s.last_change, r);
     }
 };
 
@@ -516,16 +738,42 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
         // ---- rounds to the fix-point
         const uint32_t *list = alist;
         uint32_t nl = sp.na, r = 0;
-        for (;;) {
-            ++r;
-            alive = run.round(list, nl, (r & 1) ? la : lb, r, outer, (r & 3u) == 0 && late(), total);
-            if (!alive) break;
-            if (!SYNC && !BATCH && r > 1) run.frows += lead ? nl : 0u; // the vertices that pushed
-            nl = (uint32_t)(total & RUN_COUNT);
-            list = (r & 1) ? la : lb;
-            if (total & RUN_STOP) status = ST_TIMEOUT;
-            else if (nl && r + 1 > a.max_inner) status = ST_LIMIT;
-            if (!nl || status != ST_OK) break;
+        bool scan = false; // scan mode; then `first`: the state has just been brought into its arrays
+        for (bool first = false;;) {
+            if (!scan) {
+                ++r;
+                alive = run.round(list, nl, (r & 1) ? la : lb, r, outer, (r & 3u) == 0 && late(), total);
+                if (!alive) break;
+                if (!SYNC && !BATCH && r > 1) run.frows += lead ? nl : 0u; // the vertices that pushed
+                nl = (uint32_t)(total & RUN_COUNT);
+                list = (r & 1) ? la : lb;
+                if (total & RUN_STOP) status = ST_TIMEOUT;
+                else if (nl && r + 1 > a.max_inner) status = ST_LIMIT;
+                if (!nl || status != ST_OK) break;
+                if (!sp.meta && nl >= max(n / RUN_SCAN_SHARE, RUN_SCAN_MIN)) {
+                    scan = first = true;
+                    if (!(alive = run.enter_scan(r, total))) break;
+                }
+            } else { // (one scan takes what round r pushed and pushes round r + 1)
+                const bool pushes = r + 1 <= a.max_inner;
+                if (!(alive = run.scan_round(r + 1, first, pushes, (r & 3u) == 0 && late(), total))) break;
+                first = false;
+                nl = (uint32_t)(total & RUN_COUNT); // changed in round r
+                if (!SYNC && !BATCH && lead && pushes) run.frows += nl;
+                if (total & RUN_STOP) status = ST_TIMEOUT;
+                else if (nl && !pushes) status = ST_LIMIT;
+                if (nl && pushes) ++r;
+                if (!nl || status != ST_OK) break;
+                if (nl < n / RUN_LIST_SHARE) {
+                    uint32_t *const next = (r & 1) ? la : lb;
+                    if (!(alive = run.leave_scan(r, outer, next, total))) break;
+                    scan = false;
+                    nl = (uint32_t)(total & RUN_COUNT);
+                    list = next;
+                    if (nl && r + 1 > a.max_inner) status = ST_LIMIT;
+                    if (!nl || status != ST_OK) break;
+                }
+            }
         }
         if (!alive) break;
         inner_total += r;
@@ -535,24 +783,29 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
             phase(ph_rounds);
         }
         // ---- self-map test and elimination over the vertices with a value; their state back to zero
-        const uint32_t T = *(volatile uint32_t *)&c->tcnt[outer & 1].v;
+        uint32_t T = *(volatile uint32_t *)&c->tcnt[outer & 1].v;
+        const uint32_t bound = scan ? n : T;
+        uint32_t have = 0;
         if (lead) *(volatile uint32_t *)&c->tcnt[(outer + 1) & 1].v = 0;
         uint32_t elim = 0, wit = NONE, settled = 0;
-        for (uint64_t base = tid - lane_id(); base < T; base += nthreads) { // (warp-uniform)
+        for (uint64_t base = tid - lane_id(); base < bound; base += nthreads) { // (warp-uniform)
             const uint64_t i = base + lane_id();
             uint32_t g = NONE, removed = 0, val = 0;
-            if (i < T) {
-                const uint32_t v = __ldcg(a.touched + i);
+            if (i < bound) {
+                const uint32_t v = scan ? (uint32_t)i : __ldcg(a.touched + i);
                 // (exchanges, not stores: scattered 8-byte stores ran at 14 G/s here, atomics at over 100)
                 uint32_t x;
-                if constexpr (SYNC) {
+                if (scan) {
+                    x = __ldcg(run.scan_val() + v);
+                    have += x != 0;
+                } else if constexpr (SYNC) {
                     x = max((uint32_t)atomicExch(a.W + 2ull * v, 0ull), (uint32_t)atomicExch(a.W + 2ull * v + 1, 0ull));
                 } else {
                     x = (uint32_t)(atomicExch(a.W + (uint64_t)run.S * v, 0ull) >> 32);
                     if (BATCH) atomicExch(a.W + 2ull * v + 1, 0ull);
                 }
-                a.tval[i] = x;
-                if (BATCH) g = __ldcg(sp.comp + v);
+                if (!scan) a.tval[i] = x;
+                if (BATCH && x) g = __ldcg(sp.comp + v);
                 if (status == ST_OK) val = x;
                 if (val && x - 1 == run.id_of(v)) {
                     wit = min(wit, x - 1);
@@ -594,10 +847,13 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
             elim = sh.ln;
             wit = sh.tn;
             if (threadIdx.x == 0 && wit != NONE) atomicMax(&c->witness.v, NONE - wit);
+            have = __reduce_add_sync(0xFFFFFFFFu, have);
+            if (have && lane_id() == 0) atomicAdd(&c->ocnt[0].v, have);
         }
         alive = run_barrier(c, c->bar, sh, run.seq,
                             (unsigned long long)elim + (wit != NONE ? RUN_FOUND : 0ull) + (late() ? RUN_STOP : 0ull), total);
         if (!alive) break;
+        if (scan) T = *(volatile uint32_t *)&c->ocnt[0].v;
         if (lead) phase(ph_check);
         if constexpr (!BATCH) {
             if (status != ST_OK) go = false; // a limit inside the rounds
@@ -619,17 +875,21 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
                 }
             }
             if (!go && a.out) // the last iteration's map
-                for (uint64_t i = tid; i < T; i += nthreads)
-                    a.out[run.id_of(__ldcg(a.touched + i))] = __ldcg(a.tval + i) - 1u;
+                for (uint64_t i = tid; i < bound; i += nthreads) {
+                    if (scan) a.out[i] = __ldcg(run.scan_val() + i) - 1u; // (no value: MAP_NONE)
+                    else a.out[run.id_of(__ldcg(a.touched + i))] = __ldcg(a.tval + i) - 1u;
+                }
         } else {
             if (status == ST_OK && (total & RUN_STOP)) status = ST_TIMEOUT;
             uint32_t left;
             bool limit;
             // the maps of the graphs that end here
-            for (uint64_t i = tid; a.out && i < T; i += nthreads) {
-                const uint32_t v = __ldcg(a.touched + i), g = __ldcg(sp.comp + v);
+            for (uint64_t i = tid; a.out && i < bound; i += nthreads) {
+                const uint32_t v = scan ? (uint32_t)i : __ldcg(a.touched + i), x = scan ? __ldcg(run.scan_val() + i) : __ldcg(a.tval + i);
+                if (!x) continue;
+                const uint32_t g = __ldcg(sp.comp + v);
                 if (!comp_goes_on(a.cs[g], status, a.max_outer, left, limit))
-                    a.out[run.id_of(v)] = __ldcg(a.tval + i) - 1u - *(volatile uint32_t *)&a.cs[g].off;
+                    a.out[run.id_of(v)] = x - 1u - *(volatile uint32_t *)&a.cs[g].off;
             }
             nacc -= (uint32_t)(total & RUN_COUNT);
             alive = run_barrier(c, c->bar, sh, run.seq, 0, total);
@@ -671,7 +931,7 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
         }
         // ---- compaction: go on in the graph of the vertices that had a value and the accepting ones
         const uint32_t cap = pool_cap(n);
-        if (go && compactable && (uint64_t)T + nacc <= min(sp.V / (sp.meta ? 4u : 8u), cap)) {
+        if (go && compactable && !scan && (uint64_t)T + nacc <= min(sp.V / (sp.meta ? 4u : 8u), cap)) {
             for (uint64_t i = tid; i < T; i += nthreads) a.rank[run.id_of(__ldcg(a.touched + i))] = (uint32_t)i + 1;
             if (lead) *(volatile uint32_t *)&c->acnt.v = 0;
             if (!(alive = run_barrier(c, c->bar, sh, run.seq, 0, total))) break;

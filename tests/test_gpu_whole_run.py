@@ -188,3 +188,41 @@ def test_interleaved_products_and_dense_accepting_sets(pkg, acc_p):
     compare(pkg, g)
     r = mapgen.random_graph(200_000, 1, 6, acc_p, seed=8, variant="plain")
     compare(pkg, r, pkg.MAP_FLAG_FRONTIER_START)
+
+
+@pytest.mark.parametrize("n,layers,plant", [(2_000_003, 100, True), (3_000_000, 30, True), (2_500_000, 9, False)])
+def test_floods(pkg, n, layers, plant):
+    """Lists of a large share of the whole graph: into scan mode and back, in one iteration and in several."""
+    g = mapgen.layered_graph(n, layers, seed=n, plant=plant, acc_p=0.01 if plant else 0.3)
+    compare(pkg, g, pkg.MAP_FLAG_FRONTIER_START, runs=1)
+    want = oracle.run_graph(g)
+    h = pkg.map_create(g.n, g.rowptr, g.colidx, pkg.pack_bits(g.acc))
+    try:  # stopped inside and outside of scan mode, then whole
+        for k in (1, 2, 4, 6, 9, 12, 20):
+            if k < want.rounds[0]:
+                r = pkg.map_run(h, flags=pkg.MAP_FLAG_FRONTIER_START, max_inner=k, allow_limit=True)
+                assert r.status == pkg.MAP_ERR_LIMIT and r.rounds == [k]
+        r = pkg.map_run(h, flags=pkg.MAP_FLAG_FRONTIER_START)
+        assert (r.verdict, r.outer, r.rounds, r.relaxations) == (want.verdict, want.outer, want.rounds, want.relaxations)
+    finally:
+        pkg.map_destroy(h)
+
+
+def test_batch_flood(pkg):
+    gs = [mapgen.layered_graph(n, max(8, n // 16777), seed=n, plant=bool(i % 2))
+          for i, n in enumerate([900_000, 800_000, 300_000, 50_000, 7000, 400_001])]
+    h = pkg.map_batch_create([(g.n, g.rowptr, g.colidx, pkg.pack_bits(g.acc)) for g in gs])
+    try:
+        for sched in (0, 1):
+            out = np.empty(sum(g.n for g in gs), np.uint32)
+            rs = pkg.map_batch_run(h, len(gs), sched=sched, flags=pkg.MAP_FLAG_FRONTIER_START, map_out=out)
+            off = 0
+            for g, r in zip(gs, rs):
+                want = oracle.run_graph(g)
+                assert (r.verdict, r.witness, r.outer) == (want.verdict, want.witness, want.outer)
+                assert np.array_equal(out[off:off + g.n], want.map)
+                if sched == 0:
+                    assert (r.rounds, r.relaxations) == (want.rounds, want.relaxations)
+                off += g.n
+    finally:
+        pkg.map_destroy(h)
