@@ -1503,7 +1503,7 @@ __global__ void __launch_bounds__(TT, 1) k_tail(const __grid_constant__ RunArgs 
 // -------------------------------------------------------- medium graphs --
 //
 // k_own: the same run over the grid for a whole graph, or the compact graph k_run leaves, of at most OWN_N
-// vertices per SM.  Block b owns a contiguous share of the vertices and keeps their reader ranges, own offers
+// vertices per SM.  Block b owns every gridDim.x-th piece of 32 vertices and keeps their reader ranges, own offers
 // and last values in shared memory, and their reader lists too where they fit.  A push is a maximum
 // on the reader's word in global memory that nothing waits for; every round the owner reads its share's
 // words (coalesced) and pushes for those that changed.  So a round is one coalesced read, the reader ids,
@@ -1549,8 +1549,13 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
     const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     const bool lead = blockIdx.x == 0 && tid == 0;
     const uint32_t n = a.n, V = whole ? n : *(volatile uint32_t *)&c->V;
-    const uint32_t share = (V + gridDim.x - 1) / gridDim.x, v0 = min(V, blockIdx.x * share), mine = min(V, v0 + share) - v0;
-    const uint32_t stride = (share + 3) & ~3u;
+    // pieces of 32 vertices go round the blocks (a wave through consecutive vertices is everybody's): the block's
+    // vertex i is vertex vid(i)
+    const uint32_t pieces = (V + 31) / 32, nb = gridDim.x, full = (pieces + nb - 1) / nb * 32;
+    const auto vid = [&](uint32_t i) { return ((i >> 5) * nb + blockIdx.x) * 32 + (i & 31u); };
+    const uint32_t my_pieces = pieces > blockIdx.x ? (pieces - blockIdx.x + nb - 1) / nb : 0u;
+    const uint32_t mine = my_pieces == 0 ? 0u : my_pieces * 32 - ((pieces - 1) % nb == blockIdx.x ? pieces * 32 - V : 0u);
+    const uint32_t stride = full;
     uint32_t *const last = s_mem, *const own = last + stride, *const beg = own + stride, *const end = beg + stride;
     uint16_t *const queue = reinterpret_cast<uint16_t *>(end + stride);
     uint32_t *const s_rc = end + stride + stride / 2;
@@ -1579,7 +1584,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
         const uint32_t i = i0 + tid;
         uint32_t b = 0, e = 0;
         if (i < mine) {
-            const uint32_t v = v0 + i;
+            const uint32_t v = vid(i);
             uint32_t o;
             if (whole) {
                 b = __ldg(a.rrowptr + v);
@@ -1652,13 +1657,13 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
                 if (tid == 0) sh.n = sh.hubs = 0;
                 __syncthreads();
                 const bool start = r == 1 && pass == 0;
-                const uint32_t *const words = (SYNC ? inbox : val) + v0;
+                const uint32_t *const words = SYNC ? inbox : val;
                 for (uint32_t i0 = 0; i0 < mine; i0 += TT * OWN_U) { // (block-uniform) OWN_U words in flight per thread
                     uint32_t y[OWN_U];
 #pragma unroll
                     for (int k = 0; k < OWN_U; ++k) {
                         const uint32_t i = i0 + k * TT + tid;
-                        y[k] = i >= mine ? 0u : start ? own[i] : __ldcg(words + i);
+                        y[k] = i >= mine ? 0u : start ? own[i] : __ldcg(words + vid(i));
                     }
 #pragma unroll
                     for (int k = 0; k < OWN_U; ++k) {
@@ -1669,9 +1674,9 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
                         bool hit = y[k] != 0;
                         if (!start) {
                             if (SYNC) {
-                                if (i < mine) inbox[v0 + i] = 0; // (whole lines)
+                                if (i < mine) inbox[vid(i)] = 0; // (whole lines)
                                 if (hit && r > 2) {              // a frontier row of round r - 1
-                                    const uint32_t v = v0 + i;
+                                    const uint32_t v = vid(i);
                                     relax += whole ? __ldg(a.rowptr + v + 1) - __ldg(a.rowptr + v) : __ldg(row + v);
                                     ++frows;
                                 }
@@ -1760,7 +1765,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
             const uint32_t i = i0 + tid, x = i < mine ? last[i] : 0u;
             if (x) {
                 ++have;
-                if (x - 1 == (whole ? v0 + i : __ldg(&meta[v0 + i].w))) wit = min(wit, x - 1);
+                if (x - 1 == (whole ? vid(i) : __ldg(&meta[vid(i)].w))) wit = min(wit, x - 1);
             }
             const unsigned same = __match_any_sync(0xFFFFFFFFu, x); // (many vertices share a few values)
             if (x && x != settled && lane == (unsigned)(__ffs(same) - 1)) {
@@ -1828,7 +1833,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
                 o = own[i];
                 if (o && !((__ldcg(a.acc + ((o - 1) >> 5)) >> ((o - 1) & 31u)) & 1u)) own[i] = o = 0;
                 len = end[i] - beg[i];
-                if (!SYNC && x) val[v0 + i] = 0; // (the next iteration's pushes go to the other array)
+                if (!SYNC && x) val[vid(i)] = 0; // (the next iteration's pushes go to the other array)
                 last[i] = 0;
             }
             if (!pack) continue;
@@ -1844,7 +1849,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
             const uint32_t xb = sh.xbase, eb = sh.ebase;
             if ((uint64_t)xb + nm > lim || (uint64_t)eb + ne > ecap) over = true;
             if (member && !over) {
-                const uint32_t v = v0 + i, id = whole ? v : __ldg(&meta[v].w), k = xb + at;
+                const uint32_t v = vid(i), id = whole ? v : __ldg(&meta[v].w), k = xb + at;
                 meta2[k] = make_uint4(eb + ea, eb + ea + len, o, id);
                 if (SYNC) row2[k] = whole ? __ldg(a.rowptr + v + 1) - __ldg(a.rowptr + v) : __ldg(row + v);
                 a.rank[id] = k + 1;
@@ -1898,18 +1903,18 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
         for (uint32_t i = tid; i < mine; i += TT) {
             uint32_t x = last[i];
             if (SYNC) {
-                if (status != ST_OK) in0[v0 + i] = in1[v0 + i] = 0; // (at the fix-point the inboxes are empty)
+                if (status != ST_OK) in0[vid(i)] = in1[vid(i)] = 0; // (at the fix-point the inboxes are empty)
             } else {
-                if (status != ST_OK) x = max(x, __ldcg(val + v0 + i));
-                if (x) val[v0 + i] = 0;
+                if (status != ST_OK) x = max(x, __ldcg(val + vid(i)));
+                if (x) val[vid(i)] = 0;
             }
             if (a.out) {
-                if (whole) a.out[v0 + i] = x - 1u; // (no value: MAP_NONE)
-                else if (x) a.out[__ldg(&meta[v0 + i].w)] = x - 1u;
+                if (whole) a.out[vid(i)] = x - 1u; // (no value: MAP_NONE)
+                else if (x) a.out[__ldg(&meta[vid(i)].w)] = x - 1u;
             }
         }
     } else if (hand && whole && a.out) { // k_tail writes the values of the last iteration over this
-        for (uint32_t i = tid; i < mine; i += TT) a.out[v0 + i] = NONE;
+        for (uint32_t i = tid; i < mine; i += TT) a.out[vid(i)] = NONE;
     }
     for (int q = 0; q < 2; ++q) {
         const unsigned long long s = warp_sum64(q ? frows : relax);
