@@ -286,7 +286,8 @@ bool own_fits()
     }
     if (const int k = known[dev].load()) return k == 2;
     bool ok = true;
-    for (const void *f : {(const void *)mapk::k_own<true>, (const void *)mapk::k_own<false>}) {
+    for (const void *f : {(const void *)mapk::k_own<true, false>, (const void *)mapk::k_own<false, false>,
+                          (const void *)mapk::k_own<true, true>, (const void *)mapk::k_own<false, true>}) {
         int o = 0;
         ok = ok && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mapk::OWN_SMEM) == cudaSuccess &&
              cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, f, mapk::TT, mapk::OWN_SMEM) == cudaSuccess && o >= 1;
@@ -945,8 +946,8 @@ static uint32_t tail_cap()
 }
 static bool runs_in_tail(const map_graph *g) { return !g->comp && g->n <= tail_cap(); }
 
-// single graphs that fit into the shared memory of the SMs a run may fill (k_own)
-static uint32_t own_blocks(const map_graph *g) { return g->comp || !own_fits() ? 0u : (uint32_t)(g->sm_share ? g->sm_share : g->sms); }
+// graphs that fit into the shared memory of the SMs a run may fill (k_own)
+static uint32_t own_blocks(const map_graph *g) { return !own_fits() ? 0u : (uint32_t)(g->sm_share ? g->sm_share : g->sms); }
 static bool runs_in_own(const map_graph *g) { return !runs_in_tail(g) && g->n <= (uint64_t)own_blocks(g) * mapk::OWN_N; }
 
 // Which start a run takes when neither its flags nor map_autotune say: the frontier start pushes
@@ -1087,7 +1088,7 @@ static int launch_run(map_graph *g, cudaStream_t s, const map_opts &opts, const 
     const int cluster = g->comp ? 0 : tail_blocks();
     const bool whole = runs_in_tail(g);
     if (whole) return launch_tail(a, sync_sched, true, tail_blocks_for(g->n, cluster), s);
-    a.tail_cap = tail_cap();
+    a.tail_cap = g->comp ? 0u : tail_cap(); // (k_tail takes single graphs)
     const uint32_t own = own_blocks(g);
     a.own_cap = own * mapk::OWN_N;
     CK(cudaMemsetAsync(g->run_ctl, 0, sizeof(mapk::RunCtl), s));
@@ -1116,8 +1117,11 @@ static int launch_run(map_graph *g, cudaStream_t s, const map_opts &opts, const 
         cfg.gridDim = dim3(own);
         cfg.blockDim = dim3(mapk::TT);
         cfg.dynamicSmemBytes = mapk::OWN_SMEM;
-        if (sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_own<true>, a, in_own ? 1u : 0u));
-        else CK(cudaLaunchKernelEx(&cfg, mapk::k_own<false>, a, in_own ? 1u : 0u));
+        const uint32_t w = in_own ? 1u : 0u;
+        if (g->comp && sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_own<true, true>, a, w));
+        else if (g->comp) CK(cudaLaunchKernelEx(&cfg, mapk::k_own<false, true>, a, w));
+        else if (sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_own<true, false>, a, w));
+        else CK(cudaLaunchKernelEx(&cfg, mapk::k_own<false, false>, a, w));
     }
     return cluster ? launch_tail(a, sync_sched, false, (uint32_t)cluster, s) : MAP_OK;
 }

@@ -676,6 +676,43 @@ __device__ __forceinline__ bool comp_goes_on(const volatile CompState &S, uint32
     return !limit;
 }
 
+// one block (every thread of it): the end of an outer iteration for every graph of a batch; the number that
+// go on.  s: a shared word.
+__device__ __forceinline__ uint32_t end_graphs(const RunArgs &a, uint32_t status, uint32_t *s)
+{
+    unsigned on = 0;
+    for (uint32_t g = threadIdx.x; g < a.ncomp; g += blockDim.x) {
+        volatile CompState &S = a.cs[g];
+        if (!S.active) continue;
+        const uint32_t it = S.outer, rounds = S.last_change + 1;
+        if (it - 1 < CH_CAP) a.chist[(size_t)g * CH_CAP + it - 1] = rounds;
+        S.inner_total = S.inner_total + rounds;
+        S.relax = S.relax + S.m; // round 1 covers every row
+        uint32_t left;
+        bool limit;
+        const bool more = comp_goes_on(S, status, a.max_outer, left, limit);
+        if (status != ST_OK) S.status = status;
+        else if (limit) S.status = ST_LIMIT;
+        if (status == ST_OK && S.witness != NONE) S.verdict = 1;
+        else S.nacc = left;
+        if (more) {
+            S.outer = it + 1;
+            S.witness = NONE;
+            S.elim = S.touched = S.last_change = 0;
+            ++on;
+        } else {
+            S.active = 0;
+        }
+    }
+    on = __reduce_add_sync(0xFFFFFFFFu, on);
+    __syncthreads();
+    if (threadIdx.x == 0) *s = 0;
+    __syncthreads();
+    if (lane_id() == 0 && on) atomicAdd(s, on);
+    __syncthreads();
+    return *s;
+}
+
 template <bool SYNC, bool BATCH>
 __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_constant__ RunArgs a)
 {
@@ -894,37 +931,7 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
             nacc -= (uint32_t)(total & RUN_COUNT);
             alive = run_barrier(c, c->bar, sh, run.seq, 0, total);
             if (!alive) break;
-            unsigned on = 0;
-            if (blockIdx.x == 0) {
-                for (uint32_t g = threadIdx.x; g < a.ncomp; g += RT) {
-                    volatile CompState &S = a.cs[g];
-                    if (!S.active) continue;
-                    const uint32_t it = S.outer, rounds = S.last_change + 1;
-                    if (it - 1 < CH_CAP) a.chist[(size_t)g * CH_CAP + it - 1] = rounds;
-                    S.inner_total = S.inner_total + rounds;
-                    S.relax = S.relax + S.m; // round 1 covers every row
-                    const bool more = comp_goes_on(S, status, a.max_outer, left, limit);
-                    if (status != ST_OK) S.status = status;
-                    else if (limit) S.status = ST_LIMIT;
-                    if (status == ST_OK && S.witness != NONE) S.verdict = 1;
-                    else S.nacc = left;
-                    if (more) {
-                        S.outer = it + 1;
-                        S.witness = NONE;
-                        S.elim = S.touched = S.last_change = 0;
-                        ++on;
-                    } else {
-                        S.active = 0;
-                    }
-                }
-                on = __reduce_add_sync(0xFFFFFFFFu, on);
-                __syncthreads();
-                if (threadIdx.x == 0) sh.ln = 0;
-                __syncthreads();
-                if (lane_id() == 0 && on) atomicAdd(&sh.ln, on);
-                __syncthreads();
-                on = sh.ln;
-            }
+            const uint32_t on = blockIdx.x == 0 ? end_graphs(a, status, &sh.ln) : 0u;
             alive = run_barrier(c, c->bar, sh, run.seq, on, total);
             if (!alive) break;
             go = (total & RUN_COUNT) != 0;
@@ -1007,7 +1014,7 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
                 uint32_t *const t = alist;
                 alist = la;
                 la = t;
-                if (!BATCH && V2 <= max(a.tail_cap, a.own_cap)) { // small enough for one of the kernels below
+                if (V2 <= max(a.tail_cap, a.own_cap)) { // small enough for one of the kernels below
                     hand = true;
                     break;
                 }
@@ -1539,7 +1546,7 @@ __device__ __forceinline__ uint32_t own_scan(uint32_t x, uint32_t *s, uint32_t &
     return incl - x + (warp ? s[warp - 1] : 0u);
 }
 
-template <bool SYNC>
+template <bool SYNC, bool BATCH>
 __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a, uint32_t whole)
 {
     extern __shared__ uint32_t s_mem[];
@@ -1566,6 +1573,10 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
     const uint4 *meta = reinterpret_cast<const uint4 *>(ps);
     const uint32_t *row = ps + 4ull * cap, *rc = whole ? a.rcol : ps + 6ull * cap;
     uint32_t *const in0 = reinterpret_cast<uint32_t *>(a.W), *const in1 = in0 + n;
+    // batched, asynchronous: the last round each row was reached in (its graph's relaxation count)
+    constexpr bool REACH = BATCH && !SYNC;
+    uint32_t *const reach = in1 + n;
+    const uint32_t *const comp = whole ? a.comp : row + cap; // batched: graph of each vertex
     const uint64_t t0 = whole ? global_ns() : *(volatile unsigned long long *)&c->t0;
     uint64_t mark = global_ns(), ph_rounds = 0, ph_check = 0;
     auto phase = [&](uint64_t &acc) {
@@ -1633,6 +1644,8 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
     if (whole) { // the run's accepting set, and an empty map
         const uint64_t gid = (uint64_t)blockIdx.x * TT + tid, threads = (uint64_t)gridDim.x * TT;
         for (uint64_t i = gid; i < a.words; i += threads) a.acc[i] = __ldg(a.acc0 + i);
+        if (BATCH && a.out) // (graphs end in different iterations)
+            for (uint64_t i = gid; i < n; i += threads) a.out[i] = NONE;
     }
     if (tid == 0) sh.late = 0;
     __syncthreads();
@@ -1641,6 +1654,21 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
     uint32_t status = ST_OK, verdict = 0, witness = NONE, seq = 0, gate = a.tail_cap / 2;
     unsigned long long relax = 0, frows = 0, inner_total = 0, total = 0;
     bool go = nacc != 0, alive = true, hand = false;
+    // a frontier row of n entries: to the relaxation count (batched: of its graph g); the whole warp calls it
+    const auto count_row = [&](bool is, uint32_t len, uint32_t g) {
+        if (is) {
+            relax += len;
+            ++frows;
+        }
+        if constexpr (BATCH) {
+            const uint32_t k = is ? g : NONE, l = is ? len : 0u;
+            const unsigned same = __match_any_sync(0xFFFFFFFFu, k);
+            const unsigned lo = __reduce_add_sync(same, l & 0xFFFFu), hi = __reduce_add_sync(same, l >> 16);
+            const unsigned long long sum = (unsigned long long)lo + ((unsigned long long)hi << 16);
+            if (k != NONE && lane == (unsigned)(__ffs(same) - 1) && sum)
+                atomicAdd((unsigned long long *)&a.cs[k].relax, sum);
+        }
+    };
     const auto reader = [&](uint32_t j) { return cached ? s_rc[j] : __ldg(rc + j); };
     while (go) {
         ++outer;
@@ -1651,6 +1679,10 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
             ++r;
             uint32_t *const inbox = (r & 1) ? in0 : in1; // what came in round r - 1 (synchronous)
             uint32_t *const to = SYNC ? ((r & 1) ? in1 : in0) : val;
+            const auto push = [&](uint32_t w, uint32_t o) {
+                atomicMax(to + w, o);
+                if (REACH) atomicMax(reach + w, r);
+            };
             const bool pushes = r <= a.max_inner; // (past the limit the last round's values are only taken)
             uint32_t hits = 0;
             for (uint32_t pass = 0;; ++pass) { // (asynchronous: the share once more, lc_passes times while it changes)
@@ -1659,11 +1691,12 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
                 const bool start = r == 1 && pass == 0;
                 const uint32_t *const words = SYNC ? inbox : val;
                 for (uint32_t i0 = 0; i0 < mine; i0 += TT * OWN_U) { // (block-uniform) OWN_U words in flight per thread
-                    uint32_t y[OWN_U];
+                    uint32_t y[OWN_U], f[OWN_U];
 #pragma unroll
                     for (int k = 0; k < OWN_U; ++k) {
                         const uint32_t i = i0 + k * TT + tid;
                         y[k] = i >= mine ? 0u : start ? own[i] : __ldcg(words + vid(i));
+                        if (REACH) f[k] = i >= mine || pass || r <= 2 ? 0u : __ldcg(reach + vid(i));
                     }
 #pragma unroll
                     for (int k = 0; k < OWN_U; ++k) {
@@ -1673,16 +1706,22 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
                         if (!some) continue; // (warp-uniform: nothing here)
                         bool hit = y[k] != 0;
                         if (!start) {
-                            if (SYNC) {
-                                if (i < mine) inbox[vid(i)] = 0; // (whole lines)
-                                if (hit && r > 2) {              // a frontier row of round r - 1
-                                    const uint32_t v = vid(i);
-                                    relax += whole ? __ldg(a.rowptr + v + 1) - __ldg(a.rowptr + v) : __ldg(row + v);
-                                    ++frows;
-                                }
+                            const uint32_t v = vid(i), g = BATCH && hit ? __ldg(comp + v) : NONE;
+                            if (SYNC && i < mine) inbox[v] = 0; // (whole lines)
+                            if ((SYNC || REACH) && r > 2) { // frontier rows of round r - 1
+                                const bool is = SYNC ? hit : f[k] == r - 1;
+                                uint32_t len = 0;
+                                if (is) len = whole ? __ldg(a.rowptr + v + 1) - __ldg(a.rowptr + v) : __ldg(row + v);
+                                count_row(is, len, g);
                             }
                             hit = hit && y[k] > last[i];
                             if (hit) last[i] = y[k];
+                            if constexpr (BATCH) { // the graphs that changed in round r - 1 (a later pass: in this one)
+                                const unsigned same = __match_any_sync(0xFFFFFFFFu, hit ? g : NONE);
+                                const uint32_t at = pass ? r : r - 1;
+                                if (hit && lane == (unsigned)(__ffs(same) - 1) && *(volatile uint32_t *)&a.cs[g].last_change < at)
+                                    atomicMax(&a.cs[g].last_change, at);
+                            }
                         }
                         const unsigned m = __ballot_sync(0xFFFFFFFFu, hit);
                         if (!m) continue;
@@ -1704,7 +1743,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
                         o = start ? own[i] : max(last[i], own[i]);
                         b = beg[i];
                         e = end[i];
-                        if (!SYNC) {
+                        if (!SYNC && !BATCH) {
                             if (r > 1 || pass || a.count_round1) relax += e - b;
                             if (r > 1) ++frows;
                         }
@@ -1721,7 +1760,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
                         const uint32_t ob = __shfl_sync(0xFFFFFFFFu, o, src), bb = __shfl_sync(0xFFFFFFFFu, b, src),
                                        ll = __shfl_sync(0xFFFFFFFFu, e - b, src);
 #pragma unroll 4
-                        for (uint32_t j = lane; j < ll; j += 32) atomicMax(to + reader(bb + j), ob);
+                        for (uint32_t j = lane; j < ll; j += 32) push(reader(bb + j), ob);
                         if ((int)lane == src) b = e;
                     }
                     for (uint32_t j = 0; j < e - b; j += 4) { // up to four readers in flight
@@ -1730,7 +1769,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
                         for (int k = 0; k < 4; ++k) w[k] = j + k < e - b ? reader(b + j + k) : NONE;
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
-                            if (w[k] != NONE) atomicMax(to + w[k], o);
+                            if (w[k] != NONE) push(w[k], o);
                     }
                 }
                 __syncthreads();
@@ -1738,10 +1777,10 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
                     const uint32_t i = sh.hub[h], b = beg[i], ll = end[i] - b;
                     const uint32_t o = start ? own[i] : max(last[i], own[i]);
 #pragma unroll 4
-                    for (uint32_t j = tid; j < ll; j += TT) atomicMax(to + reader(b + j), o);
+                    for (uint32_t j = tid; j < ll; j += TT) push(reader(b + j), o);
                 }
                 __syncthreads(); // (the queue and the hubs are read)
-                if (SYNC || pass >= a.lc_passes) break;
+                if (SYNC || BATCH || pass >= a.lc_passes) break;
             }
             alive = run_barrier(c, c->obar, sh, seq, (unsigned long long)hits + ((r & 3u) == 0 && late() ? RUN_STOP : 0ull), total);
             if (!alive) break;
@@ -1758,21 +1797,35 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
             if (outer - 1 < RUN_HIST) a.res->hist[outer - 1] = rounds;
             phase(ph_rounds);
         }
-        if (status != ST_OK) break;
+        if (!BATCH && status != ST_OK) break;
         // ---- self-map test and elimination (last[] holds the values)
         uint32_t wit = NONE, elim = 0, have = 0, settled = 0;
         for (uint32_t i0 = 0; i0 < mine; i0 += TT) {
             const uint32_t i = i0 + tid, x = i < mine ? last[i] : 0u;
+            const uint32_t g = BATCH && x ? __ldg(comp + vid(i)) : NONE;
+            uint32_t removed = 0;
             if (x) {
                 ++have;
-                if (x - 1 == (whole ? vid(i) : __ldg(&meta[vid(i)].w))) wit = min(wit, x - 1);
+                if (status == ST_OK && x - 1 == (whole ? vid(i) : __ldg(&meta[vid(i)].w))) {
+                    wit = min(wit, x - 1);
+                    if (BATCH) atomicMin(&a.cs[g].witness, x - 1);
+                }
             }
             const unsigned same = __match_any_sync(0xFFFFFFFFu, x); // (many vertices share a few values)
-            if (x && x != settled && lane == (unsigned)(__ffs(same) - 1)) {
+            if (x && x != settled && status == ST_OK && lane == (unsigned)(__ffs(same) - 1)) {
                 const uint32_t u = x - 1, bit = 1u << (u & 31u);
-                if ((__ldcg(a.acc + (u >> 5)) & bit) && (atomicAnd(a.acc + (u >> 5), ~bit) & bit)) ++elim;
+                if ((__ldcg(a.acc + (u >> 5)) & bit) && (atomicAnd(a.acc + (u >> 5), ~bit) & bit)) removed = 1;
             }
+            elim += removed;
             settled = x;
+            if constexpr (BATCH) { // per graph: vertices with a value and removals, one atomic per graph in the warp
+                const unsigned like = __match_any_sync(0xFFFFFFFFu, g);
+                const unsigned ne = __reduce_add_sync(like, removed);
+                if (g != NONE && lane == (unsigned)(__ffs(like) - 1)) {
+                    atomicAdd(&a.cs[g].touched, (unsigned)__popc(like));
+                    if (ne) atomicAdd(&a.cs[g].elim, ne);
+                }
+            }
         }
         wit = __reduce_min_sync(0xFFFFFFFFu, wit);
         elim = __reduce_add_sync(0xFFFFFFFFu, elim);
@@ -1798,7 +1851,22 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
         if (!alive) break;
         const uint32_t T = *(volatile uint32_t *)&c->ocnt[outer & 1].v;
         if (lead) phase(ph_check);
-        if (total & (RUN_STOP - RUN_FOUND)) {
+        if constexpr (BATCH) {
+            if (status == ST_OK && (total & RUN_STOP)) status = ST_TIMEOUT;
+            uint32_t left;
+            bool limit;
+            for (uint32_t i = tid; a.out && i < mine; i += TT) { // the maps of the graphs that end here
+                const uint32_t x = last[i], v = vid(i);
+                if (!x) continue;
+                const uint32_t g = __ldg(comp + v);
+                if (!comp_goes_on(a.cs[g], status, a.max_outer, left, limit))
+                    a.out[whole ? v : __ldg(&meta[v].w)] = x - 1u - *(volatile uint32_t *)&a.cs[g].off;
+            }
+            if (!(alive = run_barrier(c, c->obar, sh, seq, 0, total))) break;
+            const uint32_t on = blockIdx.x == 0 ? end_graphs(a, status, sh.sums) : 0u;
+            if (!(alive = run_barrier(c, c->obar, sh, seq, on, total))) break;
+            if (!(total & RUN_COUNT)) go = false;
+        } else if (total & (RUN_STOP - RUN_FOUND)) {
             verdict = 1;
             witness = NONE - *(volatile uint32_t *)&c->witness.v;
             go = false;
@@ -1817,7 +1885,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
         }
         if (!go) break;
         // ---- the next iteration: eliminated vertices offer nothing, values back to none
-        const bool pack = T <= gate;
+        const bool pack = !BATCH && T <= gate;
         uint32_t V2 = 0, E2 = 0;
         const uint32_t lim = min(a.tail_cap, cap);
         const uint64_t ecap = (uint64_t)n * 3 / 4 - 8;
@@ -1831,9 +1899,12 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
             if (i < mine) {
                 x = last[i];
                 o = own[i];
-                if (o && !((__ldcg(a.acc + ((o - 1) >> 5)) >> ((o - 1) & 31u)) & 1u)) own[i] = o = 0;
+                if (o && (!((__ldcg(a.acc + ((o - 1) >> 5)) >> ((o - 1) & 31u)) & 1u) ||
+                          (BATCH && !*(volatile uint32_t *)&a.cs[__ldg(comp + vid(i))].active)))
+                    own[i] = o = 0;
                 len = end[i] - beg[i];
                 if (!SYNC && x) val[vid(i)] = 0; // (the next iteration's pushes go to the other array)
+                if (REACH && x) reach[vid(i)] = 0;
                 last[i] = 0;
             }
             if (!pack) continue;
@@ -1907,8 +1978,9 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
             } else {
                 if (status != ST_OK) x = max(x, __ldcg(val + vid(i)));
                 if (x) val[vid(i)] = 0;
+                if (REACH && x) reach[vid(i)] = 0;
             }
-            if (a.out) {
+            if (!BATCH && a.out) {
                 if (whole) a.out[vid(i)] = x - 1u; // (no value: MAP_NONE)
                 else if (x) a.out[__ldg(&meta[vid(i)].w)] = x - 1u;
             }
