@@ -1181,6 +1181,10 @@ constexpr size_t TAIL_SMEM = (size_t)TAIL_N * 26;
 // graphs up to here run in the cluster, larger ones over the grid (k_own).  Layered graphs, synchronous, us per
 // run with k_tail / k_own: 16,000 vertices 166 / 205, 30,000 262 / 235, 60,000 317 / 238, 130,000 470 / 263
 constexpr uint32_t TAIL_BEST = 16384;
+// asynchronous, a vertex per thread: looks at the vertex per round, so that values that came in meanwhile go on
+// before the barrier (10^6 layered, us per run with 1 / 2 / 4 / 6 / 8 looks: 900 / 844 / 777 / 764 / 751; 4,000 random
+// 80 / - / 71 / 77 / 77; 16,000 layered 163 / - / 148 / 154 / 164)
+constexpr int TAIL_PASSES = 4;
 constexpr uint32_t TAIL_LONG = 16;   // reader lists longer than this are walked by a whole warp
 
 __device__ __forceinline__ uint32_t cluster_rank()
@@ -1293,9 +1297,10 @@ __global__ void __launch_bounds__(TT, 1) k_tail(const __grid_constant__ RunArgs 
             const uint32_t to = shared_addr(SYNC ? ((r & 1) ? x1 : x0) : val);
             const bool pushes = r <= a.max_inner; // (past the limit the last round's values are only taken)
             bool any = false;
-            // did vertex i change in round r - 1 (round 1: is it accepting)?  o: what it offers then
+            // did vertex i change in round r - 1 (start: is it accepting)?  o: what it offers then
+            bool start = r == 1;
             auto changed = [&](uint32_t i, uint32_t &o) {
-                if (r == 1) {
+                if (start) {
                     o = own[i];
                     return o != 0;
                 }
@@ -1346,13 +1351,16 @@ __global__ void __launch_bounds__(TT, 1) k_tail(const __grid_constant__ RunArgs 
                 }
             };
             if (mine <= TT) { // a vertex per thread
-                uint32_t o = 0, b = 0, e = 0;
-                if (tid < mine && changed(tid, o)) {
-                    any = true;
-                    b = beg[tid];
-                    e = pushes ? end[tid] : b;
+                for (int pass = 0; pass < (SYNC ? 1 : TAIL_PASSES); ++pass) {
+                    uint32_t o = 0, b = 0, e = 0;
+                    if (tid < mine && changed(tid, o)) {
+                        any = true;
+                        b = beg[tid];
+                        e = pushes ? end[tid] : b;
+                    }
+                    send(o, b, e);
+                    start = false;
                 }
-                send(o, b, e);
             } else { // several: the changed ones are queued first, so that their lists are read side by side
                 if (tid == 0) s_n = 0;
                 __syncthreads();
@@ -1375,7 +1383,7 @@ __global__ void __launch_bounds__(TT, 1) k_tail(const __grid_constant__ RunArgs 
                     if (q < nq) {
                         const uint32_t i = queue[q];
                         // (synchronous: the value just taken; asynchronous: the live one)
-                        o = r == 1 ? own[i] : max(*(volatile uint32_t *)(val + i), own[i]);
+                        o = start ? own[i] : max(*(volatile uint32_t *)(val + i), own[i]);
                         b = beg[i];
                         e = end[i];
                     }
