@@ -335,6 +335,7 @@ struct map_graph {
     int check_grid = 0;  // blocks of the self-map / elimination kernel
     int occ_dense = 1, occ_rounds = 1; // resident blocks per SM of the dense-round and fix-point kernels
     cudaStream_t stream = nullptr;
+    void *arena = nullptr; // one allocation that holds every array of fixed size below
     uint32_t *rowptr = nullptr, *colidx = nullptr, *rrowptr = nullptr, *rcol = nullptr;
     uint32_t *rpos = nullptr; // positions in colidx of the reader entries
     // (set-up only) caller arrays the ingest pass reads and copies into rowptr / colidx itself,
@@ -382,7 +383,7 @@ struct map_graph {
     bool tuned_fstart = false; // map_autotune found the frontier start faster on this graph
     bool fstart_push = false;  // ... and, with it, rounds that only push
     uint64_t acc_entries = 0;  // entries that hold an accepting vertex
-    mapk::RunCtl *run_ctl = nullptr; // control block of whole-run launches, and the result behind it (first use)
+    mapk::RunCtl *run_ctl = nullptr; // control block of whole-run launches, and the result behind it
     bool pull_on = false;     // the launches being issued may pull (the fix-point kernel's pull variant)
     bool functional = false;  // every row holds at most one entry (set-up): pointer doubling applies
     bool func_on = false;     // the launches being issued propagate by pointer doubling (k_func)
@@ -403,16 +404,11 @@ void free_graph(map_graph *g)
         if (g->exec[i]) cudaGraphExecDestroy(g->exec[i]);
         if (g->graph[i]) cudaGraphDestroy(g->graph[i]);
     }
-    void *dev[] = {g->rowptr, g->colidx, g->rrowptr, g->rcol,    g->rpos, g->elog, g->acc0, g->acc,
-                   g->mval,   g->list,   g->flist,   g->rec,     g->touched, g->xbuf, g->hist, g->ctl,
-                   g->alist};
-    for (void *p : dev)
-        if (p) cudaFreeAsync(p, g->stream); // stream-ordered: no device-wide synchronisation
-    if (g->run_ctl) cudaFreeAsync(g->run_ctl, g->stream);
+    // (stream-ordered: no device-wide synchronisation)
+    if (g->arena) cudaFreeAsync(g->arena, g->stream);
+    if (g->alist) cudaFreeAsync(g->alist, g->stream);
     if (g->comp) cudaFreeAsync(g->comp, g->stream);
     if (g->ids) cudaFreeAsync(g->ids, g->stream);
-    if (g->stale) cudaFreeAsync(g->stale, g->stream);
-    if (g->cbit) cudaFreeAsync(g->cbit, g->stream);
     if (g->cs) cudaFreeAsync(g->cs, g->stream);
     if (g->chist) cudaFreeAsync(g->chist, g->stream);
     free(g->h_cs);
@@ -758,26 +754,51 @@ int create_graph(uint32_t n, uint64_t m, cudaStream_t s, const char *who, Upload
     if (const char *e = getenv("MAPGPU_SOLO_MAX")) g->solo_max = (uint32_t)strtoul(e, nullptr, 10); // (default 256)
     if (const char *e = getenv("MAPGPU_LC_PASSES")) g->lc_passes = (uint32_t)strtoul(e, nullptr, 10); // (default 1)
 
-    auto alloc = [&](uint32_t **p, uint64_t words) -> int {
-        if (t_inject_alloc > 0 && --t_inject_alloc == 0)
-            return fail(MAP_ERR_OOM, "%s: injected device allocation failure (MAPGPU_INJECT_OOM)", who);
-        // stream-ordered allocation (does not synchronise the device; graphs on other
-        // streams keep running); 16 bytes of slack at the end
-        CK(cudaMallocAsync((void **)p, (words + 4) * sizeof(uint32_t), s));
-        return MAP_OK;
-    };
+    // Every array of fixed size in one stream-ordered allocation (it does not synchronise the device; graphs on
+    // other streams keep running): each at a 256-byte boundary with 16 bytes of slack behind it.  One call each
+    // took 17 of the 30 driver calls of a small graph's life, and a lock that every served job wants.  The
+    // arrays that start at zero are neighbours, cleared by one memset with colidx's slack in front of them.
     int rc = MAP_OK;
     const uint64_t W = g->words;
-    if ((rc = alloc(&g->rowptr, (uint64_t)n + 1)) || (rc = alloc(&g->colidx, m)) ||
-        (rc = alloc(&g->rrowptr, (uint64_t)n + 1)) || (rc = alloc(&g->rcol, m)) || (rc = alloc(&g->rpos, m)) ||
-        (rc = alloc(&g->elog, n)) || (rc = alloc(&g->acc0, W)) ||
-        (rc = alloc(&g->acc, W)) || (rc = alloc(&g->mval, n)) || (rc = alloc(&g->list, 3 * (uint64_t)n)) ||
-        (rc = alloc(&g->flist, 3 * (uint64_t)n)) || (rc = alloc((uint32_t **)&g->rec, 4 * (uint64_t)n)) ||
-        (rc = alloc(&g->touched, n)) || (rc = alloc(&g->xbuf, n)) || (rc = alloc(&g->stale, W)) ||
-        (rc = alloc(&g->cbit, 3 * (W + 4))) || (rc = alloc(&g->hist, g->hist_cap))) {
-        free_graph(g);
-        return rc;
-    }
+    struct Piece {
+        uint32_t **p;
+        uint64_t at;
+    };
+    Piece pieces[20];
+    size_t np = 0;
+    uint64_t total = 0;
+    const auto want = [&](uint32_t **p, uint64_t words) {
+        pieces[np++] = {p, total};
+        total += (words + 4 + 63) & ~uint64_t(63);
+    };
+    want(&g->rowptr, (uint64_t)n + 1);
+    want(&g->rcol, m);
+    want(&g->rpos, m);
+    want(&g->elog, n);
+    want(&g->acc0, W);
+    want(&g->acc, W);
+    want(&g->list, 3 * (uint64_t)n);
+    want(&g->flist, 3 * (uint64_t)n);
+    want(&g->touched, n);
+    want(&g->xbuf, n);
+    want(&g->hist, g->hist_cap);
+    want(&g->colidx, m);
+    // from here on: zero
+    want((uint32_t **)&g->ctl, (sizeof(Ctl) + 3) / 4);
+    want((uint32_t **)&g->run_ctl, (sizeof(mapk::RunCtl) + sizeof(mapk::RunRes) + 3) / 4);
+    want(&g->rrowptr, (uint64_t)n + 1);
+    want(&g->stale, W);
+    want(&g->cbit, 3 * (W + 4));
+    want(&g->mval, n);
+    want((uint32_t **)&g->rec, 4 * (uint64_t)n);
+    // (set-up only: each entry's place in its reader list; in the list space where that is large enough)
+    uint32_t *rank = nullptr;
+    const bool rank_in_lists = m <= 6 * (uint64_t)n;
+    for (size_t k = 0; k < np + 1; ++k) // (fault injection counts one allocation per array)
+        if (t_inject_alloc > 0 && --t_inject_alloc == 0) {
+            free_graph(g);
+            return fail(MAP_ERR_OOM, "%s: injected device allocation failure (MAPGPU_INJECT_OOM)", who);
+        }
     auto ck = [&](cudaError_t e, const char *what) -> int {
         if (e == cudaSuccess) return MAP_OK;
         cudaGetLastError();
@@ -793,53 +814,43 @@ int create_graph(uint32_t n, uint64_t m, cudaStream_t s, const char *who, Upload
     } else {
         g->h_ctl = static_cast<Ctl *>(aligned_alloc(128, sizeof(Ctl)));
     }
-    g->h_stage = static_cast<uint32_t *>(malloc((size_t)n * 4 + 16));
-    g->h_hist = static_cast<uint32_t *>(malloc((size_t)g->hist_cap * 4));
-    if (!g->h_ctl || !g->h_stage || !g->h_hist) {
+    if (!g->h_ctl) {
         free_graph(g);
         return fail(MAP_ERR_OOM, "%s: host allocation failed", who);
     }
-    if ((rc = ck(cudaMallocAsync((void **)&g->ctl, sizeof(Ctl), s), "ctl"))) {
+    if ((rc = ck(cudaMallocAsync(&g->arena, total * 4, s), "device memory"))) {
         free_graph(g);
         return rc;
     }
-    for (auto &e : g->ev)
-        if ((rc = ck(cudaEventCreate(&e), "event"))) {
+    for (size_t k = 0; k < np; ++k) *pieces[k].p = static_cast<uint32_t *>(g->arena) + pieces[k].at;
+    if (rank_in_lists) {
+        rank = g->list; // (list and flist: 6n words in a row)
+    } else if ((rc = ck(cudaMallocAsync((void **)&rank, (m + 4) * 4, s), "device memory"))) {
+        free_graph(g);
+        return rc;
+    }
+    const auto free_rank = [&]() {
+        if (!rank_in_lists) cudaFreeAsync(rank, s);
+    };
+    for (int e = 0; e < 2; ++e) // (the others on the first profiled run)
+        if ((rc = ck(cudaEventCreate(&g->ev[e]), "event"))) {
+            free_rank();
             free_graph(g);
             return rc;
         }
 
     // inputs into g->rowptr, g->colidx and an accepting bitmap (host or device sources)
     uint32_t *acc_in = nullptr;
-    if ((rc = ck(cudaMemsetAsync(g->ctl, 0, sizeof(Ctl), s), "memset ctl")) || (rc = upload(g, &acc_in))) {
-        free_graph(g);
-        return rc;
-    }
-    if ((rc = ck(cudaMemsetAsync(g->colidx + m, 0, 16, s), "pad")) ||
-        (rc = ck(cudaMemsetAsync(g->mval, 0, ((size_t)n + 4) * 4, s), "memset mval")) ||
-        (rc = ck(cudaMemsetAsync(g->rec, 0, (size_t)n * 16, s), "memset rec")) ||
-        (rc = ck(cudaMemsetAsync(g->stale, 0, ((size_t)W + 4) * 4, s), "memset stale")) ||
-        (rc = ck(cudaMemsetAsync(g->cbit, 0, 3 * ((size_t)W + 4) * 4, s), "memset cbit"))) {
+    const uint32_t *const zero_end = reinterpret_cast<uint32_t *>(g->rec) + 4 * (uint64_t)n;
+    if ((rc = ck(cudaMemsetAsync(g->colidx + m, 0, (size_t)(zero_end - (g->colidx + m)) * 4, s), "memset")) ||
+        (rc = upload(g, &acc_in))) {
+        free_rank();
         free_graph(g);
         return rc;
     }
     // the accepting set, then one pass over the CSR: validation, in-degree histogram of the reverse
     // CSR, and the accepting flag of each target into bit 31 of its entry (restored after every run)
-    if ((rc = ck(cudaMemsetAsync(g->rrowptr, 0, ((size_t)n + 1) * 4, s), "memset rrowptr"))) {
-        free_graph(g);
-        return rc;
-    }
     mapk::k_acc_init<<<grid_for(g, W, 1), 256, 0, s>>>(n, acc_in, g->acc0, &g->ctl->elim.v);
-    // (each entry's place in its reader list, kept for the scatter; freed at the end of set-up)
-    uint32_t *rank = nullptr;
-    if ((rc = alloc(&rank, m))) {
-        free_graph(g);
-        return rc;
-    }
-    const auto free_rank = [&]() {
-        cudaFreeAsync(rank, s);
-        rank = nullptr;
-    };
     mapk::k_ingest<<<grid_for(g, std::max<uint64_t>(m / 4, n), 1), 256, 0, s>>>(
         n, g->in_rowptr ? g->in_rowptr : g->rowptr, g->in_rowptr ? g->rowptr : nullptr, m,
         g->in_colidx ? g->in_colidx : g->colidx, g->colidx, g->acc0, g->rrowptr, rank, &g->ctl->bad,
@@ -1018,13 +1029,6 @@ static int take_result(const mapk::RunRes &R, const map_opts &opts, uint64_t m, 
     return MAP_OK;
 }
 
-// the control block of whole-run launches, allocated on first use
-static int ensure_run_ctl(map_graph *g)
-{
-    if (!g->run_ctl) CK(cudaMallocAsync((void **)&g->run_ctl, sizeof(mapk::RunCtl) + sizeof(mapk::RunRes), g->stream));
-    return MAP_OK;
-}
-
 // where a launch leaves its result: the handle's page-locked slot, or (without one) behind its control block
 static mapk::RunRes *run_result(const map_graph *g)
 {
@@ -1050,7 +1054,6 @@ static int launch_run(map_graph *g, cudaStream_t s, const map_opts &opts, const 
 {
     static const int occ = run_occupancy();
     const size_t n = g->n;
-    if (const int rc = ensure_run_ctl(g)) return rc;
     mapk::RunArgs a;
     memset(&a, 0, sizeof a);
     a.n = g->n;
@@ -1253,6 +1256,10 @@ static int run_impl(map_graph *g, const map_opts *opts_in, map_result *res, uint
         if ((rc = read_ctl(g))) return rc;
         res->launches = 0; // filled below from the counts
     } else {
+        if (opts.trace && !g->h_stage && !(g->h_stage = static_cast<uint32_t *>(malloc((size_t)n * 4 + 16))))
+            return fail(MAP_ERR_OOM, "map_run: host allocation failed");
+        for (int e = 2; profile && e < 8; ++e)
+            if (!g->ev[e]) CK(cudaEventCreate(&g->ev[e]));
         const mapk::Handles none{};
         *g->h_ctl = init;
         CK(cudaEventRecord(g->ev[0], s));
@@ -1338,6 +1345,8 @@ static int run_impl(map_graph *g, const map_opts *opts_in, map_result *res, uint
     res->launches = 3 + ((fstart ? 1ull : 2ull) + (stepped ? 1ull : 0ull)) * c.outer;
     const uint32_t nh = std::min<uint32_t>(c.outer, g->hist_cap);
     if (opts.rounds_out && nh) {
+        if (!g->h_hist && !(g->h_hist = static_cast<uint32_t *>(malloc((size_t)g->hist_cap * 4))))
+            return fail(MAP_ERR_OOM, "map_run: host allocation failed");
         CK(cudaMemcpyAsync(g->h_hist, g->hist, (size_t)nh * 4, cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
         memcpy(opts.rounds_out, g->h_hist, (size_t)std::min(nh, opts.rounds_cap) * 4);
@@ -1547,8 +1556,7 @@ int map_lasso(map_graph *g, uint32_t init, uint32_t witness, uint32_t *path, uin
     *prefix_len = *cycle_len = 0;
     cudaStream_t s = g->stream;
     const size_t n = g->n;
-    int rc = ensure_run_ctl(g);
-    if (rc) return rc;
+    int rc = MAP_OK;
     mapk::LassoArgs a;
     a.n = g->n;
     a.rowptr = g->rowptr;
