@@ -234,7 +234,8 @@ int tail_blocks()
     if (const int k = known[dev].load()) return k - 1;
     int best = 0;
     const void *const both[] = {(const void *)mapk::k_tail<true>, (const void *)mapk::k_tail<false>};
-    bool ok = cudaFuncSetAttribute(mapk::k_prepare, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    bool ok = cudaFuncSetAttribute(mapk::k_prepare<false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+              cudaFuncSetAttribute(mapk::k_prepare<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
     for (const void *f : both)
         ok = ok && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mapk::TAIL_SMEM) == cudaSuccess &&
              cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
@@ -693,6 +694,52 @@ int map_graph_info(const map_graph *g, uint32_t *n, uint64_t *m)
 
 namespace {
 
+// where a launch leaves its result: the handle's page-locked slot, or (without one) behind its control block
+mapk::RunRes *run_result(const map_graph *g)
+{
+    return g->h_ctl_pinned ? reinterpret_cast<mapk::RunRes *>(reinterpret_cast<uint8_t *>(g->h_ctl) + PinnedSlots::RES)
+                           : reinterpret_cast<mapk::RunRes *>(g->run_ctl + 1);
+}
+
+// what a batch's own checks, graph by graph, left in ctl->bad (synchronises)
+int read_bad(map_graph *g)
+{
+    g->h_ctl->bad = 0;
+    return g->comp ? read_ctl(g) : MAP_OK;
+}
+
+// Graphs up to here are set up in one cluster (k_prepare): one launch and one stream wait instead of six launches,
+// a control-block read and two waits.  What bounds either is latency; sixteen SMs keep up with the whole chip until
+// each thread has some eight entries.  map_create from device memory, launches / cluster, us: 1,000 vertices with
+// 4,000 entries 76 / 55, 16,384 with 65,536 85 / 63, 65,536 with 65,536 85 / 67, 32,768 with 131,072 90 / 76;
+// 65,536 with 262,144 89 / 104, 131,072 with 262,144 90 / 110.
+constexpr uint32_t PREPARE_N = 65536, PREPARE_M = 131072;
+
+// a launch of `blocks` blocks of TT threads as one cluster
+void cluster_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &attr, uint32_t blocks, size_t smem, cudaStream_t s)
+{
+    cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(mapk::TT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = blocks;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+}
+
+// blocks of k_tail for a whole graph of n vertices: one vertex per thread as far as the cluster goes (random
+// graphs, synchronous, us per run with 1 / 2 / 4 / 8 / 16 blocks: 4,000 vertices 131 / 115 / 88 / 92 / 104,
+// 8,000 vertices 223 / 178 / 152 / 124 / 132, 16,384 vertices - / 231 / 180 / 160 / 141)
+uint32_t tail_blocks_for(uint32_t n, int cluster)
+{
+    uint32_t blocks = 1;
+    while ((int)blocks < cluster && n > blocks * (uint32_t)mapk::TT) blocks *= 2;
+    return blocks;
+}
+
 // Allocate and prepare a graph of n vertices and m edges.  `upload(g, &acc)`
 // fills g->rowptr (n + 1 words) and g->colidx (m words) on stream s and sets acc
 // to a device bitmap of the accepting vertices; it may also set up the batch
@@ -848,14 +895,43 @@ int create_graph(uint32_t n, uint64_t m, cudaStream_t s, const char *who, Upload
         free_graph(g);
         return rc;
     }
+    const uint32_t *const rp_in = g->in_rowptr ? g->in_rowptr : g->rowptr, *const ci_in = g->in_colidx ? g->in_colidx : g->colidx;
+    const uint32_t *const rp_copy = g->in_rowptr;
+    g->in_rowptr = g->in_colidx = nullptr;
+    const int cluster = n <= PREPARE_N && m <= PREPARE_M ? tail_blocks() : 0;
+    if (cluster) { // a small graph: everything in one cluster, one launch and one wait
+        uint32_t *const prep = reinterpret_cast<uint32_t *>(run_result(g)); // (a page-locked slot, or device memory)
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attr;
+        cluster_config(cfg, attr, tail_blocks_for(std::max<uint32_t>(n, (uint32_t)m / 2), cluster), 0, s);
+        uint32_t h[6];
+        if ((rc = ck(cudaLaunchKernelEx(&cfg, mapk::k_prepare<true>, n, rp_in, ci_in, (const uint32_t *)acc_in, (uint32_t)m, g->acc0,
+                                        g->rrowptr, g->rcol, rank, prep, mapk::PrepareOut{g->rowptr, g->colidx, g->rpos}),
+                     "set-up")) ||
+            (!g->h_ctl_pinned && (rc = ck(cudaMemcpyAsync(h, prep, sizeof h, cudaMemcpyDeviceToHost, s), "set-up"))) ||
+            (rc = ck(cudaStreamSynchronize(s), "set-up")) || (rc = read_bad(g))) {
+            free_rank();
+            free_graph(g);
+            return rc;
+        }
+        free_rank();
+        if (g->h_ctl_pinned) memcpy(h, prep, sizeof h);
+        if (h[0] || g->h_ctl->bad) {
+            free_graph(g);
+            return fail(MAP_ERR_CSR, "%s: invalid CSR (decreasing rowptr or colidx out of range)", who);
+        }
+        g->nacc0 = h[1];
+        g->functional = m > 0 && h[4] == 0;
+        g->acc_entries = h[5];
+        *out = g;
+        return MAP_OK;
+    }
     // the accepting set, then one pass over the CSR: validation, in-degree histogram of the reverse
     // CSR, and the accepting flag of each target into bit 31 of its entry (restored after every run)
     mapk::k_acc_init<<<grid_for(g, W, 1), 256, 0, s>>>(n, acc_in, g->acc0, &g->ctl->elim.v);
     mapk::k_ingest<<<grid_for(g, std::max<uint64_t>(m / 4, n), 1), 256, 0, s>>>(
-        n, g->in_rowptr ? g->in_rowptr : g->rowptr, g->in_rowptr ? g->rowptr : nullptr, m,
-        g->in_colidx ? g->in_colidx : g->colidx, g->colidx, g->acc0, g->rrowptr, rank, &g->ctl->bad,
+        n, rp_in, rp_copy ? g->rowptr : nullptr, m, ci_in, g->colidx, g->acc0, g->rrowptr, rank, &g->ctl->bad,
         &g->ctl->long_rows, (unsigned long long *)&g->ctl->relax.v);
-    g->in_rowptr = g->in_colidx = nullptr;
     if ((rc = ck(cudaGetLastError(), "validate")) || (rc = read_ctl(g))) {
         free_rank();
         free_graph(g);
@@ -969,31 +1045,6 @@ static bool runs_in_own(const map_graph *g) { return !runs_in_tail(g) && g->n <=
 // 0.44 ms, that product 1.5 ms in k_own).
 static bool default_fstart(const map_graph *g) { return runs_in_tail(g) || runs_in_own(g) || g->acc_entries <= g->m / 16; }
 
-// a launch of `blocks` blocks of TT threads as one cluster
-static void cluster_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &attr, uint32_t blocks, size_t smem, cudaStream_t s)
-{
-    cfg = {};
-    cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(mapk::TT);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = blocks;
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-}
-
-// blocks of k_tail for a whole graph of n vertices: one vertex per thread as far as the cluster goes (random
-// graphs, synchronous, us per run with 1 / 2 / 4 / 8 / 16 blocks: 4,000 vertices 131 / 115 / 88 / 92 / 104,
-// 8,000 vertices 223 / 178 / 152 / 124 / 132, 16,384 vertices - / 231 / 180 / 160 / 141)
-static uint32_t tail_blocks_for(uint32_t n, int cluster)
-{
-    uint32_t blocks = 1;
-    while ((int)blocks < cluster && n > blocks * (uint32_t)mapk::TT) blocks *= 2;
-    return blocks;
-}
-
 static int launch_tail(const mapk::RunArgs &a, bool sync_sched, bool whole, uint32_t blocks, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg;
@@ -1027,13 +1078,6 @@ static int take_result(const mapk::RunRes &R, const map_opts &opts, uint64_t m, 
         }
     }
     return MAP_OK;
-}
-
-// where a launch leaves its result: the handle's page-locked slot, or (without one) behind its control block
-static mapk::RunRes *run_result(const map_graph *g)
-{
-    return g->h_ctl_pinned ? reinterpret_cast<mapk::RunRes *>(reinterpret_cast<uint8_t *>(g->h_ctl) + PinnedSlots::RES)
-                           : reinterpret_cast<mapk::RunRes *>(g->run_ctl + 1);
 }
 
 // wait for the stream; *R: the result, copied to *pageable where there is no page-locked slot
@@ -2140,7 +2184,7 @@ static int run_static_cluster(uint32_t n, const uint32_t *rowptr, const uint32_t
         acc_bits = base + ST_ACC;
     }
     struct Back { // what comes back: k_prepare's verdict and the run's result
-        uint32_t prep[4];
+        uint32_t prep[6];
         mapk::RunRes res;
     };
     Back *const dev = reinterpret_cast<Back *>(base + ST_LIST);
@@ -2165,8 +2209,8 @@ static int run_static_cluster(uint32_t n, const uint32_t *rowptr, const uint32_t
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr;
     cluster_config(cfg, attr, tail_blocks_for(n, cluster), 0, s);
-    CK(cudaLaunchKernelEx(&cfg, mapk::k_prepare, n, rowptr, colidx, acc_bits, (uint32_t)ST_MAX_M, base + ST_ACC0,
-                          base + ST_RROWPTR, base + ST_RCOL, base + ST_RPOS, dev->prep));
+    CK(cudaLaunchKernelEx(&cfg, mapk::k_prepare<false>, n, rowptr, colidx, acc_bits, (uint32_t)ST_MAX_M, base + ST_ACC0,
+                          base + ST_RROWPTR, base + ST_RCOL, base + ST_RPOS, dev->prep, mapk::PrepareOut{}));
     int rc = launch_tail(a, sync_sched, true, tail_blocks_for(n, cluster), s);
     if (rc) return rc;
     Back h;

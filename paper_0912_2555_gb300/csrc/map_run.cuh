@@ -2044,16 +2044,25 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
 // increment of u's in-degree returned; the row of an entry is found by binary search, so that a row of any
 // length is spread over all threads.  Replaces eight launches, five memsets and two stream waits: at 1,000
 // vertices they were most of map_run_static's 480 us.
+// (rowptr and colidx by plain loads: in place, they are written here too.)
 // prep: (0 = good, 1 = rowptr[0] != 0, 2 = more than max_m entries, 3 = invalid), accepting vertices, entries,
-// rowptr[0]; rank: m words; cnt: n + 1 words, becomes rrowptr.
+// rowptr[0], whether some row holds two entries or more, entries that hold an accepting vertex; rank: m words;
+// cnt: n + 1 words, becomes rrowptr.  FULL (map_create): also the handle's copies of rowptr and colidx (with the
+// accepting flag in bit 31; they may be the inputs themselves) and the reader entries' positions; there max_m is
+// the number of entries, which the host has read already, and the inputs may lie across the link: each word of them
+// is read once.
+struct PrepareOut {
+    uint32_t *rowptr, *colidx, *rpos;
+};
+template <bool FULL>
 __global__ void __launch_bounds__(TT, 1)
     k_prepare(uint32_t n, const uint32_t *rowptr, const uint32_t *colidx, const uint32_t *acc_in, uint32_t max_m,
-              uint32_t *acc0, uint32_t *cnt, uint32_t *rcol, uint32_t *rank, uint32_t *prep)
+              uint32_t *acc0, uint32_t *cnt, uint32_t *rcol, uint32_t *rank, uint32_t *prep, PrepareOut out)
 {
-    __shared__ uint32_t s_warp[TT / 32], s_part[TAIL_C], s_bad, s_acc;
+    __shared__ uint32_t s_warp[TT / 32], s_part[TAIL_C], s_bad, s_acc, s_ent;
     const uint32_t C = gridDim.x, me = cluster_rank(), tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     const uint32_t gid = me * TT + tid, threads = C * TT;
-    const uint32_t r0 = __ldg(rowptr), m = __ldg(rowptr + n);
+    const uint32_t r0 = FULL ? 0u : rowptr[0], m = FULL ? max_m : rowptr[n];
     if (r0 != 0 || m > max_m) { // (every block)
         if (gid == 0) {
             prep[0] = r0 != 0 ? 1u : 2u;
@@ -2063,11 +2072,17 @@ __global__ void __launch_bounds__(TT, 1)
         }
         return;
     }
-    if (tid == 0) s_bad = s_acc = 0;
+    if (tid == 0) s_bad = s_acc = s_ent = 0;
     cluster_barrier();
-    uint32_t bad = 0, na = 0;
+    uint32_t bad = 0, na = 0, ne = 0; // (bad: bit 0 invalid, bit 1 a row of two entries or more)
     for (uint32_t i = gid; i <= n; i += threads) cnt[i] = 0;
-    for (uint32_t i = gid; i < n; i += threads) bad |= __ldg(rowptr + i) > __ldg(rowptr + i + 1);
+    for (uint32_t i0 = gid - lane; i0 <= n; i0 += threads) { // (a lane's row end comes from the next lane)
+        const uint32_t i = i0 + lane, b = i <= n ? rowptr[i] : 0u;
+        uint32_t e = __shfl_down_sync(0xFFFFFFFFu, b, 1);
+        if (lane == 31 && i < n) e = rowptr[i + 1];
+        if (i < n) bad |= (b > e ? 1u : 0u) | (e - b > 1u ? 2u : 0u);
+        if (FULL && i <= n) out.rowptr[i] = b; // (in place, the same word)
+    }
     const uint32_t words = (n + 31) / 32;
     for (uint32_t i = gid; i < words; i += threads) {
         uint32_t x = __ldg(acc_in + i);
@@ -2076,20 +2091,41 @@ __global__ void __launch_bounds__(TT, 1)
         na += __popc(x);
     }
     cluster_barrier(); // the counts are zero
-    for (uint32_t i = gid; i < m; i += threads) {
-        const uint32_t u = __ldg(colidx + i);
-        if (u >= n) bad = 1;
-        else rank[i] = atomicAdd(cnt + u + 1, 1u);
+    // (U entries in flight per thread, here and in the scatter: map_create of 32,768 vertices with 131,072 entries
+    // took 86 us with one, 76 with four)
+    constexpr int U = 4;
+    for (uint32_t i0 = gid; i0 < m; i0 += U * threads) {
+        uint32_t u[U], at[U], flag[U];
+#pragma unroll
+        for (int j = 0; j < U; ++j) u[j] = i0 + j * threads < m ? colidx[i0 + j * threads] : 0u;
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            const bool in = i0 + j * threads < m && u[j] < n;
+            at[j] = in ? atomicAdd(cnt + u[j] + 1, 1u) : 0u;
+            flag[j] = FULL && in ? (__ldg(acc_in + (u[j] >> 5)) >> (u[j] & 31u)) & 1u : 0u;
+        }
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            const uint32_t i = i0 + j * threads;
+            if (i >= m) break;
+            bad |= u[j] >= n ? 1u : 0u;
+            rank[i] = at[j];
+            ne += flag[j];
+            if (FULL) out.colidx[i] = u[j] | flag[j] << 31;
+        }
     }
-    // verdict on the input, and the accepting vertices, to block 0
-    bad = __any_sync(0xFFFFFFFFu, bad);
+    // an invalid input to every block, the counts to block 0
+    const auto add = [&](uint32_t *to, uint32_t x) {
+        asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(cluster_addr(shared_addr(to), 0)), "r"(x)
+                     : "memory");
+    };
+    bad = __reduce_or_sync(0xFFFFFFFFu, bad);
     na = __reduce_add_sync(0xFFFFFFFFu, na);
+    ne = __reduce_add_sync(0xFFFFFFFFu, ne);
     if (lane == 0) {
-        if (bad) cluster_or(cluster_addr(shared_addr(&s_bad), 0), 1u);
-        if (na)
-            asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(cluster_addr(shared_addr(&s_acc), 0)),
-                         "r"(na)
-                         : "memory");
+        for (uint32_t q = 0; q < ((bad & 1u) ? C : bad ? 1u : 0u); ++q) cluster_or(cluster_addr(shared_addr(&s_bad), q), bad);
+        if (na) add(&s_acc, na);
+        if (ne) add(&s_ent, ne);
     }
     cluster_barrier(); // the counts are complete
     // inclusive scan of cnt[0 .. n]: a contiguous share per block
@@ -2125,21 +2161,37 @@ __global__ void __launch_bounds__(TT, 1)
         run += s_warp[TT / 32 - 1];
     }
     if (gid == 0) {
-        prep[0] = s_bad ? 3u : 0u;
+        prep[0] = (s_bad & 1u) ? 3u : 0u;
         prep[1] = s_acc;
         prep[2] = m;
         prep[3] = 0;
+        prep[4] = s_bad >> 1;
+        prep[5] = s_ent;
     }
-    cluster_barrier(); // the starts are in place, and the verdict
-    if (*(volatile uint32_t *)prep) return;
-    for (uint32_t i = gid; i < m; i += threads) {
-        uint32_t lo = 0, hi = n; // rowptr[lo] <= i < rowptr[hi]
-        while (hi - lo > 1) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (__ldg(rowptr + mid) <= i) lo = mid;
-            else hi = mid;
+    cluster_barrier(); // the starts are in place
+    if (s_bad & 1u) return; // (the same in every block; nobody's shared memory is read from here on)
+    const uint32_t *const rows = FULL ? out.rowptr : rowptr, *const cols = FULL ? out.colidx : colidx;
+    for (uint32_t i0 = gid; i0 < m; i0 += U * threads) {
+        uint32_t slot[U], lo[U], left = n; // rows[lo] <= i < rows[lo + left]
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            const uint32_t i = min(i0 + j * threads, m - 1);
+            slot[j] = __ldcg(cnt + (cols[i] & 0x7FFFFFFFu)) + rank[i];
+            lo[j] = 0;
         }
-        rcol[__ldcg(cnt + __ldg(colidx + i)) + rank[i]] = lo;
+        while (left > 1) { // (the same steps for all: where left is odd, its larger half stays)
+            const uint32_t half = left >> 1;
+#pragma unroll
+            for (int j = 0; j < U; ++j) lo[j] += rows[lo[j] + half] <= min(i0 + j * threads, m - 1) ? half : 0u;
+            left -= half;
+        }
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            const uint32_t i = i0 + j * threads;
+            if (i >= m) break;
+            rcol[slot[j]] = lo[j];
+            if (FULL) out.rpos[slot[j]] = i;
+        }
     }
 }
 

@@ -226,3 +226,62 @@ def test_batch_flood(pkg):
                 off += g.n
     finally:
         pkg.map_destroy(h)
+
+
+LIMIT = 65536  # vertices of the largest graph that is set up in one cluster (131,072 entries)
+
+
+@pytest.mark.parametrize("n,m", [(1, 0), (1, 3), (33, 0), (1023, 5000), (1025, 1024), (16_385, 65_537),
+                                 (LIMIT, 2 * LIMIT), (LIMIT, 2 * LIMIT + 1), (LIMIT + 1, 2 * LIMIT), (700, 2 * LIMIT)])
+@pytest.mark.parametrize("where", ["device", "unaligned", "host", "pinned"])
+def test_set_up(pkg, n, m, where):
+    """Graphs around the limits of the one-cluster set-up, wherever the input lies: rows without entries, repeated
+    entries, one row of a quarter of all entries, bits set past the last vertex."""
+    rng = np.random.default_rng(n + m)
+    at = np.sort(rng.integers(0, n, m))
+    at[: m // 4] = at[: max(1, m // 4)][0] if m else 0
+    rowptr = np.searchsorted(np.sort(at), np.arange(n + 1)).astype(np.uint32)
+    rowptr[n] = m
+    col = rng.integers(0, n, m).astype(np.uint32)
+    acc = (rng.random(n) < 0.1).astype(np.uint8)
+    g = mapgen.Graph(n, rowptr, col, acc, (0,) * 8, "set-up", {})
+    want = oracle.run_graph(g)
+    bits = pkg.pack_bits(acc).copy()
+    if n & 31:
+        bits[-1] |= np.uint32(0xFFFFFFFF << (n & 31) & 0xFFFFFFFF)
+    args = [rowptr, col, bits]
+    if where != "host":
+        shift = 1 if where == "unaligned" else 0
+        args = [torch.from_numpy(np.concatenate([np.zeros(shift, np.uint32), x]).view(np.int32)) for x in args]
+        args = [(x.pin_memory() if where == "pinned" else x.cuda())[shift:] for x in args]
+    h = pkg.map_create(n, args[0], args[1] if m else None, args[2])
+    try:
+        assert pkg.map_graph_info(h) == (n, m)
+        for flags in (pkg.MAP_FLAG_FRONTIER_START, pkg.MAP_FLAG_DENSE_START):
+            out = torch.empty(n, dtype=torch.int32, device="cuda")
+            r = pkg.map_run(h, flags=flags, map_out=out)
+            assert (r.verdict, r.witness, r.outer) == (want.verdict, want.witness, want.outer)
+            assert (r.rounds, r.relaxations) == (want.rounds, want.relaxations)
+            assert np.array_equal(out.cpu().numpy().view(np.uint32), want.map)
+        assert np.array_equal(np.asarray(pkg.map_graph_csr(h)[1]).view(np.uint32)[:m], col)
+    finally:
+        pkg.map_destroy(h)
+
+
+@pytest.mark.parametrize("n", [40, 20_000, LIMIT])
+@pytest.mark.parametrize("fault", ["decreasing", "entry", "first"])
+@pytest.mark.parametrize("on_device", [False, True])
+def test_set_up_refuses(pkg, n, fault, on_device):
+    rowptr = np.arange(n + 1, dtype=np.uint32)
+    col = np.arange(n, dtype=np.uint32)
+    if fault == "decreasing":
+        rowptr[n - 1] = n + 1
+    elif fault == "entry":
+        col[n // 2] = n
+    else:
+        col[0] = 0xFFFFFFFF
+    args = [rowptr, col, np.zeros((n + 31) // 32, np.uint32)]
+    if on_device:
+        args = [torch.from_numpy(x.view(np.int32)).cuda() for x in args]
+    with pytest.raises(pkg.MapError, match="CSR"):
+        pkg.map_create(n, *args)
