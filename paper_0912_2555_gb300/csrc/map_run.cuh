@@ -1530,6 +1530,11 @@ __global__ void __launch_bounds__(TT, 1) k_tail(const __grid_constant__ RunArgs 
 constexpr uint32_t OWN_N = 12288;              // vertices per block: 18 bytes of shared memory each
 constexpr uint32_t OWN_SMEM = 224 * 1024;      // the rest holds reader lists
 constexpr int OWN_U = 4;                       // words read ahead per thread
+// asynchronous: looks at the share per round after the first, while it changes (a look is one coalesced read, the
+// barrier two dependent accesses through L2 and the wait for the slowest block).  us per run with 0 / 1 / 2 / 3 / 5:
+// layered 4 M 1260 / 1174 / 1150 / 1177 / 1185, 2^24 1557 / 1437 / 1387 / 1381 / 1374, 2^26 2641 / 2464 / 2440 / 2444 /
+// 2434, random 300,000 395 / 368 / 362 / 366 / 380, interleaved product 6x7 255 / 221 / 204 / 199 / 193
+constexpr uint32_t OWN_PASSES = 2;
 constexpr uint32_t OWN_HUB = 2048;             // reader lists longer than this are walked by the whole block
 
 struct OwnSmem {
@@ -1693,7 +1698,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
             };
             const bool pushes = r <= a.max_inner; // (past the limit the last round's values are only taken)
             uint32_t hits = 0;
-            for (uint32_t pass = 0;; ++pass) { // (asynchronous: the share once more, lc_passes times while it changes)
+            for (uint32_t pass = 0;; ++pass) { // (asynchronous: the share once more, a few times while it changes)
                 if (tid == 0) sh.n = sh.hubs = 0;
                 __syncthreads();
                 const bool start = r == 1 && pass == 0;
@@ -1788,7 +1793,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
                     for (uint32_t j = tid; j < ll; j += TT) push(reader(b + j), o);
                 }
                 __syncthreads(); // (the queue and the hubs are read)
-                if (SYNC || BATCH || pass >= a.lc_passes) break;
+                if (SYNC || BATCH || pass >= max(a.lc_passes, OWN_PASSES)) break;
             }
             alive = run_barrier(c, c->obar, sh, seq, (unsigned long long)hits + ((r & 3u) == 0 && late() ? RUN_STOP : 0ull), total);
             if (!alive) break;
