@@ -262,7 +262,7 @@ MAP_API int map_batch_run(map_graph *g, const map_opts *opts, map_result *result
  * does).  When no other worker is waiting for work, queued jobs join its run,
  * as one batched run (see map_batch_create), oldest first, while they fit into
  * the budget and may share it: the same schedule, flags and timeout, no early
- * exit, limit or MAP_FLAG_PROFILE, and at most 2^20 vertices each (a batched
+ * exit, limit or MAP_FLAG_PROFILE, and at most 2^16 vertices each (a batched
  * run lasts as long as its slowest graph, so larger jobs run alone); at most
  * 128 jobs (map_server_batch_limit) and 2^26 vertices per run.  Jobs that
  * cannot join keep their place in the queue.  Jobs that arrive while

@@ -1,8 +1,9 @@
 // map_api.cu -- host side of the C ABI declared in include/map.h.
 //
 // The outer loop of MAP (Section 2: propagate to the fix-point, self-map test,
-// eliminate, restart) and the fix-point loop are driven from here; every step
-// of the arithmetic runs in the kernels of map_kernels.cuh.
+// eliminate, restart) and the fix-point loop are launched from here, as one
+// kernel for the whole run (map_run.cuh), as a CUDA graph or step by step; every
+// step of the arithmetic runs in the kernels of map_run.cuh and map_kernels.cuh.
 #include <cuda_runtime.h>
 #include <stdarg.h>
 #include <stdint.h>
@@ -1039,10 +1040,10 @@ static bool runs_in_own(const map_graph *g) { return !runs_in_tail(g) && g->n <=
 
 // Which start a run takes when neither its flags nor map_autotune say: the frontier start pushes
 // from the accepting vertices (one random access per entry that holds one) and runs in one launch, the
-// dense start streams the whole matrix.  Measured: layered graphs (1 entry in 200) 3.4 against 16.4 ms at
+// dense start streams the whole matrix.  Measured: layered graphs (1 entry in 200) 2.5 against 16.7 ms at
 // 2^26 vertices, an interleaved product with 1 entry in 7 (1.6 M vertices) 6.4 against 4.6 ms in k_run.  Graphs
-// that fit into one cluster or the SMs' shared memory gain whatever the share (16,384 vertices 0.12 against
-// 0.44 ms, that product 1.5 ms in k_own).
+// that fit into one cluster or the SMs' shared memory gain whatever the share (16,384 vertices 0.16 against
+// 0.52 ms, that product 1.0 ms in k_own).
 static bool default_fstart(const map_graph *g) { return runs_in_tail(g) || runs_in_own(g) || g->acc_entries <= g->m / 16; }
 
 static int launch_tail(const mapk::RunArgs &a, bool sync_sched, bool whole, uint32_t blocks, cudaStream_t s)
@@ -2484,8 +2485,12 @@ constexpr uint32_t kBatchFlags = MAP_FLAG_FRONTIER_START | MAP_FLAG_DENSE_START 
 constexpr uint32_t kMaxBatchJobs = 128;
 constexpr uint64_t kMaxBatchVertices = 1ull << 26;
 // a batched run lasts as long as its slowest graph: larger jobs run alone, so that the small
-// ones batched together do not wait for them
-constexpr uint32_t kMaxBatchedJobN = 1u << 20;
+// ones batched together do not wait for them.  A run alone is one launch now and a small part of its job's
+// copies, so only jobs that are mostly launches and waits gain by sharing.  1,200 jobs (median 10^5 vertices) at
+// 2,000 / 4,000 / 16,000 per second, 8 workers, jobs served per second: up to 2^20 vertices 1,504 / 1,418 / 1,345,
+// 2^16 2,024 / 2,731 / 2,742, 2^14 2,023 / 2,719 / 2,738 (none: 2,023 / 2,755 / 2,771; with the launches per round
+// of before, 2^20 1,886 / 2,261 / 2,233); 38 synchronous jobs at once, ms: 76 / 59 / 67.
+constexpr uint32_t kMaxBatchedJobN = 1u << 16;
 
 // device bytes of a graph: the allocations of create_graph
 size_t graph_footprint(uint64_t n, uint64_t m)

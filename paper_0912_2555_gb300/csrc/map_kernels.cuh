@@ -26,7 +26,8 @@
 //   alist[|A0|]              the initially accepting vertices (frontier start only);
 //   Ctl                      the control block below (one per graph).
 //
-// One outer iteration: the dense round (every row, k_dense), then push rounds
+// Runs that push from the accepting vertices throughout are in map_run.cuh.  Here, one
+// outer iteration of the others: the dense round (every row, k_dense), then push rounds
 // until a round changes nothing (k_rounds, one persistent cooperative launch
 // with a grid barrier between rounds), then the self-map test and the
 // elimination over the touched vertices (check_phase: the tail of k_rounds when

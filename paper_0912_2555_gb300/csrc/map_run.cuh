@@ -30,12 +30,12 @@
 //
 // Floods.  When a list holds a large share of the whole graph's vertices (one value sweeping a giant
 // component), its random accesses cost more than reading everything in order: from there on the iteration
-// runs in scan mode (Run::scan_round), with 4-byte state arrays, pushes that nothing waits for and each block
-// reading its contiguous share of the vertices every round.
+// runs in scan mode (Run::scan_round), with 4-byte state arrays, pushes that nothing waits for and all vertices
+// read in order every round, in pieces that go round the blocks.
 //
-// What it measured, ms per run (dense start in a CUDA graph -> here, k_tail included): layered 2^26
-// asynchronous 16.35 -> 3.4, 2^24 synchronous 7.3 -> 2.6, 10^6 asynchronous 2.82 -> 0.89, the 16,384-vertex
-// random graph 0.44 -> 0.12.
+// What it measured, ms per run (dense start in a CUDA graph -> here, k_own and k_tail included): layered 2^26
+// asynchronous 16.7 -> 2.5, 2^24 synchronous 7.9 -> 1.7, 10^6 asynchronous 3.0 -> 0.81, a random graph of 16,384
+// vertices synchronous 0.52 -> 0.16.
 #pragma once
 #include "map_kernels.cuh"
 
@@ -1524,7 +1524,10 @@ __global__ void __launch_bounds__(TT, 1) k_tail(const __grid_constant__ RunArgs 
 // words (coalesced) and pushes for those that changed.  So a round is one coalesced read, the reader ids,
 // and the barrier, where k_run's lists take seven dependent accesses (list, state, reader range, reader,
 // returning atomic, list position, barrier) and 1.3 us more.  Reading the whole share costs V * 4 bytes a round
-// from L2, about 1 us at the largest size.
+// from L2, about 1 us at the largest size.  Rounds over few vertices are bound by that chain (2.3 to 3 us); floods
+// by the reductions: an interleaved product of 1.6 M vertices, synchronous, sends 131 M of them in 0.99 ms, 133 G/s,
+// the rate at which L2 takes scattered ones.  (Reading the word first, to leave out what raises nothing, took 1.7 ms:
+// the loads wait for the reductions on their lines.)  That run took 4.4 ms with the dense start.
 //   asynchronous  in[0] / in[1] = the values, by outer iteration mod 2; last = the value pushed last
 //   synchronous   in[0] / in[1] = the inboxes, by round mod 2 (as in k_tail); last = the value
 constexpr uint32_t OWN_N = 12288;              // vertices per block: 18 bytes of shared memory each
@@ -2048,7 +2051,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
 // and its size, and the readers (reverse CSR).  Entry i holding u goes to slot start(u) + the count its
 // increment of u's in-degree returned; the row of an entry is found by binary search, so that a row of any
 // length is spread over all threads.  Replaces eight launches, five memsets and two stream waits: at 1,000
-// vertices they were most of map_run_static's 480 us.
+// vertices they were most of map_run_static's 490 us (107 now).
 // (rowptr and colidx by plain loads: in place, they are written here too.)
 // prep: (0 = good, 1 = rowptr[0] != 0, 2 = more than max_m entries, 3 = invalid), accepting vertices, entries,
 // rowptr[0], whether some row holds two entries or more, entries that hold an accepting vertex; rank: m words;

@@ -2,6 +2,8 @@
 they change: a vertex more or less than a thread per vertex, a block, the cluster's capacity; compaction into a
 small and into a large graph; reader lists longer than a warp walks alone; limits; a map buffer of odd alignment.
 Integer work: everything must be equal."""
+import time
+
 import numpy as np
 import pytest
 
@@ -285,3 +287,27 @@ def test_set_up_refuses(pkg, n, fault, on_device):
         args = [torch.from_numpy(x.view(np.int32)).cuda() for x in args]
     with pytest.raises(pkg.MapError, match="CSR"):
         pkg.map_create(n, *args)
+
+
+def test_large_jobs_run_alone(pkg):
+    """Queued behind a long job, jobs of up to 65,536 vertices share runs, larger ones run alone."""
+    big = mapgen.layered_graph(4_000_000, 240, seed=8)
+    gs = [mapgen.layered_graph(LIMIT + d, 12, seed=40 + i, plant=bool(i & 1)) for i, d in enumerate([-1, 0, 1, 0, 1, -7])]
+    with pkg.Server(slots=1) as sv:
+        first = sv.submit(big.n, big.rowptr, big.colidx, pkg.pack_bits(big.acc))
+        ids = [sv.submit(g.n, g.rowptr, g.colidx, pkg.pack_bits(g.acc)) for g in gs]
+        left, done = {first, *ids}, {}
+        deadline = time.time() + 60
+        while left and time.time() < deadline:
+            for jid in list(left):
+                got = sv.poll(jid)
+                if got is not None:
+                    done[jid] = got
+                    left.discard(jid)
+    assert not left
+    for g, jid in zip(gs, ids):
+        r, mp = done[jid]
+        want = oracle.run_graph(g)
+        assert (r.verdict, r.witness, r.outer, r.relaxations) == (want.verdict, want.witness, want.outer, want.relaxations)
+        assert np.array_equal(mp, want.map)
+        assert (r.batch_jobs > 1) == (g.n <= LIMIT), g.n
