@@ -553,6 +553,7 @@ template <bool SYNC, bool BATCH> struct Run {
             }
             __syncthreads();
             const uint32_t nq = sh.ln; // (the hits of several chunks are pushed together)
+            __syncthreads();           // (read by every warp before the next chunk's hits are added: all take one branch)
             if (nq + CHUNK <= RUN_CAP && c0 + step * U < v1) continue;
             hits += nq;
             if (pushes)
