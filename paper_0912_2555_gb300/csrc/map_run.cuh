@@ -2023,7 +2023,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
         ph_rounds += c->ph_rounds;
         ph_check += c->ph_check;
     }
-    if (hand) {
+    if (hand && alive) { // (after a wait that gave up the reader lists may be unwritten: nothing is left to k_tail)
         c->outer = outer;
         c->nacc = nacc;
         c->inner_total = inner_total;
