@@ -987,7 +987,9 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
                     if ((uint64_t)first + tot > ecap) over = true;
                     if (in) {
                         const uint32_t v = __ldcg(a.touched + i), u = run.id_of(v);
-                        meta2[i] = make_uint4(first + excl, first + excl + len, run.accepting(v) ? u + 1 : 0u, u);
+                        // (batched: a graph that has ended keeps its values, and offers nothing any more)
+                        const bool offers = run.accepting(v) && !(BATCH && !*(volatile uint32_t *)&a.cs[__ldcg(sp.comp + v)].active);
+                        meta2[i] = make_uint4(first + excl, first + excl + len, offers ? u + 1 : 0u, u);
                         if (SYNC || BATCH)
                             row2[i] = sp.row ? __ldcg(sp.row + v) : __ldg(a.rowptr + v + 1) - __ldg(a.rowptr + v);
                         if (BATCH) comp2[i] = __ldcg(sp.comp + v);

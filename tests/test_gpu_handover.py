@@ -1,0 +1,102 @@
+"""What one kernel of a whole run leaves to the next (k_run to k_own to k_tail), against the oracle: graphs of a batch that
+end in the iteration after which the rest is renumbered."""
+import time
+
+import numpy as np
+import pytest
+
+import mapgen
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+OWN = 152 * 12288  # vertices that k_own holds whole
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import __graft_entry__
+
+    __graft_entry__.build()
+    import paper_0912_2555_gb300 as p
+
+    return p
+
+
+def padded(g, n):
+    """g with vertices without edges behind it."""
+    rowptr = np.concatenate([g.rowptr, np.full(n - g.n, g.rowptr[-1], np.uint32)])
+    acc = np.concatenate([g.acc, np.zeros(n - g.n, np.uint8)])
+    return mapgen.Graph(n, rowptr, g.colidx, acc, (0,) * 8, g.name, {})
+
+
+def same(r, want, sched, got):
+    assert (r.verdict, r.witness, r.outer) == (want.verdict, want.witness, want.outer)
+    assert np.array_equal(got, want.map)
+    if sched == 0:
+        assert (r.rounds, r.relaxations) == (want.rounds, want.relaxations)
+
+
+def two_cycles(n):
+    """Two accepting vertices on cycles, the smaller one leads to the larger: 5 is the witness, 2 is left with a value."""
+    rows = [[] for _ in range(n)]
+    rows[2], rows[5] = [2, 5], [5]
+    return mapgen.from_lists(rows, [int(v in (2, 5)) for v in range(n)])
+
+
+@pytest.mark.parametrize("large", [OWN + 1, 3_000_000])
+def test_batch_renumbered_while_graphs_end(pkg, large):
+    """Small graphs end with a cycle in iteration 1, the large ones go on renumbered: the ended ones stay as they are."""
+    gs = [two_cycles(6), padded(mapgen.layered_graph(90_000, 30, seed=7), large), two_cycles(70)]
+    gs += [mapgen.tiny_graph(seed, 40, max_deg=3, acc_p=0.4) for seed in range(12)]
+    gs += [mapgen.layered_graph(50_000, 20, seed=9), mapgen.layered_graph(5000, 8, seed=10, plant=True)]
+    wants = [oracle.run_graph(g) for g in gs]
+    assert max(w.outer for w in wants) > 2 and sum(w.verdict == 1 and w.outer == 1 for w in wants) > 4
+    h = pkg.map_batch_create([(g.n, g.rowptr, g.colidx, pkg.pack_bits(g.acc)) for g in gs])
+    try:
+        for sched in (0, 1):
+            out = np.empty(sum(g.n for g in gs), np.uint32)
+            rs = pkg.map_batch_run(h, len(gs), sched=sched, flags=pkg.MAP_FLAG_FRONTIER_START, map_out=out)
+            off = 0
+            for g, r, want in zip(gs, rs, wants):
+                same(r, want, sched, out[off:off + g.n])
+                off += g.n
+    finally:
+        pkg.map_destroy(h)
+
+
+def test_served_batch_on_a_share_of_the_chip(pkg):
+    """The same through a server: a worker's share of the chip holds fewer vertices, so that a shared run of a few hundred
+    thousand is renumbered."""
+    n = 65_536
+    gs = [padded(mapgen.layered_graph(12_000, 14, seed=s), n) for s in range(6)]
+    gs += [two_cycles(n), two_cycles(6), padded(mapgen.layered_graph(4000, 8, seed=4, plant=True), n)]
+    wants = [oracle.run_graph(g) for g in gs]
+    length = n + 1  # a chain: one vertex per round, so that every worker is busy while the jobs are queued
+    chain = mapgen.Graph(length, np.concatenate([[0], np.arange(length)]).astype(np.uint32), np.arange(length - 1, dtype=np.uint32),
+                         (np.arange(length) == 0).astype(np.uint8), (0,) * 8, "chain", {})
+    with pkg.Server(slots=8) as sv:
+        first = [sv.submit(chain.n, chain.rowptr, chain.colidx, pkg.pack_bits(chain.acc)) for _ in range(8)]
+        for sched in (0, 1):
+            ids = [sv.submit(g.n, g.rowptr, g.colidx, pkg.pack_bits(g.acc), sched=sched) for g in gs]
+            left, done = set(ids), {}
+            deadline = time.time() + 60
+            while left and time.time() < deadline:
+                for jid in list(left):
+                    got = sv.poll(jid)
+                    if got is not None:
+                        done[jid] = got
+                        left.discard(jid)
+            assert not left
+            assert sched or max(r.batch_jobs for r, _ in done.values()) == len(gs)
+            for want, jid in zip(wants, ids):
+                r, mp = done[jid]
+                assert (r.verdict, r.witness, r.outer) == (want.verdict, want.witness, want.outer)
+                assert sched or r.relaxations == want.relaxations
+                assert np.array_equal(mp, want.map)
+        for jid in first:
+            while sv.poll(jid) is None:
+                pass
