@@ -1046,6 +1046,7 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
             c->ph_rounds = ph_rounds;
             c->ph_check = ph_check;
             c->t0 = t0;
+            c->ocnt[0].v = c->ocnt[1].v = 0; // (scan mode has counted there; k_own starts from zero)
             c->hand = sp.V <= a.tail_cap ? 2u : 1u;
         }
         return;

@@ -1,5 +1,5 @@
 """What one kernel of a whole run leaves to the next (k_run to k_own to k_tail), against the oracle: graphs of a batch that
-end in the iteration after which the rest is renumbered."""
+end in the iteration after which the rest is renumbered, counters that scan mode has used."""
 import time
 
 import numpy as np
@@ -100,3 +100,34 @@ def test_served_batch_on_a_share_of_the_chip(pkg):
         for jid in first:
             while sv.poll(jid) is None:
                 pass
+
+
+@pytest.mark.parametrize("n", [OWN + 1000, 4_000_000])
+def test_scan_mode_then_the_grid_kernel(pkg, n):
+    """Accepting h1 > h2 > h3 and h0.  The same quarter of the rows holds h1 and h2 (their iterations end in scan mode), 20,000
+    of these hold h3 (renumbered, the rest in k_own), none holds h0: the fourth iteration gives nobody a value and is
+    the last."""
+    rows = n // 4
+    deg = np.zeros(n, np.int64)
+    deg[:rows] = 2
+    deg[:20_000] = 3
+    rowptr = np.zeros(n + 1, np.uint32)
+    np.cumsum(deg, out=rowptr[1:])
+    col = np.tile(np.array([n - 1, n - 2], np.uint32), rows + 10_000)
+    col[rowptr[:rows]], col[rowptr[:rows] + 1] = n - 1, n - 2
+    col[rowptr[:20_000] + 2] = n - 3
+    acc = np.zeros(n, np.uint8)
+    acc[n - 4:] = 1
+    g = mapgen.Graph(n, rowptr, col[:rowptr[-1]], acc, (0,) * 8, "stars", {})
+    want = oracle.run_graph(g)
+    assert want.outer == 4
+    h = pkg.map_create(g.n, g.rowptr, g.colidx, pkg.pack_bits(g.acc))
+    try:
+        for sched in (0, 1):
+            for kw in ({}, dict(max_outer=want.outer)):
+                out = np.empty(n, np.uint32)
+                r = pkg.map_run(h, sched=sched, flags=pkg.MAP_FLAG_FRONTIER_START, map_out=out, **kw)
+                same(r, want, sched, out)
+                assert (r.edges_total, r.accepting_left) == (4 * g.m, 1)
+    finally:
+        pkg.map_destroy(h)
