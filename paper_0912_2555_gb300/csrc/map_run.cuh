@@ -458,10 +458,12 @@ template <bool SYNC, bool BATCH> struct Run {
 
     // ---- scan mode (whole graph): three arrays of n words in the pool.
     //   synchronous   A / B = the inboxes of even / odd rounds, val = the values (as in k_tail)
-    //   asynchronous  val = the values, A = the value pushed last, B = (batched) the last round a row was reached in
+    //   asynchronous  val = the values, A = the value pushed last; batched, B / tval = the last odd / even round a row was
+    //                 reached in (the round before is read while this round's pushes come in)
     __device__ __forceinline__ uint32_t *scan_val() const { return a.pool; }
     __device__ __forceinline__ uint32_t *scan_a() const { return a.pool + a.n; }
     __device__ __forceinline__ uint32_t *scan_b() const { return a.pool + 2ull * a.n; }
+    __device__ __forceinline__ uint32_t *scan_reach(uint32_t r) const { return (r & 1) ? scan_b() : a.tval; }
 
     // from lists to scans after round r: the state words into the arrays and back to zero; a vertex of round r's
     // list looks as if its value had just come in
@@ -487,7 +489,7 @@ template <bool SYNC, bool BATCH> struct Run {
                 x = (uint32_t)(q >> 32);
                 scan_val()[v] = x;
                 scan_a()[v] = (uint32_t)q == (uint32_t)~r ? 0u : x;
-                if (BATCH) scan_b()[v] = 0;
+                if (BATCH) scan_reach(0)[v] = scan_reach(1)[v] = 0;
             }
         }
         if (blockIdx.x == 0 && threadIdx.x == 0) *(volatile uint32_t *)&a.ctl->ocnt[0].v = 0;
@@ -516,7 +518,7 @@ template <bool SYNC, bool BATCH> struct Run {
                 const uint64_t v = c0 + k * step + threadIdx.x;
                 y[k] = v < v1 ? __ldcg((SYNC ? in : val) + v) : 0u;
                 if (!SYNC) z[k] = v < v1 ? __ldcg(scan_a() + v) : 0u;
-                row[k] = !SYNC && BATCH && v < v1 && __ldcg(scan_b() + v) == r - 1;
+                row[k] = !SYNC && BATCH && v < v1 && __ldcg(scan_reach(r - 1) + v) == r - 1;
             }
             uint32_t some = 0; // (warp-uniform) bit k: something in the warp's word k
 #pragma unroll
@@ -574,7 +576,7 @@ template <bool SYNC, bool BATCH> struct Run {
                             if (!live[j]) continue;
                             const uint32_t w = __ldcg(sp.rc + pos[j]);
                             atomicMax(to + w, o[j]);
-                            if (!SYNC && BATCH) atomicMax(scan_b() + w, r);
+                            if (!SYNC && BATCH) atomicMax(scan_reach(r) + w, r);
                         }
                     });
             __syncthreads();
@@ -615,7 +617,7 @@ template <bool SYNC, bool BATCH> struct Run {
                     x[k] = max(x[k], y);
                 } else if (v < a.n) {
                     ch = x[k] > __ldcg(scan_a() + v);
-                    row = BATCH && __ldcg(scan_b() + v) == r;
+                    row = BATCH && __ldcg(scan_reach(r) + v) == r;
                 }
                 if ((SYNC || BATCH) && r > 1 && __any_sync(0xFFFFFFFFu, row)) add_row(row, (uint32_t)v);
                 if (ch) {
@@ -1593,9 +1595,10 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
     const uint4 *meta = reinterpret_cast<const uint4 *>(ps);
     const uint32_t *row = ps + 4ull * cap, *rc = whole ? a.rcol : ps + 6ull * cap;
     uint32_t *const in0 = reinterpret_cast<uint32_t *>(a.W), *const in1 = in0 + n;
-    // batched, asynchronous: the last round each row was reached in (its graph's relaxation count)
+    // batched, asynchronous: the last even and the last odd round each row was reached in (its graph's relaxation count;
+    // the round before is read while this round's pushes come in)
     constexpr bool REACH = BATCH && !SYNC;
-    uint32_t *const reach = in1 + n;
+    uint32_t *const reach0 = in1 + n, *const reach1 = reach0 + n;
     const uint32_t *const comp = whole ? a.comp : row + cap; // batched: graph of each vertex
     const uint64_t t0 = whole ? global_ns() : *(volatile unsigned long long *)&c->t0;
     uint64_t mark = global_ns(), ph_rounds = 0, ph_check = 0;
@@ -1701,7 +1704,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
             uint32_t *const to = SYNC ? ((r & 1) ? in1 : in0) : val;
             const auto push = [&](uint32_t w, uint32_t o) {
                 atomicMax(to + w, o);
-                if (REACH) atomicMax(reach + w, r);
+                if (REACH) atomicMax(((r & 1) ? reach1 : reach0) + w, r);
             };
             const bool pushes = r <= a.max_inner; // (past the limit the last round's values are only taken)
             uint32_t hits = 0;
@@ -1716,7 +1719,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
                     for (int k = 0; k < OWN_U; ++k) {
                         const uint32_t i = i0 + k * TT + tid;
                         y[k] = i >= mine ? 0u : start ? own[i] : __ldcg(words + vid(i));
-                        if (REACH) f[k] = i >= mine || pass || r <= 2 ? 0u : __ldcg(reach + vid(i));
+                        if (REACH) f[k] = i >= mine || pass || r <= 2 ? 0u : __ldcg(((r & 1) ? reach0 : reach1) + vid(i));
                     }
 #pragma unroll
                     for (int k = 0; k < OWN_U; ++k) {
@@ -1924,7 +1927,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
                     own[i] = o = 0;
                 len = end[i] - beg[i];
                 if (!SYNC && x) val[vid(i)] = 0; // (the next iteration's pushes go to the other array)
-                if (REACH && x) reach[vid(i)] = 0;
+                if (REACH && x) reach0[vid(i)] = reach1[vid(i)] = 0;
                 last[i] = 0;
             }
             if (!pack) continue;
@@ -1998,7 +2001,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
             } else {
                 if (status != ST_OK) x = max(x, __ldcg(val + vid(i)));
                 if (x) val[vid(i)] = 0;
-                if (REACH && x) reach[vid(i)] = 0;
+                if (REACH && x) reach0[vid(i)] = reach1[vid(i)] = 0;
             }
             if (!BATCH && a.out) {
                 if (whole) a.out[vid(i)] = x - 1u; // (no value: MAP_NONE)

@@ -1,5 +1,6 @@
 """What one kernel of a whole run leaves to the next (k_run to k_own to k_tail), against the oracle: graphs of a batch that
-end in the iteration after which the rest is renumbered, counters that scan mode has used."""
+end in the iteration after which the rest is renumbered, counters that scan mode has used, rows that are
+reached in every round."""
 import time
 
 import numpy as np
@@ -129,5 +130,36 @@ def test_scan_mode_then_the_grid_kernel(pkg, n):
                 r = pkg.map_run(h, sched=sched, flags=pkg.MAP_FLAG_FRONTIER_START, map_out=out, **kw)
                 same(r, want, sched, out)
                 assert (r.edges_total, r.accepting_left) == (4 * g.m, 1)
+    finally:
+        pkg.map_destroy(h)
+
+
+@pytest.mark.parametrize("n", [60_000, OWN - 40, OWN + 100_000])
+def test_batched_rows_reached_in_every_round(pkg, n):
+    """One value runs down a chain of 200 vertices, and thousands of rows in one block's share hold the whole chain: they are
+    in every round's frontier, and each time their length belongs to the relaxation count of an asynchronous batch too, also
+    where the next round's pushes come in before their block has looked."""
+    length = 200
+    share = np.arange(n) // 32 % 152 == 0
+    wides = np.flatnonzero(share)[:10_000]
+    chain = np.random.default_rng(5).permutation(np.flatnonzero(~share))[:length]
+    deg = np.zeros(n, np.int64)
+    deg[wides], deg[chain[1:]] = length - 1, 1
+    rowptr = np.zeros(n + 1, np.uint32)
+    np.cumsum(deg, out=rowptr[1:])
+    col = np.zeros(int(rowptr[-1]), np.uint32)
+    col[(rowptr[wides][:, None] + np.arange(length - 1)).ravel()] = np.tile(chain[1:], wides.size)
+    col[rowptr[chain[1:]]] = chain[:-1]
+    acc = np.zeros(n, np.uint8)
+    acc[chain[0]] = 1
+    g = mapgen.Graph(n, rowptr, col, acc, (0,) * 8, "chain", {})
+    small = mapgen.tiny_graph(3, 20)
+    h = pkg.map_batch_create([(x.n, x.rowptr, x.colidx, pkg.pack_bits(x.acc)) for x in (g, small)])
+    try:
+        for sched in (1, 0, 1):
+            r = pkg.map_batch_run(h, 2, sched=sched, flags=pkg.MAP_FLAG_FRONTIER_START)[0]
+            assert (r.verdict, r.outer) == (0, 1)
+            # the whole chain but its head pushes to them, from round 2 to the last; a chain vertex once, from round 2 on
+            assert r.relaxations == g.m + (r.inner_iters - 1) * wides.size * (length - 1) + length - 2, sched
     finally:
         pkg.map_destroy(h)
