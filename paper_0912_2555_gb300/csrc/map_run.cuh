@@ -31,7 +31,10 @@
 // Floods.  When a list holds a large share of the whole graph's vertices (one value sweeping a giant
 // component), its random accesses cost more than reading everything in order: from there on the iteration
 // runs in scan mode (Run::scan_round), with 4-byte state arrays, pushes that nothing waits for and all vertices
-// read in order every round, in pieces that go round the blocks.
+// read in order every round, in pieces that go round the blocks.  Asynchronous, a vertex's value is read again when it
+// is pushed (acyclic graphs of 4 M vertices, degree 4 / 8 / 16, ms for six iterations, without 17.6 / 29.5 / 47.2, with 11.7 /
+// 18.7 / 28.0; dense start 16.7 / 18.4 / 22.1: from degree 10 or so such floods would be better off with that, but others of
+// the same size and degree are not -- random 1.3 against 2.5 ms, layered 1.9 against 7.4).
 //
 // What it measured, ms per run (dense start in a CUDA graph -> here, k_own and k_tail included): layered 2^26
 // asynchronous 16.7 -> 2.5, 2^24 synchronous 7.9 -> 1.7, 10^6 asynchronous 3.0 -> 0.81, a random graph of 16,384
@@ -565,7 +568,9 @@ template <bool SYNC, bool BATCH> struct Run {
                         const uint32_t u = sh.list[i];
                         b = __ldg(a.rrowptr + u);
                         len = __ldg(a.rrowptr + u + 1) - b;
-                        o = max(sh.touch[i], ((__ldcg(a.acc + (u >> 5)) >> (u & 31u)) & 1u) ? u + 1 : 0u);
+                        uint32_t x = sh.touch[i];
+                        if (!SYNC) scan_a()[u] = x = __ldcg(val + u); // (raised since, perhaps: not pushed twice)
+                        o = max(x, ((__ldcg(a.acc + (u >> 5)) >> (u & 31u)) & 1u) ? u + 1 : 0u);
                     },
                     [&](bool, uint64_t, uint32_t, uint32_t, uint32_t tot) {
                         if (!SYNC && !BATCH && threadIdx.x == 0) relax += tot;
@@ -1544,6 +1549,13 @@ constexpr int OWN_U = 4;                       // words read ahead per thread
 // layered 4 M 1260 / 1174 / 1150 / 1177 / 1185, 2^24 1557 / 1437 / 1387 / 1381 / 1374, 2^26 2641 / 2464 / 2440 / 2444 /
 // 2434, random 300,000 395 / 368 / 362 / 366 / 380, interleaved product 6x7 255 / 221 / 204 / 199 / 193
 constexpr uint32_t OWN_PASSES = 2;
+// asynchronous, more vertices than this to push from: the value is read again just before, since a flood has raised many
+// meanwhile, and the older value would be pushed along all of its readers for nothing.  us per run (six iterations of
+// the first four) without / with: acyclic graphs of 10^6 vertices and degree 4 3,440 / 2,000, degree 16 10,760 / 3,650
+// (dense start 4,900 and 7,580), 1.8 M and degree 8 10,280 / 3,680 (8,430), 500,000 and degree 64 12,500 / 4,600 (14,170);
+// interleaved product 7x7 880 / 505, random 10^6 of degree 16 463 / 300.  With few vertices the read is one more access
+// in a chain: layered 4 M 1,167 / 1,240 where every value is read again
+constexpr uint32_t OWN_LIVE = 256;
 constexpr uint32_t OWN_HUB = 2048;             // reader lists longer than this are walked by the whole block
 
 struct OwnSmem {
@@ -1763,6 +1775,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
                     uint32_t o = 0, b = 0, e = 0;
                     if (q < nq) {
                         const uint32_t i = queue[q];
+                        if (!SYNC && !start && nq > OWN_LIVE) last[i] = max(last[i], __ldcg(val + vid(i)));
                         o = start ? own[i] : max(last[i], own[i]);
                         b = beg[i];
                         e = end[i];
