@@ -1032,10 +1032,13 @@ static uint32_t tail_cap()
     const uint32_t room = (uint32_t)tail_blocks() * mapk::TAIL_N;
     return own_fits() ? std::min(room, mapk::TAIL_BEST) : room;
 }
-static bool runs_in_tail(const map_graph *g) { return !g->comp && g->n <= tail_cap(); }
+// blocks of k_own: one on each SM a run may fill
+static uint32_t own_blocks(const map_graph *g) { return !own_fits() ? 0u : (uint32_t)(g->sm_share ? g->sm_share : g->sms); }
+// entries up to which the cluster is preferred: a worker's share of the chip pushes no faster than the cluster does
+static uint32_t tail_entries(const map_graph *g) { return own_blocks(g) >= 2 * mapk::TAIL_C ? mapk::TAIL_BEST_M : 0xFFFFFFFFu; }
+static bool runs_in_tail(const map_graph *g) { return !g->comp && g->n <= tail_cap() && g->m <= tail_entries(g); }
 
 // graphs that fit into the shared memory of the SMs a run may fill (k_own)
-static uint32_t own_blocks(const map_graph *g) { return !own_fits() ? 0u : (uint32_t)(g->sm_share ? g->sm_share : g->sms); }
 static bool runs_in_own(const map_graph *g) { return !runs_in_tail(g) && g->n <= (uint64_t)own_blocks(g) * mapk::OWN_N; }
 
 // Which start a run takes when neither its flags nor map_autotune say: the frontier start pushes
@@ -1139,6 +1142,7 @@ static int launch_run(map_graph *g, cudaStream_t s, const map_opts &opts, const 
     a.tail_cap = g->comp ? 0u : tail_cap(); // (k_tail takes single graphs)
     const uint32_t own = own_blocks(g);
     a.own_cap = own * mapk::OWN_N;
+    a.tail_m = tail_entries(g);
     CK(cudaMemsetAsync(g->run_ctl, 0, sizeof(mapk::RunCtl), s));
     if (g->comp) {
         mapk::k_batch_begin<<<(g->ncomp + 255) / 256, 256, 0, s>>>(dev_of(g));

@@ -110,6 +110,7 @@ struct RunArgs {
     uint64_t timeout_ns;
     const uint32_t *prep;        // not NULL: (error, accepting vertices, entries) that k_prepare found
     uint32_t tail_cap, own_cap;  // compact graphs of at most this many vertices are left to k_tail / k_own (0: none)
+    uint32_t tail_m;             // ... and of at most this many entries to k_tail where k_own could go on
     // batched runs
     const uint32_t *comp;
     CompState *cs;
@@ -777,6 +778,7 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
     uint32_t outer = 0, status = ST_OK, verdict = 0, witness = NONE, nacc = a.nacc0, set = 1;
     unsigned long long inner_total = 0;
     bool go = a.nacc0 != 0, compactable = true, hand = false;
+    uint32_t entries = 0; // (lead) of the compact graph
     while (go && alive) {
         ++outer;
         if (lead && (SYNC || !a.count_round1)) run.relax += a.m; // round 1 covers every row
@@ -1010,7 +1012,10 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
                         if (live[j]) rc2[first + pair[j]] = __ldcg(a.rank + run.id_of(__ldcg(sp.rc + pos[j]))) - 1;
                 });
             if (!(alive = run_barrier(c, c->bar, sh, run.seq, over ? 1 : 0, total))) break;
-            if (lead) *(volatile uint32_t *)&c->xcnt.v = *(volatile uint32_t *)&c->ecnt.v = 0;
+            if (lead) {
+                entries = *(volatile uint32_t *)&c->ecnt.v;
+                *(volatile uint32_t *)&c->xcnt.v = *(volatile uint32_t *)&c->ecnt.v = 0;
+            }
             if (total & RUN_COUNT) { // too many readers for the pool: stay in the whole graph
                 compactable = false;
             } else {
@@ -1054,7 +1059,7 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
             c->ph_check = ph_check;
             c->t0 = t0;
             c->ocnt[0].v = c->ocnt[1].v = 0; // (scan mode has counted there; k_own starts from zero)
-            c->hand = sp.V <= a.tail_cap ? 2u : 1u;
+            c->hand = sp.V <= a.tail_cap && (entries <= a.tail_m || sp.V > a.own_cap) ? 2u : 1u;
         }
         return;
     }
@@ -1192,6 +1197,12 @@ constexpr size_t TAIL_SMEM = (size_t)TAIL_N * 26;
 // graphs up to here run in the cluster, larger ones over the grid (k_own).  Layered graphs, synchronous, us per
 // run with k_tail / k_own: 16,000 vertices 166 / 205, 30,000 262 / 235, 60,000 317 / 238, 130,000 470 / 263
 constexpr uint32_t TAIL_BEST = 16384;
+// ... and of at most this many entries: sixteen SMs take some 15 G pushes/s, the chip 133 G.  us per run with k_tail / k_own:
+// acyclic graphs (20 iterations, synchronous), 16,384 vertices with 147,456 entries 10,104 / 3,501, with 1 M 56,453 / 8,910,
+// with 4 M 221,713 / 27,697 (dense start 0.18 s); random ones of 16,384 with 262,144 178 / 106, with 4 M 1,168 / 196 (1,340), 4,000
+// with 1 M 786 / 135.  Where few vertices change a round is a chain of latencies and k_tail stays ahead: layered 16,000
+// with 250,531 entries 373 / 422, asynchronous 301 / 354
+constexpr uint32_t TAIL_BEST_M = 262144;
 // asynchronous, a vertex per thread: looks at the vertex per round, so that values that came in meanwhile go on
 // before the barrier (10^6 layered, us per run with 1 / 2 / 4 / 6 / 8 looks: 900 / 844 / 777 / 764 / 751; 4,000 random
 // 80 / - / 71 / 77 / 77; 16,000 layered 163 / - / 148 / 154 / 164)
@@ -1924,7 +1935,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
         const bool pack = !BATCH && T <= gate;
         uint32_t V2 = 0, E2 = 0;
         const uint32_t lim = min(a.tail_cap, cap);
-        const uint64_t ecap = (uint64_t)n * 3 / 4 - 8;
+        const uint64_t ecap = min((uint64_t)n * 3 / 4 - 8, (uint64_t)a.tail_m);
         uint32_t *const ps2 = pool_set(a, set ^ 1);
         uint4 *const meta2 = reinterpret_cast<uint4 *>(ps2);
         uint32_t *const row2 = ps2 + 4ull * cap, *const rc2 = ps2 + 6ull * cap;

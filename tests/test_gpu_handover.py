@@ -1,6 +1,6 @@
 """What one kernel of a whole run leaves to the next (k_run to k_own to k_tail), against the oracle: graphs of a batch that
 end in the iteration after which the rest is renumbered, counters that scan mode has used, rows that are
-reached in every round."""
+reached in every round, graphs of few vertices and many entries."""
 import time
 
 import numpy as np
@@ -161,5 +161,54 @@ def test_batched_rows_reached_in_every_round(pkg, n):
             assert (r.verdict, r.outer) == (0, 1)
             # the whole chain but its head pushes to them, from round 2 to the last; a chain vertex once, from round 2 on
             assert r.relaxations == g.m + (r.inner_iters - 1) * wides.size * (length - 1) + length - 2, sched
+    finally:
+        pkg.map_destroy(h)
+
+
+TAIL_N, TAIL_M = 16384, 262144  # the largest graph that runs in one cluster
+
+
+def clumps(n, m, seed):
+    """m entries, each row's among its next vertices: reader lists as long as rows, no cycle but through the last rows."""
+    rng = np.random.default_rng(seed)
+    row = np.sort(rng.integers(0, n, m))
+    rowptr = np.searchsorted(row, np.arange(n + 1)).astype(np.uint32)
+    col = np.minimum(row + 1 + (rng.random(m) * max(1, n // 20)).astype(np.int64), n - 1).astype(np.uint32)
+    acc = (rng.random(n) < 0.02).astype(np.uint8)
+    acc[n - 1] = 0
+    return mapgen.Graph(n, rowptr, col, acc, (0,) * 8, "clumps", {})
+
+
+@pytest.mark.parametrize("n,m,launches", [(TAIL_N, TAIL_M, 1), (TAIL_N, TAIL_M + 1, 2), (700, TAIL_M, 1), (700, TAIL_M + 1, 2),
+                                          (5000, 1_000_000, 2)])
+def test_graphs_of_many_entries_use_the_whole_chip(pkg, n, m, launches):
+    """Sixteen SMs fall behind the whole chip where every vertex has many readers, however few the vertices."""
+    g = clumps(n, m, n)
+    want = oracle.run_graph(g, max_outer=12)
+    h = pkg.map_create(g.n, g.rowptr, g.colidx, pkg.pack_bits(g.acc))
+    try:
+        for sched in (0, 1):
+            out = np.empty(n, np.uint32)
+            r = pkg.map_run(h, sched=sched, map_out=out, max_outer=12, allow_limit=True)
+            same(r, want, sched, out)
+            assert r.launches == launches
+    finally:
+        pkg.map_destroy(h)
+
+
+@pytest.mark.parametrize("pad", [100_000, OWN])
+def test_renumbered_graph_of_many_entries(pkg, pad):
+    """A graph of few vertices and many entries inside a large one: what is left after an iteration is small enough for the
+    cluster by its vertices and too large by its entries, later by neither."""
+    core = clumps(6000, 400_000, 3)
+    g = padded(core, core.n + pad)
+    want = oracle.run_graph(g)
+    assert want.outer > 20
+    h = pkg.map_create(g.n, g.rowptr, g.colidx, pkg.pack_bits(g.acc))
+    try:
+        for sched in (0, 1):
+            out = np.empty(g.n, np.uint32)
+            r = pkg.map_run(h, sched=sched, flags=pkg.MAP_FLAG_FRONTIER_START, map_out=out)
+            same(r, want, sched, out)
     finally:
         pkg.map_destroy(h)
