@@ -1096,7 +1096,27 @@ static int await_result(const map_graph *g, cudaStream_t s, mapk::RunRes *pageab
     return MAP_OK;
 }
 
-// Queue one whole run as a single launch (k_run) and fill in the result from where the kernel left it.
+static int launch_own(const mapk::RunArgs &a, bool sync_sched, bool batch, bool whole, uint32_t blocks, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(mapk::TT);
+    cfg.dynamicSmemBytes = mapk::OWN_SMEM;
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const uint32_t w = whole ? 1u : 0u;
+    if (batch && sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_own<true, true>, a, w));
+    else if (batch) CK(cudaLaunchKernelEx(&cfg, mapk::k_own<false, true>, a, w));
+    else if (sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_own<true, false>, a, w));
+    else CK(cudaLaunchKernelEx(&cfg, mapk::k_own<false, false>, a, w));
+    return MAP_OK;
+}
+
+// Queue one whole run (k_run, k_own, k_tail: whichever may have a part in it); the last of them leaves the result.
 static int launch_run(map_graph *g, cudaStream_t s, const map_opts &opts, const Ctl &init, bool count_round1,
                       uint32_t *out)
 {
@@ -1148,15 +1168,15 @@ static int launch_run(map_graph *g, cudaStream_t s, const map_opts &opts, const 
         mapk::k_batch_begin<<<(g->ncomp + 255) / 256, 256, 0, s>>>(dev_of(g));
         CK(cudaGetLastError());
     }
-    cudaLaunchConfig_t cfg = {};
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
     const bool in_own = runs_in_own(g);
     if (!in_own) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.stream = s;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
         const int sms = g->sm_share ? g->sm_share : g->sms;
         cfg.gridDim = dim3((unsigned)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)sms * occ, (n + mapk::RT - 1) / mapk::RT)));
         cfg.blockDim = dim3(mapk::RT);
@@ -1165,16 +1185,8 @@ static int launch_run(map_graph *g, cudaStream_t s, const map_opts &opts, const 
         else if (sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_run<true, false>, a));
         else CK(cudaLaunchKernelEx(&cfg, mapk::k_run<false, false>, a));
     }
-    if (own) {
-        cfg.gridDim = dim3(own);
-        cfg.blockDim = dim3(mapk::TT);
-        cfg.dynamicSmemBytes = mapk::OWN_SMEM;
-        const uint32_t w = in_own ? 1u : 0u;
-        if (g->comp && sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_own<true, true>, a, w));
-        else if (g->comp) CK(cudaLaunchKernelEx(&cfg, mapk::k_own<false, true>, a, w));
-        else if (sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_own<true, false>, a, w));
-        else CK(cudaLaunchKernelEx(&cfg, mapk::k_own<false, false>, a, w));
-    }
+    int rc = MAP_OK;
+    if (own && (rc = launch_own(a, sync_sched, g->comp != nullptr, in_own, own, s))) return rc;
     return cluster ? launch_tail(a, sync_sched, false, (uint32_t)cluster, s) : MAP_OK;
 }
 
@@ -2062,9 +2074,10 @@ int map_batch_run(map_graph *g, const map_opts *opts, map_result *results, uint3
 // all of its work space in the file-scope device array below, which every GPU
 // that loads this library holds until the process exits, and it calls no
 // cudaMalloc, cudaFree or allocating routine.  It runs the same kernels as
-// map_run: set-up and run are one launch each in one thread-block cluster, and the
-// call waits for its stream once (an early exit or the dense start: stepped from the
-// host, with several waits).  So it blocks, and it cannot be issued on a stream that
+// map_run: set-up is one launch in one thread-block cluster, the run another one there
+// (above TAIL_BEST vertices: over the grid, and what is left of the graph in the
+// cluster), and the call waits for its stream once (an early exit or the dense start:
+// stepped from the host, with several waits).  So it blocks, and it cannot be issued on a stream that
 // is being captured.
 // ============================================================================
 
@@ -2149,6 +2162,8 @@ int static_read_ctl(Ctl *h, const Ctl *d, cudaStream_t s)
 
 } // namespace
 
+static_assert(sizeof(mapk::RunCtl) <= ST_MAX_N * 4, "a run's control block lies in the space of the touched list");
+
 // what run_static_impl reports for a CSR that map_run_static does not take (k_prepare's codes)
 static int static_refused(uint32_t code, uint32_t r0, uint64_t m)
 {
@@ -2210,14 +2225,33 @@ static int run_static_cluster(uint32_t n, const uint32_t *rowptr, const uint32_t
     a.max_inner = opts.max_inner ? opts.max_inner : n + 1;
     a.timeout_ns = (uint64_t)(opts.timeout_ms ? opts.timeout_ms : 120000u) * 1000000ull;
     a.prep = dev->prep;
+    // larger ones over the grid, and what is left of them in the cluster; every word of state starts at zero.  us per call
+    // stepped from the host / in the cluster / over the grid: acyclic graphs (six iterations, synchronous) of 65,536 vertices
+    // with 457,023 entries 4,692 / 8,148 / 1,354, with 261,787 4,179 / 5,322 / 1,226, layered 65,536 808 / 280 / 242, 32,000 765 / 216 / 215
+    int dev_id = 0, sms = 0;
+    CK(cudaGetDevice(&dev_id));
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev_id));
+    const bool own = n > tail_cap() && (uint64_t)sms * mapk::OWN_N >= n; // (tail_cap: all of it where k_own does not fit)
+    if (own) {
+        a.acc = base + ST_ACC;
+        a.W = reinterpret_cast<unsigned long long *>(base + ST_REC);
+        a.rank = base + ST_MVAL;
+        a.pool = base + ST_FLIST;
+        a.ctl = reinterpret_cast<mapk::RunCtl *>(base + ST_TOUCHED);
+        a.tail_cap = tail_cap();
+        a.own_cap = (uint32_t)sms * mapk::OWN_N;
+        a.tail_m = mapk::TAIL_BEST_M;
+        CK(cudaMemsetAsync(a.W, 0, (size_t)n * 16, s));
+        CK(cudaMemsetAsync(a.ctl, 0, sizeof(mapk::RunCtl), s));
+    }
     const int cluster = tail_blocks();
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr;
     cluster_config(cfg, attr, tail_blocks_for(n, cluster), 0, s);
     CK(cudaLaunchKernelEx(&cfg, mapk::k_prepare<false>, n, rowptr, colidx, acc_bits, (uint32_t)ST_MAX_M, base + ST_ACC0,
                           base + ST_RROWPTR, base + ST_RCOL, base + ST_RPOS, dev->prep, mapk::PrepareOut{}));
-    int rc = launch_tail(a, sync_sched, true, tail_blocks_for(n, cluster), s);
-    if (rc) return rc;
+    int rc = own ? launch_own(a, sync_sched, false, true, (uint32_t)sms, s) : MAP_OK;
+    if (rc || (rc = launch_tail(a, sync_sched, !own, own ? (uint32_t)cluster : tail_blocks_for(n, cluster), s))) return rc;
     Back h;
     CK(cudaMemcpyAsync(&h, dev, sizeof h, cudaMemcpyDeviceToHost, s));
     if (map_out && !out_dev) { // (into the caller's buffer only once the graph is known to be good)
@@ -2227,7 +2261,7 @@ static int run_static_cluster(uint32_t n, const uint32_t *rowptr, const uint32_t
     CK(cudaStreamSynchronize(s));
     if (h.prep[0]) return static_refused(h.prep[0], h.prep[3], h.prep[2]);
     if ((rc = take_result(h.res, opts, h.prep[2], sync_sched, base + ST_HISTW, (uint32_t)ST_HIST, s, res))) return rc;
-    res->launches = 2;
+    res->launches = own ? 3 : 2;
     if (h.res.status == mapk::ST_LIMIT) return fail(MAP_ERR_LIMIT, "map_run_static: max_outer or max_inner reached");
     if (h.res.status == mapk::ST_TIMEOUT) return fail(MAP_ERR_TIMEOUT, "map_run_static: stopped after the timeout");
     return MAP_OK;

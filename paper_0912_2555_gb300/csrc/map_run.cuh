@@ -1598,6 +1598,9 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
     __shared__ OwnSmem sh;
     RunCtl *c = a.ctl;
     if (!whole && *(volatile uint32_t *)&c->hand != 1) return; // finished, or left to k_tail (every block returns)
+    if (a.prep && a.prep[0]) return;                           // k_prepare refused the graph
+    const uint32_t nacc0 = a.prep ? a.prep[1] : a.nacc0;
+    const uint64_t m = a.prep ? a.prep[2] : a.m;
     const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     const bool lead = blockIdx.x == 0 && tid == 0;
     const uint32_t n = a.n, V = whole ? n : *(volatile uint32_t *)&c->V;
@@ -1696,7 +1699,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
     if (tid == 0) sh.late = 0;
     __syncthreads();
 
-    uint32_t outer = whole ? 0u : *(volatile uint32_t *)&c->outer, nacc = whole ? a.nacc0 : *(volatile uint32_t *)&c->nacc;
+    uint32_t outer = whole ? 0u : *(volatile uint32_t *)&c->outer, nacc = whole ? nacc0 : *(volatile uint32_t *)&c->nacc;
     uint32_t status = ST_OK, verdict = 0, witness = NONE, seq = 0, gate = a.tail_cap / 2;
     unsigned long long relax = 0, frows = 0, inner_total = 0, total = 0;
     bool go = nacc != 0, alive = true, hand = false;
@@ -1719,7 +1722,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
     while (go) {
         ++outer;
         uint32_t *const val = (outer & 1) ? in1 : in0; // (asynchronous)
-        if (lead && (SYNC || !a.count_round1)) relax += a.m; // round 1 covers every row
+        if (lead && (SYNC || !a.count_round1)) relax += m; // round 1 covers every row
         uint32_t r = 0;
         for (;;) {
             ++r;
@@ -1922,7 +1925,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
         } else {
             nacc -= (uint32_t)(total & RUN_COUNT);
             if (nacc == 0) go = false;
-            else if ((a.max_outer && outer >= a.max_outer) || outer > a.nacc0) {
+            else if ((a.max_outer && outer >= a.max_outer) || outer > nacc0) {
                 status = ST_LIMIT;
                 go = false;
             } else if (total & RUN_STOP) {

@@ -212,3 +212,25 @@ def test_renumbered_graph_of_many_entries(pkg, pad):
             same(r, want, sched, out)
     finally:
         pkg.map_destroy(h)
+
+
+@pytest.mark.parametrize("n,m,launches", [(TAIL_N, 300_000, 2), (TAIL_N + 1, 60_000, 3), (40_001, 500_000, 3), (65_536, 524_288, 3)])
+@pytest.mark.parametrize("on_device", [False, True])
+def test_static_runs_over_the_grid(pkg, n, m, launches, on_device):
+    """map_run_static: set-up in one cluster, runs of more than 16,384 vertices over the grid, what is left of them in the
+    cluster; an invalid graph is still refused, and the call after that one sees nothing of either."""
+    gs = [clumps(n, m, n), mapgen.layered_graph(n, max(8, n // 4000), seed=n)]
+    for g in gs * 2:
+        want = oracle.run_graph(g, max_outer=12)
+        args = [g.rowptr, g.colidx, pkg.pack_bits(g.acc)]
+        if on_device:
+            args = [torch.from_numpy(x.view(np.int32)).cuda() for x in args]
+        for sched in (0, 1):
+            out = np.full(n, 7, np.uint32)
+            r = pkg.map_run_static(n, *args, sched=sched, map_out=out, max_outer=12, allow_limit=True)
+            same(r, want, sched, out)
+            assert r.launches == launches
+            bad = [args[0], args[1].copy() if not on_device else args[1].clone(), args[2]]
+            bad[1][g.m // 2] = n
+            with pytest.raises(pkg.MapError, match="CSR"):
+                pkg.map_run_static(n, *bad, sched=sched, map_out=out)
