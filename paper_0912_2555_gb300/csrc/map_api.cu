@@ -365,8 +365,8 @@ struct map_graph {
     Ctl *ctl = nullptr;
     Ctl *h_ctl = nullptr;        // mirror of ctl: a page-locked slot (ctl_slots) or pageable memory
     bool h_ctl_pinned = false;
-    uint32_t *h_stage = nullptr; // pinned n words for traces / host output
-    uint32_t *h_hist = nullptr;  // pinned mirror of hist
+    uint32_t *h_stage = nullptr; // n words for traces (host memory, on the first traced run)
+    uint32_t *h_hist = nullptr;  // copy of hist (host memory, on the first run that wants it)
     uint32_t nacc0 = 0;
     cudaEvent_t ev[8] = {};
     // batched graphs (disjoint union of several graphs; see map_batch_create)
@@ -374,7 +374,7 @@ struct map_graph {
     uint32_t *comp = nullptr;        // graph of each union vertex
     mapk::CompState *cs = nullptr;   // one record per graph
     uint32_t *chist = nullptr;       // rounds per outer iteration, CH_CAP per graph
-    mapk::CompState *h_cs = nullptr; // pinned mirrors
+    mapk::CompState *h_cs = nullptr; // mirrors in host memory
     uint32_t *h_chist = nullptr;
     // frontier start: the initially accepting vertices (built on first use), and whether the
     // launches being issued use it
@@ -2530,11 +2530,12 @@ constexpr uint64_t kMaxBatchVertices = 1ull << 26;
 // of before, 2^20 1,886 / 2,261 / 2,233); 38 synchronous jobs at once, ms: 76 / 59 / 67.
 constexpr uint32_t kMaxBatchedJobN = 1u << 16;
 
-// device bytes of a graph: the allocations of create_graph
+// device bytes of a graph: the allocation of create_graph, and the set-up's rank array beside it (where m <= 6n it lies in
+// the list space; it is counted all the same, since jobs that share a run may need it for their union)
 size_t graph_footprint(uint64_t n, uint64_t m)
 {
     const uint64_t W = (n + 31) / 32;
-    // (colidx, rcol, rpos, and the set-up's rank array: 4 words per entry at the peak)
+    // (colidx, rcol, rpos, rank: 4 words per entry at the peak)
     const uint64_t words = 2 * (n + 5) + 4 * (m + 4) + 3 * (W + 4) + (n + 4) + 2 * 3 * (n + 4) + 4 * (n + 4) +
                            3 * (n + 4) + (1u << 16);
     // the changed-vertex bitmaps of pull rounds

@@ -1571,7 +1571,7 @@ constexpr uint32_t OWN_HUB = 2048;             // reader lists longer than this 
 
 struct OwnSmem {
     unsigned long long word;
-    uint32_t ok, n, hubs, late, ebase, xbase;
+    uint32_t ok, n, hubs, ebase, xbase;
     uint32_t scan[TT / 32], scan2[TT / 32], mins[TT / 32], sums[TT / 32];
     uint32_t hub[32];
     unsigned long long part[TT / 32];
@@ -1696,7 +1696,6 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
         if (BATCH && a.out) // (graphs end in different iterations)
             for (uint64_t i = gid; i < n; i += threads) a.out[i] = NONE;
     }
-    if (tid == 0) sh.late = 0;
     __syncthreads();
 
     uint32_t outer = whole ? 0u : *(volatile uint32_t *)&c->outer, nacc = whole ? nacc0 : *(volatile uint32_t *)&c->nacc;
@@ -1765,11 +1764,10 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
                             }
                             hit = hit && y[k] > last[i];
                             if (hit) last[i] = y[k];
-                            if constexpr (BATCH) { // the graphs that changed in round r - 1 (a later pass: in this one)
+                            if constexpr (BATCH) { // the graphs that changed in round r - 1
                                 const unsigned same = __match_any_sync(0xFFFFFFFFu, hit ? g : NONE);
-                                const uint32_t at = pass ? r : r - 1;
-                                if (hit && lane == (unsigned)(__ffs(same) - 1) && *(volatile uint32_t *)&a.cs[g].last_change < at)
-                                    atomicMax(&a.cs[g].last_change, at);
+                                if (hit && lane == (unsigned)(__ffs(same) - 1) && *(volatile uint32_t *)&a.cs[g].last_change < r - 1)
+                                    atomicMax(&a.cs[g].last_change, r - 1);
                             }
                         }
                         const unsigned m = __ballot_sync(0xFFFFFFFFu, hit);
@@ -1936,7 +1934,6 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
         if (!go) break;
         // ---- the next iteration: eliminated vertices offer nothing, values back to none
         const bool pack = !BATCH && T <= gate;
-        uint32_t V2 = 0, E2 = 0;
         const uint32_t lim = min(a.tail_cap, cap);
         const uint64_t ecap = min((uint64_t)n * 3 / 4 - 8, (uint64_t)a.tail_m);
         uint32_t *const ps2 = pool_set(a, set ^ 1);
@@ -1981,8 +1978,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
         if (!pack) continue;
         alive = run_barrier(c, c->obar, sh, seq, over ? 1u : 0u, total);
         if (!alive) break;
-        V2 = *(volatile uint32_t *)&c->xcnt.v;
-        E2 = *(volatile uint32_t *)&c->ecnt.v;
+        const uint32_t V2 = *(volatile uint32_t *)&c->xcnt.v;
         const bool fits = (total & RUN_COUNT) == 0;
         for (uint32_t i0 = 0; i0 < mine; i0 += TT) {
             const uint32_t i = i0 + tid, k = i < mine ? last[i] : 0u;
@@ -2016,7 +2012,6 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
         alive = run_barrier(c, c->obar, sh, seq, 0, total); // (every block has read the counts)
         if (!alive) break;
         if (lead) *(volatile uint32_t *)&c->xcnt.v = *(volatile uint32_t *)&c->ecnt.v = 0;
-        (void)E2;
     }
     // ---- the map of the last iteration; the state back to zero
     if (alive && !hand) {
