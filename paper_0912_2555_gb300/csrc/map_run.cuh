@@ -86,7 +86,7 @@ struct RunCtl {
     Line64 obar[3];   // k_own's grid barriers
     Cnt32 ocnt[2];    // k_own: vertices with a value, by outer iteration mod 2
     // what k_run leaves to k_own (hand = 1), and either to k_tail (2): the compact graph and where the run stands
-    uint32_t hand, V, set, outer, nacc;
+    uint32_t hand, next, V, set, outer, nacc;
     unsigned long long inner_total, ph_rounds, ph_check, t0;
 };
 
@@ -778,7 +778,6 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
     uint32_t outer = 0, status = ST_OK, verdict = 0, witness = NONE, nacc = a.nacc0, set = 1;
     unsigned long long inner_total = 0;
     bool go = a.nacc0 != 0, compactable = true, hand = false;
-    uint32_t entries = 0; // (lead) of the compact graph
     while (go && alive) {
         ++outer;
         if (lead && (SYNC || !a.count_round1)) run.relax += a.m; // round 1 covers every row
@@ -1013,7 +1012,8 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
                 });
             if (!(alive = run_barrier(c, c->bar, sh, run.seq, over ? 1 : 0, total))) break;
             if (lead) {
-                entries = *(volatile uint32_t *)&c->ecnt.v;
+                // (who goes on, if the compact graph is left to a kernel below)
+                c->next = V2 <= a.tail_cap && (*(volatile uint32_t *)&c->ecnt.v <= a.tail_m || V2 > a.own_cap) ? 2u : 1u;
                 *(volatile uint32_t *)&c->xcnt.v = *(volatile uint32_t *)&c->ecnt.v = 0;
             }
             if (total & RUN_COUNT) { // too many readers for the pool: stay in the whole graph
@@ -1059,7 +1059,7 @@ __global__ void __launch_bounds__(RT, MAPGPU_RUN_BLOCKS) k_run(const __grid_cons
             c->ph_check = ph_check;
             c->t0 = t0;
             c->ocnt[0].v = c->ocnt[1].v = 0; // (scan mode has counted there; k_own starts from zero)
-            c->hand = sp.V <= a.tail_cap && (entries <= a.tail_m || sp.V > a.own_cap) ? 2u : 1u;
+            c->hand = c->next;
         }
         return;
     }
@@ -1565,8 +1565,9 @@ constexpr uint32_t OWN_PASSES = 2;
 // the first four) without / with: acyclic graphs of 10^6 vertices and degree 4 3,440 / 2,000, degree 16 10,760 / 3,650
 // (dense start 4,900 and 7,580), 1.8 M and degree 8 10,280 / 3,680 (8,430), 500,000 and degree 64 12,500 / 4,600 (14,170);
 // interleaved product 7x7 880 / 505, random 10^6 of degree 16 463 / 300.  With few vertices the read is one more access
-// in a chain: layered 4 M 1,167 / 1,240 where every value is read again
-constexpr uint32_t OWN_LIVE = 256;
+// in a chain: layered 4 M 1,167 / 1,240 where every value is read again; limit 256 / 512 / 1,024: layered 2^24 1,422 / 1,404 /
+// 1,405, acyclic 100,000 of degree 16 1,258 / 1,355 / 1,390, 300,000 of degree 4 1,128 / 1,135 / 1,144
+constexpr uint32_t OWN_LIVE = 512;
 constexpr uint32_t OWN_HUB = 2048;             // reader lists longer than this are walked by the whole block
 
 struct OwnSmem {
@@ -1599,8 +1600,9 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
     RunCtl *c = a.ctl;
     if (!whole && *(volatile uint32_t *)&c->hand != 1) return; // finished, or left to k_tail (every block returns)
     if (a.prep && a.prep[0]) return;                           // k_prepare refused the graph
-    const uint32_t nacc0 = a.prep ? a.prep[1] : a.nacc0;
-    const uint64_t m = a.prep ? a.prep[2] : a.m;
+    // (read where they are wanted: kept in registers over the rounds, they cost layered 2^26 2 %)
+    const auto nacc0 = [&] { return a.prep ? __ldg(a.prep + 1) : a.nacc0; };
+    const auto entries_all = [&] { return a.prep ? (uint64_t)__ldg(a.prep + 2) : a.m; };
     const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     const bool lead = blockIdx.x == 0 && tid == 0;
     const uint32_t n = a.n, V = whole ? n : *(volatile uint32_t *)&c->V;
@@ -1698,7 +1700,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
     }
     __syncthreads();
 
-    uint32_t outer = whole ? 0u : *(volatile uint32_t *)&c->outer, nacc = whole ? nacc0 : *(volatile uint32_t *)&c->nacc;
+    uint32_t outer = whole ? 0u : *(volatile uint32_t *)&c->outer, nacc = whole ? nacc0() : *(volatile uint32_t *)&c->nacc;
     uint32_t status = ST_OK, verdict = 0, witness = NONE, seq = 0, gate = a.tail_cap / 2;
     unsigned long long relax = 0, frows = 0, inner_total = 0, total = 0;
     bool go = nacc != 0, alive = true, hand = false;
@@ -1721,7 +1723,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
     while (go) {
         ++outer;
         uint32_t *const val = (outer & 1) ? in1 : in0; // (asynchronous)
-        if (lead && (SYNC || !a.count_round1)) relax += m; // round 1 covers every row
+        if (lead && (SYNC || !a.count_round1)) relax += entries_all(); // round 1 covers every row
         uint32_t r = 0;
         for (;;) {
             ++r;
@@ -1923,7 +1925,7 @@ __global__ void __launch_bounds__(TT, 1) k_own(const __grid_constant__ RunArgs a
         } else {
             nacc -= (uint32_t)(total & RUN_COUNT);
             if (nacc == 0) go = false;
-            else if ((a.max_outer && outer >= a.max_outer) || outer > nacc0) {
+            else if ((a.max_outer && outer >= a.max_outer) || outer > nacc0()) {
                 status = ST_LIMIT;
                 go = false;
             } else if (total & RUN_STOP) {
