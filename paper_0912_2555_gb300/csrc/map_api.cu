@@ -288,8 +288,9 @@ bool own_fits()
     }
     if (const int k = known[dev].load()) return k == 2;
     bool ok = true;
-    for (const void *f : {(const void *)mapk::k_own<true, false>, (const void *)mapk::k_own<false, false>,
-                          (const void *)mapk::k_own<true, true>, (const void *)mapk::k_own<false, true>}) {
+    for (const void *f : {(const void *)mapk::k_own<true, false, false>, (const void *)mapk::k_own<false, false, false>,
+                          (const void *)mapk::k_own<true, true, false>, (const void *)mapk::k_own<false, true, false>,
+                          (const void *)mapk::k_own<true, false, true>, (const void *)mapk::k_own<false, false, true>}) {
         int o = 0;
         ok = ok && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mapk::OWN_SMEM) == cudaSuccess &&
              cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, f, mapk::TT, mapk::OWN_SMEM) == cudaSuccess && o >= 1;
@@ -1109,10 +1110,12 @@ static int launch_own(const mapk::RunArgs &a, bool sync_sched, bool batch, bool 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const uint32_t w = whole ? 1u : 0u;
-    if (batch && sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_own<true, true>, a, w));
-    else if (batch) CK(cudaLaunchKernelEx(&cfg, mapk::k_own<false, true>, a, w));
-    else if (sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_own<true, false>, a, w));
-    else CK(cudaLaunchKernelEx(&cfg, mapk::k_own<false, false>, a, w));
+    if (batch && sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_own<true, true, false>, a, w));
+    else if (batch) CK(cudaLaunchKernelEx(&cfg, mapk::k_own<false, true, false>, a, w));
+    else if (a.prep && sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_own<true, false, true>, a, w));
+    else if (a.prep) CK(cudaLaunchKernelEx(&cfg, mapk::k_own<false, false, true>, a, w));
+    else if (sync_sched) CK(cudaLaunchKernelEx(&cfg, mapk::k_own<true, false, false>, a, w));
+    else CK(cudaLaunchKernelEx(&cfg, mapk::k_own<false, false, false>, a, w));
     return MAP_OK;
 }
 
