@@ -453,10 +453,10 @@ MAP_API int map_graph_info(const map_graph *g, uint32_t *n, uint64_t *m);
  *   cuda_stream: the stream all work is issued on.
  * The call blocks: it waits for cuda_stream once, for the result (with
  * MAP_FLAG_EARLY_EXIT or MAP_FLAG_DENSE_START after every step of the loop), so
- * it must not be issued on a stream that is being captured into a CUDA graph.  The first call on a device also looks the array's device
- * address up (cudaGetSymbolAddress) with that device current; make that first
- * call before any stream capture begins in the process.  Every call on a
- * device shares the one array and overwrites what the previous call left
+ * it must not be issued on a stream that is being captured into a CUDA graph.
+ * The first call on a device also looks the array's device address up
+ * (cudaGetSymbolAddress) with that device current; make that first call before
+ * any stream capture begins in the process.  Every call on a device shares the one array and overwrites what the previous call left
  * there, so calls that overlap on the GPU (from several host threads, or on
  * several streams) race and must be serialised by the caller.
  */
